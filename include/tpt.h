@@ -82,13 +82,13 @@ enum { TPT_XFORM_AUTO = 0, TPT_XFORM_GEMM = 1, TPT_XFORM_FFT = 2 };
  * cores (BF16, split BF16 with three products, or TF32; FP32 accumulation),
  * FP32 Thomas except the singular null line (float64), and a float64
  * residual driving iterative refinement to `rtol`.  FP64_OZAKI: the float64
- * solve with its eigenbasis-transform GEMMs on the bf16 tensor cores by the
- * Ozaki scheme (each operand row split into seven bf16 slices of six bits,
- * slice products summed exactly in float32 level by level and the levels in
- * float64; ~1e-13 of sum |a||b| per product) -- float64-accurate after the
- * plan's float64 refinement steps, everything else as FP64; GEMM directions
- * of at most 576 points (else UNSUPPORTED).  Reported as TPT_PREC_FP64 by the
- * plan's inspection calls.                                                   */
+ * solve with every eigenbasis-transform GEMM on the bf16 tensor cores by
+ * exact integer arithmetic in a residue number system (Ozaki scheme II: each
+ * operand row rounded to 53 bits or more of its maximum, the products exact),
+ * also in the single-step tpt_transform; GEMM directions of at most 576 points
+ * (else UNSUPPORTED).  A FP64 plan runs the same transforms in its solves for
+ * directions of 24 to 2048 points and the float64 FMA GEMM otherwise and in
+ * tpt_transform.  Reported as TPT_PREC_FP64 by the plan's inspection calls. */
 enum { TPT_PREC_FP64 = 0, TPT_PREC_MIXED_BF16 = 1, TPT_PREC_MIXED_BF16X3 = 2,
        TPT_PREC_MIXED_TF32 = 3, TPT_PREC_FP64_OZAKI = 4 };
 
@@ -175,10 +175,11 @@ int tpt_set_coefficients(tpt_plan plan, double alpha, double beta);
 int tpt_plan_destroy(tpt_plan plan);
 const char* tpt_status_string(int status);
 
-/* ---- single steps of the solve (the same kernels tpt_solve launches) ---- */
+/* ---- single steps of the solve ---- */
 /* Forward or inverse transform along x (dir = 0) or y (dir = 1) in float64:
  * forward applies Q^{-1} (Eq. forward-xy), inverse applies Q (Eq. inverse-xy),
- * with whichever transform the plan chose for that direction.  in_dev and
+ * with whichever transform the plan chose for that direction (a FP64 plan's
+ * GEMM directions: the float64 FMA GEMM, which needs no scratch).  in_dev and
  * out_dev hold Nx*Ny*Nz doubles and must not overlap.                      */
 int tpt_transform(tpt_plan plan, int dir, int inverse, const double* in_dev, double* out_dev,
                   void* stream);

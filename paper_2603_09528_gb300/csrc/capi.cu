@@ -64,7 +64,7 @@ void free_plan(tpt_plan_s* p) {
     if (p->h_ring) cudaFreeHost(p->h_ring);
     if (p->solve_exec) cudaGraphExecDestroy(p->solve_exec);
     if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
-    if (p->oz_scratch) cudaFree(p->oz_scratch);
+    if (p->res_scratch) cudaFree(p->res_scratch);
     tpt::pinned_slot_release(p->h_scal);
     cudaGetLastError();
   }
@@ -73,15 +73,23 @@ void free_plan(tpt_plan_s* p) {
 
 bool on_device(const tpt_plan_s* p) { return p && p->dev >= 0 && p->d_scal; }
 
+// Whether direction d of a float64 plan takes the tensor-core transform.  Per
+// transform (GB300, x; float64 FMA GEMM / residues): 16^3 21 / 30 us, 24^3 38 /
+// 31, 64^3 71 / 35, 256^3 6885 / 332, 512^3 109,690 / 3297: the FMA GEMM needs
+// 1.1 us per K step of a wave of tiles, the residue kernel ~25 us for its first
+// tile, so the line lies at 24 points whatever the other sizes.
+bool residue_pays(const tpt_plan_s* p, int d) { return p->n[d] >= 24 && p->n[d] <= tpt::kResidueMaxK; }
+
 int apply_transform(const tpt_plan_s* p, int d, bool inverse, const double* in, double* out,
-                    bool accumulate, void* oz, int* err, cudaStream_t s) {
+                    bool accumulate, void* scratch, int* err, cudaStream_t s) {
   if (p->dir[d].excluded()) {   // identity transform: no GEMM along a direction outside the operator
     if (!accumulate) return cuda_status(cudaMemcpyAsync(out, in, tpt::npts(p) * sizeof(double),
                                                         cudaMemcpyDeviceToDevice, s));
     return cuda_status(tpt::add_fp64(static_cast<long long>(tpt::npts(p)), in, out, s));
   }
   if (p->xform[d] == TPT_XFORM_FFT) return cuda_status(tpt::fft_fp64(p, d, inverse, in, out, accumulate, s));
-  if (p->ozaki) return cuda_status(tpt::ozaki_transform(p, d, inverse, in, out, accumulate, oz, err, s));
+  if (p->res[d].ready && scratch)
+    return cuda_status(tpt::residue_transform(p, d, inverse, in, out, accumulate, scratch, err, s));
   const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
   const double* mat = inverse ? p->ddir[d].inv : p->ddir[d].fwd;
   if (d == 0) {
@@ -104,12 +112,12 @@ size_t region_bytes(const tpt_plan_s* p) {
 
 // One correction solve: out (=|+=) Q_x Q_y (Thomas) Q_y^{-1} Q_x^{-1} rhs.
 int inner_fp64(const tpt_plan_s* p, const double* rhs, double* out, bool accumulate, double* t1,
-               double* t2, double* defect, void* oz, int* err, cudaStream_t s) {
-  TPT_TRY(apply_transform(p, 0, false, rhs, t1, false, oz, err, s));      // step 2.1
-  TPT_TRY(apply_transform(p, 1, false, t1, t2, false, oz, err, s));       // step 2.2
+               double* t2, double* defect, void* rs, int* err, cudaStream_t s) {
+  TPT_TRY(apply_transform(p, 0, false, rhs, t1, false, rs, err, s));      // step 2.1
+  TPT_TRY(apply_transform(p, 1, false, t1, t2, false, rs, err, s));       // step 2.2
   TPT_CUDA(tpt::thomas_fp64(p, t2, t2, t1, defect, s));                   // step 2.3
-  TPT_TRY(apply_transform(p, 1, true, t2, t1, false, oz, err, s));        // step 2.4
-  TPT_TRY(apply_transform(p, 0, true, t1, out, accumulate, oz, err, s));  // step 2.5
+  TPT_TRY(apply_transform(p, 1, true, t2, t1, false, rs, err, s));        // step 2.4
+  TPT_TRY(apply_transform(p, 0, true, t1, out, accumulate, rs, err, s));  // step 2.5
   return TPT_OK;
 }
 
@@ -159,9 +167,9 @@ int fp64_solve(tpt_plan_s* p, const double* f, double* phi, void* work, cudaStre
   }
   TPT_CUDA(cudaMemsetAsync(ds, 0, 16 * sizeof(double), s));
   TPT_CUDA(tpt::field_sums(p, fu, ds + 5, s));
-  void* oz = p->ozaki ? static_cast<void*>(w + 4 * rb) : nullptr;   // Ozaki scratch after fcopy
-  int* oz_err = reinterpret_cast<int*>(ds + 10);
-  TPT_TRY(inner_fp64(p, fu, phi, false, t1, t2, ds + 4, oz, oz_err, s));
+  void* rs = w + 4 * rb;   // scratch of the tensor-core transforms after fcopy
+  int* gemm_err = reinterpret_cast<int*>(ds + 10);
+  TPT_TRY(inner_fp64(p, fu, phi, false, t1, t2, ds + 4, rs, gemm_err, s));
   int iters = 1;
   const double np = static_cast<double>(tpt::npts(p));
   double fn2 = -1.0, rel = -1.0;
@@ -190,7 +198,7 @@ int fp64_solve(tpt_plan_s* p, const double* f, double* phi, void* work, cudaStre
       }
     }
     if (iters >= corrections) break;
-    TPT_TRY(inner_fp64(p, r, phi, true, t1, t2, ds, oz, oz_err, s));
+    TPT_TRY(inner_fp64(p, r, phi, true, t1, t2, ds, rs, gemm_err, s));
     ++iters;
   }
   // the canonical gauge: phi shifted to zero volume-weighted mean in physical
@@ -359,17 +367,17 @@ int create_plan_impl(const tpt_desc* desc, int cuda_device, tpt::BasisCache* cac
     st = tpt::mixed_setup(p);
     if (st != TPT_OK) return fail(st);
   }
+  p->ozaki = desc->precision == TPT_PREC_FP64_OZAKI;
+  for (int d = 0; d < 2 && p->precision == TPT_PREC_FP64; ++d) {   // residues of the transform matrices
+    if (p->dir[d].excluded() || p->xform[d] != TPT_XFORM_GEMM) continue;
+    if (p->ozaki && p->n[d] > tpt::kOzakiMaxK) return fail(TPT_ERR_UNSUPPORTED);
+    if (!p->ozaki && !residue_pays(p, d)) continue;
+    st = tpt::residue_setup(p, d);
+    if (st != TPT_OK) return fail(st);
+  }
   if (cudaStreamSynchronize(p->arena.stream) != cudaSuccess) {
     cudaGetLastError();
     return fail(TPT_ERR_CUDA);
-  }
-  if (desc->precision == TPT_PREC_FP64_OZAKI && p->dev >= 0) {   // slices of the transform matrices
-    st = tpt::ozaki_setup(p);
-    if (st != TPT_OK) return fail(st);
-    if (cudaStreamSynchronize(p->arena.stream) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(TPT_ERR_CUDA);
-    }
   }
   *out = p;
   return TPT_OK;
@@ -423,12 +431,15 @@ int solve_info(const tpt_plan_s* p, const double* h, tpt_info* info) {
   const double np = static_cast<double>(npts(p));
   const double fn2 = projected_norm2(h[5], h[6], h[7], np, p->vol, p->singular);
   const double rel = (fn2 > 0.0) ? std::sqrt(h[1] / fn2) : std::sqrt(h[1]);
+  int gemm_err;   // a bounded GEMM wait ran out
+  std::memcpy(&gemm_err, h + 10, sizeof(gemm_err));
   if (info) {
     std::memset(info, 0, sizeof(*info));
     info->iters = 1 + p->max_refine;
     info->rel_residual = rel;
     info->compat_defect = h[4];
   }
+  if (gemm_err) return TPT_ERR_TIMEOUT;
   if (!std::isfinite(rel)) return TPT_ERR_NONFINITE;
   if (p->rtol > 0.0 && !(rel <= p->rtol)) return TPT_ERR_NOT_CONVERGED;
   return TPT_OK;
@@ -648,7 +659,7 @@ int tpt_plan_get_tiles(tpt_plan p, int* tiles_out) {
 int tpt_workspace_bytes(tpt_plan p, size_t* bytes) {
   if (!p || !bytes) return TPT_ERR_INVALID_ARG;
   *bytes = (p->precision == TPT_PREC_FP64)
-               ? 256 + 4 * region_bytes(p) + (p->ozaki ? tpt::ozaki_scratch_bytes(p) : 0)
+               ? 256 + 4 * region_bytes(p) + tpt::residue_scratch_bytes(p)
                : tpt::mixed_workspace_bytes(p);
   return TPT_OK;
 }
@@ -679,9 +690,9 @@ int tpt_solve_host(tpt_plan p, const double* f_host, double* phi_host, double* f
 int tpt_transform(tpt_plan p, int dir, int inverse, const double* in, double* out, void* stream) {
   if (!on_device(p) || !in || !out || in == out || (dir != 0 && dir != 1)) return TPT_ERR_INVALID_ARG;
   DeviceGuard guard(p->dev);
-  if (p->ozaki && !p->oz_scratch)   // this entry point's own scratch, kept by the plan
-    TPT_CUDA(cudaMalloc(&p->oz_scratch, tpt::ozaki_scratch_bytes(p)));
-  return apply_transform(p, dir, inverse != 0, in, out, false, p->oz_scratch, nullptr,
+  if (p->ozaki && p->res[dir].ready && !p->res_scratch)   // this entry point's own scratch, kept by the plan
+    TPT_CUDA(cudaMalloc(&p->res_scratch, tpt::residue_scratch_bytes(p)));
+  return apply_transform(p, dir, inverse != 0, in, out, false, p->res_scratch, nullptr,
                          static_cast<cudaStream_t>(stream));
 }
 

@@ -114,8 +114,8 @@ __device__ __forceinline__ void store_chunk(const GemmOut& g, long long mterm, i
     return;
   }
   if (OUT == kOutF64 && acc) {
-    // float64 read-modify-write (the levels of an Ozaki product): every load
-    // of the chunk is issued before the first store, so the 32 loads overlap
+    // float64 read-modify-write: every load of the chunk is issued before the
+    // first store, so the 32 loads overlap
     double* o = static_cast<double*>(g.out0);
     double old[32];
 #pragma unroll
@@ -263,15 +263,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
     }
     return true;
   };
-  // products per tile (float64 levels), K chunks of product lv and its B offset
-  constexpr bool kLevels = OUT == kOutF64;
-  auto npass_of = [&](const GemmOut& gg) -> int { return (kLevels && gg.levels > 0) ? gg.levels : 1; };
-  auto nk_of = [&](const GemmOut& gg, int lv, int nkq) -> int {
-    return (kLevels && gg.levels > 0) ? ((lv + 1) * gg.level_k) / C::BK : nkq;
-  };
-  auto bofs_of = [&](const GemmOut& gg, int lv) -> int {
-    return (kLevels && gg.levels > 0) ? (gg.levels - 1 - lv) * gg.level_k : 0;
-  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::STAGES; ++s) {
@@ -320,10 +311,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
       const CUtensorMap* mB1 = MULTI ? &mq[3] : &tB1;
       volatile int* abort_q = MULTI ? reinterpret_cast<volatile int*>(gq->err) : abort_flag;
       last_err = gq->err;
-      const int npass = npass_of(*gq);
-      for (int lv = 0; lv < npass && ok; ++lv) {
-      const int nkp = nk_of(*gq, lv, nkq), kb = bofs_of(*gq, lv);
-      for (int kc = 0; kc < nkp; ++kc, ++it) {
+      for (int kc = 0; kc < nkq; ++kc, ++it) {
         const int s = static_cast<int>(it % C::STAGES);
         const long long round = it / C::STAGES;
         if (round > 0)
@@ -340,35 +328,34 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
         uint8_t* st = smem + s * C::STAGE;
         const uint32_t full = ptx::smem_u32(&bars[s]);
         ptx::mbar_arrive_expect_tx(full, C::STAGE);
-        const int kx = kc * C::BK, kxb = kx + kb;
+        const int kx = kc * C::BK;
         if (PAIR == 1) {          // own A; half of the shared B tile, to both CTAs
           const int hb = BN / 2;
           ptx::tma_load_2d(ptx::smem_u32(st), mA0, full, kx, m0);   // n0: the pair's common n-tile
-          ptx::tma_load_2d_mc(ptx::smem_u32(st + NPL * C::A_BYTES + rank * hb * C::SW), mB0, full, kxb,
+          ptx::tma_load_2d_mc(ptx::smem_u32(st + NPL * C::A_BYTES + rank * hb * C::SW), mB0, full, kx,
                               n0 + rank * hb, kPairMask);
           if (NPL == 2) {
             ptx::tma_load_2d(ptx::smem_u32(st + C::A_BYTES), mA1, full, kx, m0);
             ptx::tma_load_2d_mc(ptx::smem_u32(st + NPL * C::A_BYTES + C::B_BYTES + rank * hb * C::SW), mB1, full,
-                                kxb, n0 + rank * hb, kPairMask);
+                                kx, n0 + rank * hb, kPairMask);
           }
         } else if (PAIR == 2) {   // half of the shared A tile, to both CTAs; own B
           const int ha = BM / 2;
           ptx::tma_load_2d_mc(ptx::smem_u32(st + rank * ha * C::SW), mA0, full, kx, m0 + rank * ha, kPairMask);
-          ptx::tma_load_2d(ptx::smem_u32(st + NPL * C::A_BYTES), mB0, full, kxb, n0);
+          ptx::tma_load_2d(ptx::smem_u32(st + NPL * C::A_BYTES), mB0, full, kx, n0);
           if (NPL == 2) {
             ptx::tma_load_2d_mc(ptx::smem_u32(st + C::A_BYTES + rank * ha * C::SW), mA1, full, kx, m0 + rank * ha,
                                 kPairMask);
-            ptx::tma_load_2d(ptx::smem_u32(st + NPL * C::A_BYTES + C::B_BYTES), mB1, full, kxb, n0);
+            ptx::tma_load_2d(ptx::smem_u32(st + NPL * C::A_BYTES + C::B_BYTES), mB1, full, kx, n0);
           }
         } else {
           ptx::tma_load_2d(ptx::smem_u32(st), mA0, full, kx, m0);
-          ptx::tma_load_2d(ptx::smem_u32(st + NPL * C::A_BYTES), mB0, full, kxb, n0);
+          ptx::tma_load_2d(ptx::smem_u32(st + NPL * C::A_BYTES), mB0, full, kx, n0);
           if (NPL == 2) {
             ptx::tma_load_2d(ptx::smem_u32(st + C::A_BYTES), mA1, full, kx, m0);
-            ptx::tma_load_2d(ptx::smem_u32(st + NPL * C::A_BYTES + C::B_BYTES), mB1, full, kxb, n0);
+            ptx::tma_load_2d(ptx::smem_u32(st + NPL * C::A_BYTES + C::B_BYTES), mB1, full, kx, n0);
           }
         }
-      }
       }
     }
     // drain: every issued stage's copies have landed before the CTA may exit
@@ -392,9 +379,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
       if (!resolve(q, m0, n0, nkq, gq, mq)) continue;
       volatile int* abort_q = MULTI ? reinterpret_cast<volatile int*>(gq->err) : abort_flag;
       last_err = gq->err;
-      const int npass = npass_of(*gq);
-      for (int lv = 0; lv < npass && ok; ++lv) {
-      const int nkp = nk_of(*gq, lv, nkq);
       const int b = tcount & 1, use = tcount >> 1;
       ++tcount;
       if (use > 0)
@@ -406,7 +390,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
       }
       ptx::tc_fence_after();
       const uint32_t d = tmem + static_cast<uint32_t>(b * BN);
-      for (int kc = 0; kc < nkp; ++kc, ++it) {
+      for (int kc = 0; kc < nkq; ++kc, ++it) {
         const int s = static_cast<int>(it % C::STAGES);
         ok = ptx::mbar_wait(ptx::smem_u32(&bars[s]), static_cast<uint32_t>((it / C::STAGES) & 1), gq->err,
                             ptx::kErrWaitFull, polls);
@@ -433,7 +417,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
         else ptx::mma_commit(ptx::smem_u32(&bars[C::STAGES + s]));                  // in both CTAs
       }
       ptx::mma_commit(ptx::smem_u32(&accf[b]));                 // accumulator b ready
-      }
     }
     // every MMA this thread issued has completed before the tensor memory is
     // freed, also when a timed-out wait ended the loop early
@@ -465,9 +448,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
       const CUtensorMap* mO0 = MULTI ? &mq[4] : &tO0;
       const CUtensorMap* mO1 = MULTI ? &mq[5] : &tO1;
       volatile int* abort_q = MULTI ? reinterpret_cast<volatile int*>(gu.err) : abort_flag;
-      const int npass = npass_of(gu);
-      for (int lv = 0; lv < npass; ++lv) {
-      const bool acc_out = gu.accumulate != 0 || lv > 0;   // later levels add to the earlier ones
+      const bool acc_out = gu.accumulate != 0;
       const int b = tcount & 1, use = tcount >> 1;
       ++tcount;
       const bool ok = ptx::mbar_wait(ptx::smem_u32(&accf[b]), static_cast<uint32_t>(use & 1), gu.err,
@@ -531,7 +512,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&acce[b]));   // buffer b may be refilled
-      }
     }
     if (TMAO && lane == 0) ptx::bulk_wait_all();   // staging buffers stay until the stores are done
   }
@@ -728,6 +708,10 @@ cudaError_t launch_out(const Operand& A, const Operand& B, const GemmOut& g, cud
 }
 
 }  // namespace
+
+bool make_operand_map(CUtensorMap* map, const void* base, int rows, int K, int ld, int box_rows) {
+  return make_map(map, base, kKindBF16, rows, K, ld, box_rows, 128);
+}
 
 bool make_plain_map(CUtensorMap* map, const void* base, int elem_bytes, long long inner, long long outer,
                     long long row_stride_bytes, int box_inner, int box_outer) {

@@ -1,0 +1,742 @@
+// Float64 transform GEMMs on the bf16 tensor cores, exact in a residue number
+// system: the eigenbasis transforms of the float64 and Ozaki plans (Sec. 2.2.2
+// solution steps 2.1, 2.2, 2.4, 2.5; Algorithm 1 steps 1, 3, 7, 9).
+//
+// Method (Ozaki, Uchino and Imamura, "Ozaki Scheme II", 2025: integer products
+// by modular arithmetic and the Chinese remainder theorem).  Every row of an
+// operand (the K values one output contracts with) is rounded once to integers
+// on its own scale: |X_B| <= 2^bB for a line of the field, |X_A| <= 2^54 for a
+// row of the transform matrix.  For pairwise coprime moduli p_1 .. p_n with
+// product P, the integer product x = sum_k X_A X_B, |x| < P / 2, is fixed by
+// its residues, and each residue is one bf16 GEMM over centred residues
+// |r| <= rmax (exact in bf16 up to 256) with rmax^2 K <= 2^24, so that every
+// partial sum is an integer below 2^24 and the float32 accumulator is exact in
+// any order.  With  K = 512: 14 moduli below 364 (P > 2^117); K <= 256: 13
+// below 514.  Summing slice products instead (Ozaki scheme I, eight 7-bit
+// slices, 36 products) needs 2.6 times the tensor-core work for the same 54
+// bits.
+//
+// Reconstruction.  x / P mod 1 = sum_i (r_i y_i mod p_i) / p_i with
+// y_i = (P / p_i)^-1 mod p_i; y_i is folded into the matrix's residues, and the
+// sum is kept as a 64-bit binary fraction F in registers, whose wrap-around is
+// the "mod 1".  Two moduli are taken together: n = r_i p_j + r_j p_i (exact in
+// float32), F += n C + rint(n e) with C + e = 2^64 / (p_i p_j).  F is off by at
+// most half a unit per pair, 2^-61 P in all, which is below 2^-54 of a typical
+// |x| even though |x| is ~2^-9.5 P.  The matrix is scaled by P / 2^L (L the bit
+// length of P) when it is rounded, so x = F 2^(L-64) times powers of two and the
+// result is assembled from its bits: no operation of the float64 pipe (1/64 of
+// the float32 rate on GB300) is spent on a point, except the sum of an
+// accumulating transform.  The rounding of the operands (2^-54 of a row's
+// maximum) is the whole error; the float64 FMA chain it replaces rounds at each
+// of the K steps (relative 2-norm error of one transform of noise, K = 512: 9e-17
+// against 7.5e-16; K = 64: 9e-17 against 2.6e-16).
+//
+// Measured (GB300, one transform of 512^3 points): 3.3 ms along x, 4.1 ms along
+// y, where the float64 FMA GEMM, at that pipe's peak, takes 109.7 ms; 256^3 0.33
+// / 0.35 ms against 6.9.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <climits>
+#include <cmath>
+#include <cstdint>
+#include <cstring>
+#include <vector>
+
+#include "ptx.h"
+#include "residue.h"
+#include "tc.h"
+#include "tpt_internal.h"
+
+namespace tpt {
+namespace {
+
+size_t al256(size_t b) { return (b + 255) & ~static_cast<size_t>(255); }
+
+constexpr float kMagic = 12582912.0f;           // 1.5 * 2^23: adding it rounds to an integer
+constexpr uint32_t kMagicBits = 0x4B400000u;    // its bits; bits(kMagic + n) = kMagicBits + n
+
+// ------------------------------------------------------------------ residues of the operands
+
+// The bits of a row's maximum |x| -> e with max < 2^e (0 for a zero or
+// subnormal row, kRowNonFinite when the row holds an infinity or a NaN).
+constexpr int kRowNonFinite = INT_MAX;
+__device__ __forceinline__ int row_exponent(unsigned long long maxbits) {
+  const int ex = static_cast<int>(maxbits >> 52);
+  return ex == 0x7ff ? kRowNonFinite : ex == 0 ? 0 : ex - 1022;
+}
+
+// X = round(x 2^(b - e)) for |x| < 2^e, from the bits of x (subnormal: 0).
+__device__ __forceinline__ long long fixed_point(unsigned long long bits, int e, int b) {
+  const int ex = static_cast<int>((bits >> 52) & 0x7ff);
+  const unsigned long long mant = (bits & ((1ull << 52) - 1)) | (1ull << 52);
+  const int sh = 1075 - b + e - ex;   // x = mant 2^(ex - 1075)
+  long long X = sh <= 0 ? static_cast<long long>(mant << (-sh & 63))
+                        : static_cast<long long>((mant + (1ull << ((sh - 1) & 63))) >> (sh & 63));
+  if (ex == 0 || sh > 54) X = 0;
+  return static_cast<long long>(bits) < 0 ? -X : X;
+}
+
+// X in balanced base-2^14 digits as floats: X = l0 + 2^14 l1 + 2^28 l2 + 2^42 l3.
+__device__ __forceinline__ void limbs(long long X, float (&l)[4]) {
+  const unsigned long long Y = static_cast<unsigned long long>(X) + ((1ull << 13) + (1ull << 27) + (1ull << 41));
+  const uint32_t lo = static_cast<uint32_t>(Y);
+  const uint32_t m1 = static_cast<uint32_t>(Y >> 14) & 0x3fffu;
+  const uint32_t m2 = static_cast<uint32_t>(Y >> 28) & 0x3fffu;
+  const int top = static_cast<int>(static_cast<long long>(Y) >> 42);
+  l[0] = __uint_as_float(0x4B000000u | (lo & 0x3fffu)) - (8388608.0f + 8192.0f);
+  l[1] = __uint_as_float(0x4B000000u | m1) - (8388608.0f + 8192.0f);
+  l[2] = __uint_as_float(0x4B000000u | m2) - (8388608.0f + 8192.0f);
+  l[3] = __uint_as_float(kMagicBits + static_cast<uint32_t>(top)) - kMagic;
+}
+
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+
+// Residues of two neighbouring values (limbs as pairs) for every modulus:
+// v = 2^k X mod p up to a multiple of p, from the digits times 2^(k + 14 j) mod p
+// (|v| <= 2^23, exact), r = v - p rint(v / p), stored as two bf16 at dst + i * Kp for modulus i.  Paired float32
+// instructions; v / p is an odd multiple of 1/(2p) away from a tie by more
+// than the error of v * (1/p), so |r| <= p / 2 exactly.
+__device__ __forceinline__ void store_residues(const SliceConst& sc, int k, const float (&a)[4],
+                                               const float (&b)[4], __nv_bfloat16* dst, int Kp) {
+  const float2 l0 = make_float2(a[0], b[0]), l1 = make_float2(a[1], b[1]);
+  const float2 l2 = make_float2(a[2], b[2]), l3 = make_float2(a[3], b[3]);
+  const float2 mg = both(kMagic), nmg = both(-kMagic);
+#pragma unroll 2
+  for (int i = 0; i < sc.nm; ++i) {
+    const float4 c = sc.c[k][i];
+    float2 v = __fmul2_rn(l0, both(c.x));
+    v = __ffma2_rn(l1, both(c.y), v);
+    v = __ffma2_rn(l2, both(c.z), v);
+    v = __ffma2_rn(l3, both(c.w), v);
+    const float2 q = __fadd2_rn(__ffma2_rn(v, both(sc.inv[i]), mg), nmg);
+    const float2 r = __ffma2_rn(q, both(-sc.p[i]), v);
+    *reinterpret_cast<__nv_bfloat162*>(dst + static_cast<long long>(i) * Kp) = __float22bfloat162_rn(r);
+  }
+}
+
+// One line of K values (get(k): the bits of value k) by one warp: the row
+// exponent, then the residue planes; columns K..Kp-1 are zero.  A non-finite
+// line gets zero residues and the exponent kRowNonFinite, which the GEMM's
+// epilogue turns into NaN.
+template <typename Get>
+__device__ __forceinline__ void slice_line(const SliceConst& sc, int K, int Kp, Get get, __nv_bfloat16* dst,
+                                           int* expo, int lane) {
+  unsigned long long m = 0;
+  for (int k = lane; k < K; k += 32) m = max(m, get(k) & 0x7fffffffffffffffull);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  const int e = row_exponent(m);
+  // A line whose values are mostly small against its maximum has a product sum
+  // far below K max|X_A| max|X_B|: it is scaled up by the 2^up that its sum of
+  // |X_B| leaves free, by finer rounding and then by its residues' scale, so that
+  // x keeps the resolution of the fraction F.  t sums an upper bound of
+  // |x| / 2^(e - 20), from the leading 20 bits.
+  uint32_t t = 0;
+  for (int k = lane; k < K; k += 32) {
+    const uint32_t hi = static_cast<uint32_t>(get(k) >> 32);
+    const int d = e + 1022 - static_cast<int>((hi >> 20) & 0x7ff);
+    t += d < 20 && d >= 0 ? ((0x100000u | (hi & 0xfffffu)) >> (d + 1)) + 1u : 1u;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  int up = sc.L - 35 - sc.bits - (32 - __clz(static_cast<int>(t + 2u)));
+  up = up < 0 || e == kRowNonFinite ? 0 : up > kMaxUp ? kMaxUp : up;
+  if (lane == 0) *expo = e == kRowNonFinite ? e : e - up;
+  const int more = min(up, kMaxDataBits - sc.bits);   // as far as the digits reach, the line keeps more bits
+  const int bits = sc.bits + more;
+  up -= more;
+  for (int k = 2 * lane; k < Kp; k += 64) {
+    long long x0 = 0, x1 = 0;
+    if (e != kRowNonFinite) {
+      if (k < K) x0 = fixed_point(get(k), e, bits);
+      if (k + 1 < K) x1 = fixed_point(get(k + 1), e, bits);
+    }
+    float a[4], b[4];
+    limbs(x0, a);
+    limbs(x1, b);
+    store_residues(sc, up, a, b, dst + k, Kp);
+  }
+}
+
+// x lines: line r is K contiguous values at src + r K; one warp per line.
+__global__ void __launch_bounds__(256)
+slice_x_kernel(long long rows, int K, int Kp, const double* __restrict__ src, __nv_bfloat16* __restrict__ dst,
+               int* __restrict__ expo, const __grid_constant__ SliceConst sc) {
+  const int lane = threadIdx.x % 32;
+  const long long warps = static_cast<long long>(gridDim.x) * (blockDim.x / 32);
+  for (long long r = blockIdx.x * static_cast<long long>(blockDim.x / 32) + threadIdx.x / 32; r < rows; r += warps) {
+    const unsigned long long* row = reinterpret_cast<const unsigned long long*>(src) + r * K;
+    slice_line(sc, K, Kp, [&](int k) { return __ldg(row + k); }, dst + r * (static_cast<long long>(sc.nm) * Kp),
+               expo + r, lane);
+  }
+}
+
+// y lines of a slab of z planes: line (i, k) is the K = ny values at stride nx.
+// A block takes LB neighbouring lines of one plane through shared memory (rows
+// of LB * 8 bytes in, pitch odd in 8-byte words: no bank conflicts).
+template <int LB>
+__global__ void __launch_bounds__(256)
+slice_y_kernel(int nx, int K, int Kp, const double* __restrict__ src, __nv_bfloat16* __restrict__ dst,
+               int* __restrict__ expo, const __grid_constant__ SliceConst sc) {
+  extern __shared__ unsigned long long tile[];
+  const int pitch = K | 1;
+  const int tiles = (nx + LB - 1) / LB;
+  const long long plane = blockIdx.x / tiles;
+  const int i0 = static_cast<int>(blockIdx.x % tiles) * LB;
+  const unsigned long long* in = reinterpret_cast<const unsigned long long*>(src) + plane * nx * K;
+  for (int t = threadIdx.x; t < LB * K; t += blockDim.x) {
+    const int i = t % LB, j = t / LB;
+    if (i0 + i < nx) tile[i * pitch + j] = __ldg(in + i0 + i + static_cast<long long>(nx) * j);
+  }
+  __syncthreads();
+  const int lane = threadIdx.x % 32;
+  for (int i = threadIdx.x / 32; i < LB && i0 + i < nx; i += 8) {
+    const unsigned long long* row = tile + i * pitch;
+    const long long r = plane * nx + i0 + i;
+    slice_line(sc, K, Kp, [&](int k) { return row[k]; }, dst + r * (static_cast<long long>(sc.nm) * Kp), expo + r,
+               lane);
+  }
+}
+
+// Transform-matrix table: rows x K (element (r, k) at src[r rs + k cs]), row r
+// rounded to X_A = round(a 2^(54 - e) G / 2^64) and stored as the residues of
+// X_A y_i; one block per row.
+__global__ void __launch_bounds__(256)
+matrix_residues_kernel(int K, int Kp, long long rs, long long cs, const double* __restrict__ src,
+                       __nv_bfloat16* __restrict__ dst, int* __restrict__ expo,
+                       const __grid_constant__ MatrixConst mc) {
+  __shared__ unsigned long long wmax[8];
+  const long long r = blockIdx.x;
+  const unsigned long long* row = reinterpret_cast<const unsigned long long*>(src) + r * rs;
+  unsigned long long m = 0;
+  for (int k = threadIdx.x; k < K; k += blockDim.x) m = max(m, row[k * cs] & 0x7fffffffffffffffull);
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (threadIdx.x % 32 == 0) wmax[threadIdx.x / 32] = m;
+  __syncthreads();
+  for (int w = 0; w < 8; ++w) m = max(m, wmax[w]);
+  const int e = row_exponent(m);
+  if (threadIdx.x == 0) expo[r] = e;
+  for (int k = threadIdx.x; k < Kp; k += blockDim.x) {
+    long long X = 0;
+    if (k < K && e != kRowNonFinite) {
+      const unsigned long long bits = row[k * cs];
+      const int ex = static_cast<int>((bits >> 52) & 0x7ff);
+      if (ex != 0) {
+        const unsigned long long mant = (bits & ((1ull << 52) - 1)) | (1ull << 52);
+        const unsigned long long hi = __umul64hi(mant, mc.scale), lo = mant * mc.scale;
+        const int sh = 64 + 1075 - kMatrixBits + e - ex;   // >= 63: mant < 2^53, X <= 2^kMatrixBits
+        if (sh == 63) {
+          X = static_cast<long long>((hi << 1) | (lo >> 63)) + static_cast<long long>((lo >> 62) & 1);
+        } else if (sh == 64) {
+          X = static_cast<long long>(hi + (lo >> 63));
+        } else if (sh < 64 + 54) {
+          X = static_cast<long long>((hi + (1ull << (sh - 65))) >> (sh - 64));
+        }
+        if (bits >> 63) X = -X;
+      }
+    }
+    for (int i = 0; i < mc.nm; ++i) {
+      const int p = mc.p[i];
+      int v = static_cast<int>(X % p) * mc.y[i] % p;   // |v| < p
+      if (2 * v > p) v -= p;
+      if (2 * v < -p) v += p;
+      dst[(r * mc.nm + i) * Kp + k] = __float2bfloat16_rn(static_cast<float>(v));
+    }
+  }
+}
+
+// ------------------------------------------------------------------ the GEMM
+
+constexpr int BM = 128, BN = 128, BK = 64;
+constexpr int kABytes = BM * BK * 2, kBBytes = BN * BK * 2, kStage = kABytes + kBBytes;
+constexpr int kStages = 6;
+constexpr int kBufs = 4;                       // tensor-memory accumulators of BN columns
+constexpr int kEpiWarps = 16;
+constexpr int kCols = 4 * BN / kEpiWarps;       // columns of an epilogue thread
+constexpr int kThreads = 32 * (2 + kEpiWarps);
+constexpr int kSmem = kStages * kStage + 1024 /* alignment */ + 256 /* barriers */;
+
+// 2^k times the 64-bit integer F, rounded to nearest even
+__device__ __forceinline__ double assemble(long long F, int k) {
+  if (F == 0) return 0.0;
+  const unsigned long long a = F < 0 ? 0ull - static_cast<unsigned long long>(F) : static_cast<unsigned long long>(F);
+  const int lz = __clzll(static_cast<long long>(a));
+  const unsigned long long m = a << lz;
+  unsigned long long top = m >> 11;
+  const uint32_t rem = static_cast<uint32_t>(m) & 0x7ffu;
+  top += (rem + (static_cast<uint32_t>(top) & 1u) > 0x400u) ? 1u : 0u;
+  const int ex = 1085 - lz + k;                // exponent field less the hidden bit of top
+  if (ex < 0 || ex > 2044) {                   // subnormal or overflowing results
+    const double v = scalbn(static_cast<double>(top), 11 - lz + k);
+    return F < 0 ? -v : v;
+  }
+  unsigned long long bits = (static_cast<unsigned long long>(ex) << 52) + top;
+  if (F < 0) bits |= 1ull << 63;
+  return __longlong_as_double(static_cast<long long>(bits));
+}
+
+// D = A B^T through the residues of A (M rows) and B (N rows): persistent, one
+// CTA per SM, tiles of 128 x 128; for each tile the moduli in turn, each one
+// K = Kp bf16 product into its own tensor-memory accumulator (four of them:
+// two pairs, so the tensor cores run ahead while the epilogue folds a pair).
+//   warp 0     TMA producer (128-byte rows, 128-byte swizzle, six 32 KB stages)
+//   warp 1     tcgen05.mma issue; padding K steps of the last chunk are skipped
+//   warps 2-17 epilogue: a warp owns 32 rows x 32 columns, one 64-bit fraction
+//              per element in registers over all moduli (sixteen warps: four a
+//              scheduler, and half the unrolled code of eight)
+// Element (m, n) is written (or added) at (m % rm) + (m / rm) sm + n sn.  Every
+// wait is bounded; a timeout sets bits in *err and the CTA drains and exits.
+__global__ void __launch_bounds__(kThreads, 1)
+residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB,
+                    const __grid_constant__ ResidueGemm g) {
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStage);
+  uint64_t* accf = bars + 2 * kStages;          // accumulator full
+  uint64_t* acce = accf + kBufs;                // accumulator drained
+  uint64_t* mdone = acce + kBufs;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mdone + 1);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int num_m = (g.M + BM - 1) / BM, num_n = (g.N + BN - 1) / BN;
+  const long long tiles = static_cast<long long>(num_m) * num_n;
+  const int nk = g.Kp / BK;
+  // A timed-out CTA stops by its own bounded waits; the others look at the flag
+  // once a tile, with the load in flight over the tile before (a load per ring
+  // stage put ~700 cycles into the producer's loop).
+  auto aborted = [&]() -> int { return g.err ? *reinterpret_cast<volatile int*>(g.err) : 0; };
+  auto origin = [&](long long q, int& m0, int& n0) {
+    const long long f = g.n_fastest ? num_n : num_m;
+    const int lo = static_cast<int>(q % f), hi = static_cast<int>(q / f);
+    m0 = (g.n_fastest ? hi : lo) * BM;
+    n0 = (g.n_fastest ? lo : hi) * BN;
+  };
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      ptx::mbar_init(ptx::smem_u32(&bars[s]), 1);
+      ptx::mbar_init(ptx::smem_u32(&bars[kStages + s]), 1);
+    }
+    for (int b = 0; b < kBufs; ++b) {
+      ptx::mbar_init(ptx::smem_u32(&accf[b]), 1);
+      ptx::mbar_init(ptx::smem_u32(&acce[b]), kEpiWarps);
+    }
+    ptx::mbar_init(ptx::smem_u32(mdone), 1);
+    ptx::fence_mbar_init();
+  }
+  if (warp == 1) {
+    ptx::tmem_alloc(ptx::smem_u32(tmem_slot), kBufs * BN);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0 && lane == 0) {
+    ptx::prefetch_tmap(&tA);
+    ptx::prefetch_tmap(&tB);
+    bool ok = true;
+    long long it = 0;
+    int stop = 0;
+    for (long long q = blockIdx.x; q < tiles && ok && !stop; q += gridDim.x) {
+      int m0, n0;
+      origin(q, m0, n0);
+      stop = aborted();
+      for (int c = 0; c < g.nm * nk; ++c, ++it) {   // chunk c: modulus c / nk, K offset (c % nk) * 64
+        const int s = static_cast<int>(it % kStages);
+        const long long round = it / kStages;
+        if (round > 0)
+          ok = ptx::mbar_wait(ptx::smem_u32(&bars[kStages + s]), static_cast<uint32_t>((round - 1) & 1), g.err,
+                              ptx::kErrWaitEmpty);
+        if (!ok) break;
+        uint8_t* st = smem + s * kStage;
+        const uint32_t full = ptx::smem_u32(&bars[s]);
+        ptx::mbar_arrive_expect_tx(full, kStage);
+        ptx::tma_load_2d(ptx::smem_u32(st), &tA, full, c * BK, m0);
+        ptx::tma_load_2d(ptx::smem_u32(st + kABytes), &tB, full, c * BK, n0);
+      }
+    }
+    const long long first = it > kStages ? it - kStages : 0;
+    for (long long k = first; k < it; ++k)   // every issued copy has landed before the CTA may exit
+      ptx::mbar_wait(ptx::smem_u32(&bars[k % kStages]), static_cast<uint32_t>((k / kStages) & 1), g.err,
+                     ptx::kErrWaitDrain);
+  } else if (warp == 1) {
+    // The whole warp runs the loop and one elected lane issues: descriptors and
+    // barrier addresses stay in uniform registers (a lone thread building them
+    // took ~170 cycles per MMA, more than twice the MMA itself).
+    constexpr uint32_t idesc = ptx::instr_desc(1u, BM, BN);
+    const uint32_t issue = ptx::elect_one();
+    const uint64_t desc0 = ptx::smem_desc_k_sw128(ptx::smem_u32(smem));
+    const uint32_t bar0 = ptx::smem_u32(bars);
+    const int last = (g.K - (nk - 1) * BK + 15) / 16;   // K steps of the last chunk
+    bool ok = true;
+    uint32_t s = 0, par = 0, b = 0, bpar = 1, first = 1;   // ring stage and its parity; accumulator
+    int stop = 0;
+    for (long long q = blockIdx.x; q < tiles && ok; q += gridDim.x) {
+      if (__any_sync(0xffffffffu, stop)) break;
+      stop = aborted();
+      for (int i = 0; i < g.nm && ok; ++i) {
+        if (!first)
+          ok = ptx::mbar_wait_warp(bar0 + 8 * (2 * kStages + kBufs + b), bpar, g.err, ptx::kErrWaitAccum);
+        if (!ok) break;
+        ptx::tc_fence_after();
+        const uint32_t d = tmem + b * BN;
+        for (int kc = 0; kc < nk; ++kc) {
+          ok = ptx::mbar_wait_warp(bar0 + 8 * s, par, g.err, ptx::kErrWaitFull);
+          if (!ok) break;
+          ptx::tc_fence_after();
+          const uint64_t da = desc0 + s * (kStage >> 4), db = da + (kABytes >> 4);
+          const int steps = kc == nk - 1 ? last : BK / 16;
+#pragma unroll
+          for (int kk = 0; kk < BK / 16; ++kk)
+            if (kk < steps) ptx::mma_bf16_if(issue, d, da + 2 * kk, db + 2 * kk, idesc, (kc > 0 || kk > 0) ? 1u : 0u);
+          ptx::mma_commit_if(issue, bar0 + 8 * (kStages + s));
+          if (++s == kStages) {
+            s = 0;
+            par ^= 1;
+          }
+        }
+        ptx::mma_commit_if(issue, bar0 + 8 * (2 * kStages + b));
+        if (++b == kBufs) {
+          b = 0;
+          bpar ^= 1;
+          first = 0;
+        }
+      }
+    }
+    // every MMA has completed before the tensor memory is freed
+    ptx::mma_commit_if(issue, ptx::smem_u32(mdone));
+    ptx::mbar_wait_warp(ptx::smem_u32(mdone), 0u, g.err, ptx::kErrWaitDrain);
+  } else if (warp >= 2) {
+    const int quarter = warp % 4;                // tensor-memory lanes 32 * quarter ..
+    const int col0 = ((warp - 2) / 4) * kCols;
+    const float2 mg = both(kMagic), nmg = both(-kMagic);
+    long long t = 0;
+    bool go = true;
+    int stop = 0;
+    for (long long q = blockIdx.x; q < tiles && go; q += gridDim.x) {
+      int m0, n0;
+      origin(q, m0, n0);
+      if (__any_sync(0xffffffffu, stop)) break;   // tcgen05.ld is warp-collective
+      stop = aborted();
+      long long F[kCols];
+#pragma unroll
+      for (int c = 0; c < kCols; ++c) F[c] = g.f0;
+      for (int j = 0; j < g.npair; ++j) {
+        const ResiduePair& pr = g.pair[j];
+        const bool two = 2 * j + 1 < g.nm;
+        const int b0 = static_cast<int>(t % kBufs), b1 = static_cast<int>((t + 1) % kBufs);
+        bool ok = ptx::mbar_wait(ptx::smem_u32(&accf[b0]), static_cast<uint32_t>((t / kBufs) & 1), g.err,
+                                 ptx::kErrWaitAccum);
+        if (two && ok)
+          ok = ptx::mbar_wait(ptx::smem_u32(&accf[b1]), static_cast<uint32_t>(((t + 1) / kBufs) & 1), g.err,
+                              ptx::kErrWaitAccum);
+        ptx::tc_fence_after();
+        if (!__all_sync(0xffffffffu, ok)) {
+          go = false;
+          break;
+        }
+        const uint32_t base = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(col0);
+#pragma unroll
+        for (int c0 = 0; c0 < kCols; c0 += 8) {
+          uint32_t s1[8], s2[8];
+          ptx::tmem_ld_32x32b_x8(base + static_cast<uint32_t>(b0 * BN + c0), s1);
+          ptx::tmem_ld_32x32b_x8(base + static_cast<uint32_t>((two ? b1 : b0) * BN + c0), s2);
+          ptx::tmem_ld_wait();
+#pragma unroll
+          for (int c = 0; c < 8; c += 2) {
+            const float2 a = make_float2(__uint_as_float(s1[c]), __uint_as_float(s1[c + 1]));
+            const float2 b = make_float2(__uint_as_float(s2[c]), __uint_as_float(s2[c + 1]));
+            const float2 qa = __fadd2_rn(__ffma2_rn(a, both(pr.inv1), mg), nmg);
+            const float2 qb = __fadd2_rn(__ffma2_rn(b, both(pr.inv2), mg), nmg);
+            const float2 ra = __ffma2_rn(qa, both(-pr.p1), a);
+            const float2 rb = __ffma2_rn(qb, both(-pr.p2), b);
+            const float2 n = __ffma2_rn(ra, both(pr.f1), __fmul2_rn(rb, both(pr.f2)));
+            const float2 u = __fadd2_rn(n, mg);
+            const float2 v = __ffma2_rn(n, both(pr.e), mg);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int ui = __float_as_int(h ? u.y : u.x);
+              const uint32_t vi = __float_as_uint(h ? v.y : v.x);
+              long long w = static_cast<long long>(ui) * pr.clo + F[c0 + c + h];
+              w += static_cast<long long>(static_cast<unsigned long long>(static_cast<uint32_t>(ui * pr.chi)) << 32);
+              F[c0 + c + h] = w + vi;
+            }
+          }
+        }
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          ptx::mbar_arrive(ptx::smem_u32(&acce[b0]));
+          if (two) ptx::mbar_arrive(ptx::smem_u32(&acce[b1]));
+        }
+        t += two ? 2 : 1;
+      }
+      if (!go) break;
+      const int m = m0 + quarter * 32 + lane;
+      if (m < g.M) {
+        const int ea = g.expA[m];
+        double* out = g.out + (m % g.rm) + static_cast<long long>(m / g.rm) * g.sm;
+#pragma unroll
+        for (int c = 0; c < kCols; ++c) {
+          const int n = n0 + col0 + c;
+          if (n < g.N) {
+            const int eb = __ldg(g.expB + n);
+            double v = (ea == kRowNonFinite || eb == kRowNonFinite) ? __longlong_as_double(0x7ff8000000000000ll)
+                                                                    : assemble(F[c], ea + eb + g.shift);
+            double* o = out + static_cast<long long>(n) * g.sn;
+            if (g.accumulate) v += *o;
+            *o = v;
+          }
+        }
+      }
+    }
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == 1) ptx::tmem_dealloc(tmem, kBufs * BN);
+}
+
+// ------------------------------------------------------------------ host side
+
+int gcd(int a, int b) { return b ? gcd(b, a % b) : a; }
+
+// The inverse of a modulo p (coprime), 1 <= result < p (p is small).
+int inverse_mod(int a, int p) {
+  for (int x = 1; x < p; ++x)
+    if (static_cast<long long>(a) * x % p == 1) return x;
+  return 1;   // p == 1
+}
+
+}  // namespace
+
+bool residue_system(int K, ResidueSystem* s) {
+  if (K < 1 || K > kResidueMaxK) return false;
+  int rmax = 1;
+  while (rmax < 256 && static_cast<long long>(rmax + 1) * (rmax + 1) * K <= (1LL << 24)) ++rmax;
+  int lk = 0;
+  while ((1 << lk) < K) ++lk;
+  std::memset(s, 0, sizeof(*s));
+  unsigned __int128 P = 1;
+  for (int p = 2 * rmax + 1; p > 2; --p) {
+    if (p % 2 == 0 && p / 2 > rmax) continue;
+    bool coprime = true;
+    for (int i = 0; i < s->nm; ++i) coprime = coprime && gcd(p, s->p[i]) == 1;
+    if (!coprime) continue;
+    s->p[s->nm++] = p;
+    P *= static_cast<unsigned>(p);
+    int L = 0;
+    while (L < 128 && (P >> L) != 0) ++L;
+    // |x| <= K 2^bB (2^54 P / 2^L + 1/2) must stay below P / 2
+    const int bits = L - 2 - kMatrixBits - lk;
+    if (bits >= kDataBits) {
+      s->L = L;
+      s->bits = bits < kMaxDataBits ? bits : kMaxDataBits;
+      break;
+    }
+    if (s->nm == kMaxModuli) return false;
+  }
+  if (s->L == 0) return false;
+  s->scale = static_cast<unsigned long long>((P << (128 - s->L)) >> 64);
+  for (int i = 0; i < s->nm; ++i) {
+    int rest = 1;
+    for (int j = 0; j < s->nm; ++j)
+      if (j != i) rest = static_cast<int>(static_cast<long long>(rest) * s->p[j] % s->p[i]);
+    s->y[i] = inverse_mod(rest % s->p[i], s->p[i]);
+  }
+  return true;
+}
+
+namespace {
+
+SliceConst slice_const(const ResidueSystem& s) {
+  SliceConst c;
+  std::memset(&c, 0, sizeof(c));
+  c.nm = s.nm;
+  c.bits = s.bits;
+  c.L = s.L;
+  for (int i = 0; i < s.nm; ++i) {
+    const int p = s.p[i];
+    auto centred = [&](int bit) {
+      const long long v = (1LL << bit) % p;
+      return static_cast<float>(2 * v > p ? v - p : v);
+    };
+    for (int k = 0; k <= kMaxUp; ++k)
+      c.c[k][i] = make_float4(centred(k), centred(k + 14), centred(k + 28), centred(k + 42));
+    c.inv[i] = 1.0f / p;
+    c.p[i] = static_cast<float>(p);
+  }
+  return c;
+}
+
+void gemm_const(const ResidueSystem& s, ResidueGemm* g) {
+  g->nm = s.nm;
+  g->npair = (s.nm + 1) / 2;
+  unsigned long long f0 = 0;
+  for (int j = 0; j < g->npair; ++j) {
+    const int p1 = s.p[2 * j], p2 = 2 * j + 1 < s.nm ? s.p[2 * j + 1] : 1;
+    const int pp = p1 * p2;
+    const unsigned __int128 one = static_cast<unsigned __int128>(1) << 64;
+    const unsigned long long q = static_cast<unsigned long long>(one / pp);        // < 2^56
+    const int rem = static_cast<int>(one % pp);
+    // 2^64 / pp = C + e with |e| <= 1/2; C = chi 2^32 + clo, clo signed
+    const unsigned long long C = 2 * rem > pp ? q + 1 : q;
+    ResiduePair& pr = g->pair[j];
+    pr.e = static_cast<float>((2LL * rem > pp ? rem - pp : rem) / static_cast<double>(pp));
+    pr.clo = static_cast<int>(static_cast<uint32_t>(C));
+    pr.chi = static_cast<int>((C - static_cast<unsigned long long>(static_cast<long long>(pr.clo))) >> 32);
+    pr.p1 = static_cast<float>(p1);
+    pr.p2 = static_cast<float>(p2);
+    pr.inv1 = 1.0f / p1;
+    pr.inv2 = 1.0f / p2;
+    pr.f1 = static_cast<float>(p2);
+    pr.f2 = p2 == 1 ? 0.0f : static_cast<float>(p1);   // a lone modulus: its pair's accumulator does not count
+    f0 -= kMagicBits * C + kMagicBits;   // the magic offsets of u and v
+  }
+  g->f0 = static_cast<long long>(f0);
+  g->shift = s.L - 64 - kMatrixBits - s.bits;
+}
+
+// Lines of direction d that one pass slices and multiplies (the scratch holds
+// their residues): all of them when they fit in the plan's res_cap, else whole
+// z planes.
+long long lines_per_pass(const tpt_plan_s* p, int d) {
+  const ResidueDir& rd = p->res[d];
+  const long long per_plane = d == 0 ? p->n[1] : p->n[0];
+  const size_t line = static_cast<size_t>(rd.sys.nm) * rd.kp * 2 + sizeof(int);
+  long long planes = static_cast<long long>(p->res_cap / (line * static_cast<size_t>(per_plane)));
+  if (planes < 1) planes = 1;
+  if (planes > p->n[2]) planes = p->n[2];
+  return planes * per_plane;
+}
+
+}  // namespace
+
+int residue_setup(tpt_plan_s* p, int d) {
+  const int n = p->n[d];
+  ResidueDir& rd = p->res[d];
+  if (!residue_system(n, &rd.sys)) return TPT_ERR_UNSUPPORTED;
+  rd.kp = (n + BK - 1) / BK * BK;
+  const size_t tab = static_cast<size_t>(n) * rd.sys.nm * rd.kp * 2;
+  MatrixConst mc;
+  std::memset(&mc, 0, sizeof(mc));
+  mc.nm = rd.sys.nm;
+  mc.scale = rd.sys.scale;
+  for (int i = 0; i < rd.sys.nm; ++i) {
+    mc.p[i] = rd.sys.p[i];
+    mc.y[i] = rd.sys.y[i];
+  }
+  for (int inv = 0; inv < 2; ++inv) {
+    void* t = nullptr;
+    int st = p->arena.alloc(al256(tab) + static_cast<size_t>(n) * sizeof(int), &t);
+    if (st != TPT_OK) return st;
+    rd.tab[inv] = t;
+    rd.expo[inv] = reinterpret_cast<int*>(static_cast<char*>(t) + al256(tab));
+    // rows = output modes: x transforms read A[r][k] = mat[r + n k], y
+    // transforms B[r][k] = mat[k + n r]
+    const double* src = inv ? p->ddir[d].inv : p->ddir[d].fwd;
+    note_launch(1);
+    matrix_residues_kernel<<<n, 256, 0, p->arena.stream>>>(n, rd.kp, d == 0 ? 1 : n, d == 0 ? n : 1, src,
+                                                           static_cast<__nv_bfloat16*>(t), rd.expo[inv], mc);
+    if (cudaGetLastError() != cudaSuccess) return TPT_ERR_CUDA;
+  }
+  rd.ready = true;
+  return TPT_OK;
+}
+
+size_t residue_scratch_bytes(const tpt_plan_s* p) {
+  size_t most = 0;
+  for (int d = 0; d < 2; ++d) {
+    if (!p->res[d].ready) continue;
+    const size_t lines = static_cast<size_t>(lines_per_pass(p, d));
+    const size_t b = al256(lines * p->res[d].sys.nm * p->res[d].kp * 2) + al256(lines * sizeof(int));
+    if (b > most) most = b;
+  }
+  return most;
+}
+
+void residue_limit(tpt_plan_s* p, size_t bytes) {
+  p->res_cap = bytes;   // lines_per_pass leaves out the alignment of its two regions:
+  if (residue_scratch_bytes(p) > bytes && bytes > 512) p->res_cap = bytes - 512;
+  if (residue_scratch_bytes(p) > bytes && !p->ozaki) p->res[0].ready = p->res[1].ready = false;
+}
+
+cudaError_t residue_transform(const tpt_plan_s* p, int d, bool inverse, const double* in, double* out,
+                              bool accumulate, void* scratch, int* err, cudaStream_t s) {
+  const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
+  const ResidueDir& rd = p->res[d];
+  const int n = p->n[d], kp = rd.kp, ld = rd.sys.nm * kp;
+  int sms = 152;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->dev);
+  const long long per_pass = lines_per_pass(p, d);
+  const long long per_plane = d == 0 ? ny : nx, total = per_plane * nz, slab = static_cast<long long>(nx) * ny;
+  __nv_bfloat16* sl = static_cast<__nv_bfloat16*>(scratch);
+  int* expo = reinterpret_cast<int*>(static_cast<char*>(scratch) + al256(static_cast<size_t>(per_pass) * ld * 2));
+  const SliceConst sc = slice_const(rd.sys);
+  ResidueGemm g;
+  std::memset(&g, 0, sizeof(g));
+  gemm_const(rd.sys, &g);
+  g.K = n;
+  g.Kp = kp;
+  g.err = err;
+  g.accumulate = accumulate ? 1 : 0;
+  CUtensorMap mat, data;
+  const int tab = inverse ? 1 : 0;
+  if (!tc::make_operand_map(&mat, rd.tab[tab], n, ld, ld, 128)) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(residue_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e != cudaSuccess) return e;
+  for (long long l0 = 0; l0 < total; l0 += per_pass) {
+    const int lines = static_cast<int>(total - l0 < per_pass ? total - l0 : per_pass);
+    const long long off = l0 / per_plane * slab;   // first z plane of the pass
+    note_launch(2);
+    if (d == 0) {
+      const long long blocks = (lines + 7) / 8;
+      slice_x_kernel<<<static_cast<unsigned>(blocks < 16LL * sms ? blocks : 16LL * sms), 256, 0, s>>>(
+          lines, n, kp, in + off, sl, expo, sc);
+    } else {
+      const unsigned planes = static_cast<unsigned>(lines / nx);
+      auto run = [&](auto kern, int lb) -> cudaError_t {
+        const int bytes = lb * (n | 1) * 8;
+        const cudaError_t ea = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 1025 * 8);
+        if (ea != cudaSuccess) return ea;
+        kern<<<planes * static_cast<unsigned>((nx + lb - 1) / lb), 256, bytes, s>>>(nx, n, kp, in + off, sl, expo,
+                                                                                     sc);
+        return cudaGetLastError();
+      };
+      e = n <= 1024 ? run(slice_y_kernel<16>, 16) : run(slice_y_kernel<8>, 8);
+      if (e != cudaSuccess) return e;
+    }
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (!tc::make_operand_map(&data, sl, lines, ld, ld, 128)) return cudaErrorInvalidValue;
+    g.out = out + off;
+    g.sn = nx;
+    if (d == 0) {   // the matrix's rows are the output's x index
+      g.M = nx;
+      g.N = lines;
+      g.rm = nx;
+      g.sm = 0;
+      g.expA = rd.expo[tab];
+      g.expB = expo;
+      g.n_fastest = 0;
+    } else {
+      g.M = lines;
+      g.N = ny;
+      g.rm = nx;
+      g.sm = slab;
+      g.expA = expo;
+      g.expB = rd.expo[tab];
+      g.n_fastest = 1;
+    }
+    const long long tiles = static_cast<long long>((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
+    residue_gemm_kernel<<<static_cast<unsigned>(tiles < sms ? tiles : sms), kThreads, kSmem, s>>>(
+        d == 0 ? mat : data, d == 0 ? data : mat, g);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace tpt

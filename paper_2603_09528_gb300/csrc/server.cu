@@ -109,6 +109,14 @@ struct tpt_server_s {
       int st = tpt::create_plan(&r->desc, cfg.cuda_device, &cache, &p);
       size_t wb = 0;
       if (st == TPT_OK) st = tpt_workspace_bytes(p, &wb);
+      const size_t fields = 2 * r->npts * sizeof(double) + 3 * 256;
+      if (st == TPT_OK && cfg.cuda_device >= 0 && fields + wb > cfg.memory_budget) {
+        // a float64 request that only its transforms' scratch keeps out of the
+        // budget runs with less of it
+        const size_t rest = fields + wb - tpt::residue_scratch_bytes(p);
+        tpt::residue_limit(p, cfg.memory_budget > rest ? cfg.memory_budget - rest : 0);
+        st = tpt_workspace_bytes(p, &wb);
+      }
       std::lock_guard<std::mutex> g(mu);
       r->res.t_planned = now();
       if (st != TPT_OK) {
@@ -120,7 +128,7 @@ struct tpt_server_s {
       }
       r->plan = p;
       r->work_bytes = wb;
-      r->need = 2 * r->npts * sizeof(double) + wb + 3 * 256;
+      r->need = fields + wb;
       r->res.device_bytes = r->need;
       if (r->need > cfg.memory_budget) {   // can never fit: reject rather than wait forever
         tpt_plan_destroy(p);

@@ -46,13 +46,6 @@ struct GemmOut {
   // waits run out and the kernel returns with TPT_ERR_TIMEOUT in *err.
   unsigned polls = 0;
   int drop_loads = 0;
-  // Float64 output only: `levels` > 0 makes every tile a sequence of that
-  // many products accumulated into the output, product l over K = (l + 1) *
-  // level_k with A from K offset 0 and B from K offset (levels - 1 - l) *
-  // level_k (the levels of an Ozaki product, from operands holding all the
-  // slices); level_k a multiple of the 64-element K chunk.
-  int levels = 0;
-  int level_k = 0;
 };
 
 // One GEMM of a grouped launch: its tensor maps (A0, A1, B0, B1, O0, O1; the
@@ -80,6 +73,11 @@ int default_bn(int N);
 // encoder rejects the layout (base or stride not 16-byte aligned, box too large).
 bool make_plain_map(CUtensorMap* map, const void* base, int elem_bytes, long long inner, long long outer,
                     long long row_stride_bytes, int box_inner, int box_outer);
+
+// K-major bf16 operand map of the swizzled MMA layout: `rows` rows of K
+// elements, row stride ld elements, boxes of 64 elements (128-byte swizzle) x
+// box_rows.
+bool make_operand_map(CUtensorMap* map, const void* base, int rows, int K, int ld, int box_rows);
 
 cudaError_t gemm(int kind, int nplanes, const Operand& A, const Operand& B, const GemmOut& g,
                  cudaStream_t s);

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/tpt.h"
+#include "residue.h"
 
 namespace tpt {
 
@@ -162,13 +163,12 @@ struct tpt_plan_s {
   int ring_next = 0;
   double vol = 1.0;               // domain volume Lx Ly Lz
   tpt::MixedTables mixed;
-  // float64 transforms by the Ozaki scheme (TPT_PREC_FP64_OZAKI; ozaki.cu):
-  // bf16 slices of the four transform matrices (x forward, x inverse, y
-  // forward, y inverse) and the padded contraction lengths of x and y
-  bool ozaki = false;
-  void* oz_tab[4] = {nullptr, nullptr, nullptr, nullptr};
-  int oz_kp[2] = {0, 0};
-  void* oz_scratch = nullptr;      // scratch of the single-step transform entry point
+  // float64 GEMM transforms of x and y on the tensor cores (residue.cu); not
+  // ready: the float64 DGEMM
+  tpt::ResidueDir res[2];
+  size_t res_cap = tpt::kResidueScratch;   // bytes of residues per pass
+  bool ozaki = false;              // a TPT_PREC_FP64_OZAKI plan
+  void* res_scratch = nullptr;     // scratch of an Ozaki plan's single-step transform entry point
   int stage_timing = 0;           // record per-stage CUDA events in tpt_solve
   cudaEvent_t ev[12] = {};        // stage boundaries (created on first use)
   unsigned generation = 0;        // bumped when coefficients or tiles change
@@ -321,14 +321,18 @@ int group_enqueue(GroupSolve* g, double* d_scal, cudaStream_t s);
 // memory of 16 n doubles, after each step); synchronises s.
 int group_solve_adaptive(GroupSolve* g, double* d_scal, double* h_scal, cudaStream_t s);
 
-// Ozaki-scheme transforms (ozaki.cu): tables built at plan creation (the
-// float64 transform matrices must be on the device), scratch of one transform,
-// and the transform itself: out (+)= the float64-accurate transform of in.
-bool ozaki_supported(const tpt_plan_s* p);
-int ozaki_setup(tpt_plan_s* p);
-size_t ozaki_scratch_bytes(const tpt_plan_s* p);
-cudaError_t ozaki_transform(const tpt_plan_s* p, int d, bool inverse, const double* in, double* out,
-                            bool accumulate, void* scratch, int* err, cudaStream_t s);
+// Float64 transforms by residue arithmetic on the tensor cores (residue.cu):
+// the tables of direction d (built on the plan's stream from the float64
+// matrices already on the device), the scratch of one transform, and the
+// transform itself: out (+)= the transform of in.
+int residue_setup(tpt_plan_s* p, int d);
+size_t residue_scratch_bytes(const tpt_plan_s* p);
+// Bring that scratch down to `bytes` (before the plan's workspace is sized):
+// smaller passes, down to one z plane; a FP64 plan for which that is still too
+// much takes the float64 FMA GEMM.
+void residue_limit(tpt_plan_s* p, size_t bytes);
+cudaError_t residue_transform(const tpt_plan_s* p, int d, bool inverse, const double* in, double* out,
+                              bool accumulate, void* scratch, int* err, cudaStream_t s);
 
 // Times the transform GEMMs of a mixed plan over the candidate tiles and keeps
 // the fastest per stage (gemm_tune.cu).
