@@ -236,7 +236,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
   const int rank = PAIR ? static_cast<int>(ptx::cluster_ctarank()) : 0;
   constexpr uint16_t kPairMask = 0x3;
   const int nk = (g.K + C::BK - 1) / C::BK;
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(g.err);
+  // A timed-out CTA stops by its own bounded waits; the others look at the flag
+  // once a unit, the load in flight over the unit's work (a load per ring stage
+  // put ~700 cycles into the producer's loop).
+  auto aborted = [](const int* err) -> int { return err ? *reinterpret_cast<const volatile int*>(err) : 0; };
   const uint32_t polls = g.polls ? g.polls : (1u << 22);
   // unit q: its tile origin, K chunks, output description and tensor maps
   // (A0, A1, B0, B1, O0, O1); false when its job has stopped
@@ -300,7 +303,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
     bool ok = true;
     long long it = 0;
     int* last_err = g.err;
-    for (long long q = unit0; q < num_units && ok; q += unit_step) {
+    int stop = 0;
+    for (long long q = unit0; q < num_units && ok && !stop; q += unit_step) {
       int m0, n0, nkq;
       const GemmOut* gq;
       const CUtensorMap* mq;
@@ -309,18 +313,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
       const CUtensorMap* mA1 = MULTI ? &mq[1] : &tA1;
       const CUtensorMap* mB0 = MULTI ? &mq[2] : &tB0;
       const CUtensorMap* mB1 = MULTI ? &mq[3] : &tB1;
-      volatile int* abort_q = MULTI ? reinterpret_cast<volatile int*>(gq->err) : abort_flag;
       last_err = gq->err;
+      stop = aborted(last_err);
       for (int kc = 0; kc < nkq; ++kc, ++it) {
         const int s = static_cast<int>(it % C::STAGES);
         const long long round = it / C::STAGES;
         if (round > 0)
           ok = ptx::mbar_wait(ptx::smem_u32(&bars[C::STAGES + s]), static_cast<uint32_t>((round - 1) & 1), gq->err,
                               ptx::kErrWaitEmpty, polls);
-        if (!ok || (abort_q && *abort_q)) {
-          ok = false;
-          break;
-        }
+        if (!ok) break;
         if (g.drop_loads) {      // failure-detection test: no stage ever fills
           ok = false;
           break;
@@ -365,65 +366,71 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
     for (long long k = first; k < it; ++k)
       ptx::mbar_wait(ptx::smem_u32(&bars[k % C::STAGES]), static_cast<uint32_t>((k / C::STAGES) & 1), last_err,
                      ptx::kErrWaitDrain, polls);
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // -------------------------------------------------------- MMA issuer
+    // The whole warp runs the loop and one elected lane issues, so that
+    // descriptors and barrier addresses stay in uniform registers: a lone
+    // thread building them took ~170 cycles per MMA, more than the 128 of the
+    // MMA itself (128 x 256 x 16).  512^3: x forward 0.294 -> 0.248 ms, y
+    // forward 0.295 -> 0.260, x inverse 0.434 -> 0.354.
     constexpr uint32_t idesc = ptx::instr_desc(KIND == kKindBF16 ? 1u : 2u, BM, BN);
+    const uint32_t issue = ptx::elect_one();
+    const uint64_t desc0 = ptx::smem_desc_k_sw<C::SW>(ptx::smem_u32(smem));
+    const uint32_t bar0 = ptx::smem_u32(bars);
     bool ok = true;
-    long long it = 0;
+    uint32_t s = 0, par = 0;       // ring stage and its parity
     int tcount = 0;
     int* last_err = g.err;
+    int stop = 0;
     for (long long q = unit0; q < num_units && ok; q += unit_step) {
       int m0, n0, nkq;
       const GemmOut* gq;
       const CUtensorMap* mq;
       if (!resolve(q, m0, n0, nkq, gq, mq)) continue;
-      volatile int* abort_q = MULTI ? reinterpret_cast<volatile int*>(gq->err) : abort_flag;
+      if (__any_sync(0xffffffffu, stop)) break;
       last_err = gq->err;
-      const int b = tcount & 1, use = tcount >> 1;
+      stop = aborted(last_err);
+      const uint32_t b = tcount & 1;
+      const int use = tcount >> 1;
       ++tcount;
       if (use > 0)
-        ok = ptx::mbar_wait(ptx::smem_u32(&acce[b]), static_cast<uint32_t>((use - 1) & 1), gq->err,
-                            ptx::kErrWaitAccum, polls);
-      if (!ok || (abort_q && *abort_q)) {
-        ok = false;
-        break;
-      }
+        ok = ptx::mbar_wait_warp(bar0 + 8 * (2 * C::STAGES + 2 + b), static_cast<uint32_t>((use - 1) & 1), last_err,
+                                 ptx::kErrWaitAccum, polls);
+      if (!ok) break;
       ptx::tc_fence_after();
-      const uint32_t d = tmem + static_cast<uint32_t>(b * BN);
-      for (int kc = 0; kc < nkq; ++kc, ++it) {
-        const int s = static_cast<int>(it % C::STAGES);
-        ok = ptx::mbar_wait(ptx::smem_u32(&bars[s]), static_cast<uint32_t>((it / C::STAGES) & 1), gq->err,
-                            ptx::kErrWaitFull, polls);
+      const uint32_t d = tmem + b * BN;
+      for (int kc = 0; kc < nkq; ++kc) {
+        ok = ptx::mbar_wait_warp(bar0 + 8 * s, par, last_err, ptx::kErrWaitFull, polls);
         if (!ok) break;
         ptx::tc_fence_after();
-        const uint32_t sa = ptx::smem_u32(smem + s * C::STAGE);
-        const uint32_t sb = sa + NPL * C::A_BYTES;
+        const uint64_t da = desc0 + s * (C::STAGE >> 4), db = da + (NPL * C::A_BYTES >> 4);
 #pragma unroll
         for (int kk = 0; kk < C::BK / C::KI; ++kk) {
-          const uint32_t off = kk * C::KI * C::EB;   // bytes along the 128-byte row
+          const uint32_t off = kk * C::KI * C::EB >> 4;   // along the row
 #pragma unroll
           for (int p = 0; p < C::NPROD; ++p) {
             // products: (A0,B0), (A0,B1), (A1,B0)
-            const uint32_t a = sa + (p == 2 ? C::A_BYTES : 0) + off;
-            const uint32_t bb = sb + (p == 1 ? C::B_BYTES : 0) + off;
+            const uint64_t pa = da + (p == 2 ? C::A_BYTES >> 4 : 0) + off;
+            const uint64_t pb = db + (p == 1 ? C::B_BYTES >> 4 : 0) + off;
             const uint32_t acc = (kc > 0 || kk > 0 || p > 0) ? 1u : 0u;
-            if (KIND == kKindBF16)
-              ptx::mma_bf16(d, ptx::smem_desc_k_sw<C::SW>(a), ptx::smem_desc_k_sw<C::SW>(bb), idesc, acc);
-            else
-              ptx::mma_tf32(d, ptx::smem_desc_k_sw<C::SW>(a), ptx::smem_desc_k_sw<C::SW>(bb), idesc, acc);
+            if (KIND == kKindBF16) ptx::mma_bf16_if(issue, d, pa, pb, idesc, acc);
+            else ptx::mma_tf32_if(issue, d, pa, pb, idesc, acc);
           }
         }
-        if (PAIR) ptx::mma_commit_mc(ptx::smem_u32(&bars[C::STAGES + s]), kPairMask);   // frees the stage
-        else ptx::mma_commit(ptx::smem_u32(&bars[C::STAGES + s]));                  // in both CTAs
+        const uint32_t freed = bar0 + 8 * (C::STAGES + s);
+        if (PAIR) ptx::mma_commit_mc_if(issue, freed, kPairMask);   // frees the stage in both CTAs
+        else ptx::mma_commit_if(issue, freed);
+        if (++s == C::STAGES) {
+          s = 0;
+          par ^= 1;
+        }
       }
-      ptx::mma_commit(ptx::smem_u32(&accf[b]));                 // accumulator b ready
+      ptx::mma_commit_if(issue, bar0 + 8 * (2 * C::STAGES + b));   // accumulator b ready
     }
-    // every MMA this thread issued has completed before the tensor memory is
+    // every MMA this warp issued has completed before the tensor memory is
     // freed, also when a timed-out wait ended the loop early
-    if (it > 0) {
-      ptx::mma_commit(ptx::smem_u32(mdone));
-      ptx::mbar_wait(ptx::smem_u32(mdone), 0u, last_err, ptx::kErrWaitDrain, polls);
-    }
+    ptx::mma_commit_if(issue, ptx::smem_u32(mdone));
+    ptx::mbar_wait_warp(ptx::smem_u32(mdone), 0u, last_err, ptx::kErrWaitDrain, polls);
   } else if (warp >= 2) {
     // ---------------------------------------------------------- epilogue
     const int quarter = warp % 4;                  // tensor-memory lanes 32*quarter ..
@@ -447,14 +454,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
       const GemmOut& gu = *gq;
       const CUtensorMap* mO0 = MULTI ? &mq[4] : &tO0;
       const CUtensorMap* mO1 = MULTI ? &mq[5] : &tO1;
-      volatile int* abort_q = MULTI ? reinterpret_cast<volatile int*>(gu.err) : abort_flag;
+      const int flagged = aborted(gu.err);   // in flight over the wait below
       const bool acc_out = gu.accumulate != 0;
       const int b = tcount & 1, use = tcount >> 1;
       ++tcount;
       const bool ok = ptx::mbar_wait(ptx::smem_u32(&accf[b]), static_cast<uint32_t>(use & 1), gu.err,
                                      ptx::kErrWaitAccum, polls);
       ptx::tc_fence_after();
-      const bool flagged = abort_q && *abort_q;
       // tcgen05.ld is warp-collective: decide for the whole warp
       if (!__all_sync(0xffffffffu, ok && !flagged)) {
         go = false;
