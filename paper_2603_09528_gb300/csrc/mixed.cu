@@ -1511,7 +1511,7 @@ __device__ __forceinline__ float2 residual_pair_x2(const TermCoefs2& cx, const T
 
 // ---------------------------------------------------------------------------
 // TMA-staged residual.  A block owns a tile of kResTX x kResTY points of the
-// (x, y) plane and a segment of up to kResKseg planes; a producer warp
+// (x, y) plane and a segment of kseg <= kResKseg planes; a producer warp
 // streams, plane by plane, the phi pair with a halo (x from i0 - 4 to
 // i0 + kResTX + 4, rows j0 - 1 to j0 + kResTY) and the f pair of the tile into
 // a ring of shared-memory stages.  The tensor maps are 2D over the rows
@@ -1548,6 +1548,7 @@ struct ResJob {
   int* err;
   const int* skip;
   int first, tx, ty, tz;   // first block and tile counts of the instance
+  int kseg;                // planes of a block
 };
 
 template <int FMT, int HAS_ALPHA, int WX, int WY, int WZ, int SING>
@@ -1573,8 +1574,8 @@ __device__ __forceinline__ void residual_tma_body(const ResJob& J, int bx, int b
   TermCoefs2* xyc = reinterpret_cast<TermCoefs2*>(zc + kResKseg);   // [32 lanes | kResTY rows]
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int i0 = bx * kResTX, j0 = by * kResTY;
-  const int k0 = bz * kResKseg;
-  const int k1 = min(nz, k0 + kResKseg);
+  const int k0 = bz * J.kseg;
+  const int k1 = min(nz, k0 + J.kseg);
   const int nplanes = k1 - k0 + 2;                           // planes k0 - 1 .. k1
   if (threadIdx.x == 0) {
     for (int s = 0; s < kResStages; ++s) {
@@ -2495,9 +2496,40 @@ BRows rows_of(const float* t, int n) {
   return BRows{t, t + n, t + 2 * n, t + 3 * n, t + 4 * n, t + 5 * n};
 }
 
+int sm_count(int dev) {
+  int sms = 152;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) cudaGetLastError();
+  return sms;
+}
+
+// Planes of a residual block.  A plane costs a block ~0.6 us (one dependent
+// float-pair chain) however empty the chip is, and a block another ~6 planes'
+// worth of halo and start-up, so the segment is the one with the fewest planes
+// in sequence: rounds of blocks over the resident slots times (kseg + 6).
+// 512^3 keeps 64 planes (9 rounds); 64^3, whose eight tiles of 64 planes left
+// 144 SMs idle, takes 4: 39.5 -> 9.0 us.
+template <typename Blocks>
+int res_kseg(Blocks blocks, long long slots) {
+  int best = kResKseg;
+  long long cost = -1;
+  for (int k = kResKseg; k >= 4; k /= 2) {
+    const long long c = (blocks(k) + slots - 1) / slots * (k + 6);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = k;
+    }
+  }
+  return best;
+}
+
+long long res_blocks(const tpt_plan_s* p, int kseg) {
+  return static_cast<long long>((p->n[0] + kResTX - 1) / kResTX) * ((p->n[1] + kResTY - 1) / kResTY) *
+         ((p->n[2] + kseg - 1) / kseg);
+}
+
 // The residual job of a plan on workspace w with tensor maps m (phi pair,
-// f pair), its blocks numbered from `first`.
-ResJob res_job(const tpt_plan_s* p, const MixedWork& w, const CUtensorMap m[4], int first) {
+// f pair), kseg planes a block, its blocks numbered from `first`.
+ResJob res_job(const tpt_plan_s* p, const MixedWork& w, const CUtensorMap m[4], int kseg, int first) {
   const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
   ResJob J;
   std::memset(&J, 0, sizeof(J));
@@ -2528,7 +2560,8 @@ ResJob res_job(const tpt_plan_s* p, const MixedWork& w, const CUtensorMap m[4], 
   J.first = first;
   J.tx = (nx + kResTX - 1) / kResTX;
   J.ty = (ny + kResTY - 1) / kResTY;
-  J.tz = (nz + kResKseg - 1) / kResKseg;
+  J.kseg = kseg;
+  J.tz = (nz + kseg - 1) / kseg;
   return J;
 }
 
@@ -2560,7 +2593,9 @@ cudaError_t launch_res(const tpt_plan_s* p, const MixedWork& w, cudaStream_t s) 
       auto kern = residual_tma_kernel<FMT, HA, WX, WY, WZ, SING>;
       cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
       if (e != cudaSuccess) return e;
-      const ResJob J = res_job(p, w, m, 0);
+      // the kernel's blocks per SM (its launch bounds): three on a problem without walls or alpha
+      const long long slots = ((WX || WY || WZ || HA) ? 2LL : 3LL) * sm_count(p->dev);
+      const ResJob J = res_job(p, w, m, res_kseg([&](int k) { return res_blocks(p, k); }, slots), 0);
       kern<<<dim3(J.tx, J.ty, J.tz), kResThreads, kResSmem, s>>>(J);
       return cudaGetLastError();
     }
@@ -3620,7 +3655,16 @@ int group_prepare(GroupSolve* g, const double* const* f, double* const* phi, voi
     }
     CUtensorMap m4[4];
     if (!res_maps(p, ws[i], m4)) return TPT_ERR_UNSUPPORTED;
-    const ResJob R = res_job(p, ws[i], m4, rg[r].blocks);
+    // planes a block over every instance of the variant (two blocks per SM)
+    const int kseg = res_kseg(
+        [&](int ks) {
+          long long b = 0;
+          for (int q = 0; q < n; ++q)
+            if (res_code(g->plans[q]) == code) b += res_blocks(g->plans[q], ks);
+          return b;
+        },
+        2LL * sm_count(g->plans[0]->dev));
+    const ResJob R = res_job(p, ws[i], m4, kseg, rg[r].blocks);
     rg[r].blocks += R.tx * R.ty * R.tz;
     rj[r].push_back(R);
   }
