@@ -325,8 +325,8 @@ int tpt_project(tpt_plan plan, double* u, double* v, double* w, double gamma_dt,
  * zeros.  Errors: INVALID_ARG, CUDA, TIMEOUT.                              */
 int tpt_plan_autotune(tpt_plan plan, void* work_dev, void* stream, int* tiles_out);
 
-/* Set the four column-tile widths directly (0 = default: the smallest of
- * 32..256 covering the column count), e.g. to reuse a tuned choice on a plan
+/* Set the four column-tile widths directly (0 = default: chosen from the
+ * GEMM's size), e.g. to reuse a tuned choice on a plan
  * of the same shape.  Each width 0, 32, 64, 128 or 256, else INVALID_ARG.
  * Not to be called while a solve on this plan is in flight.                */
 int tpt_plan_set_tiles(tpt_plan plan, const int* tiles);

@@ -690,9 +690,35 @@ cudaError_t launch_pair(const Operand& A, const Operand& B, const GemmOut& g, cu
   return launch<KIND, NPL, BN, OUT, 0>(A, B, g, s);
 }
 
+// Column tile of a GEMM without a chosen one: rounds of tiles over the SMs times
+// (columns + 100), 100 columns being a tile's fixed cost (pipeline fill, first
+// loads).  It leaves the widest tile where rounds are many, takes two or three
+// narrower ones where they cover N with less padding (N = 277: 128 columns, y
+// inverse of 150x277x133 43.0 -> 28.7 us; N = 320: x forward of 320^3 86 -> 69)
+// and narrow ones where wide tiles would leave SMs idle (64^3 x inverse, 16
+// tiles of 256: 16.4 -> 10.2 us).
+int pick_bn(int M, int N) {
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    cudaGetLastError();
+  const long long mt = (M + BM - 1) / BM;
+  int best = 0;
+  long long cost = 0;
+  for (int bn = widest_bn(N); bn >= 32; bn /= 2) {
+    const long long tiles = mt * ((N + bn - 1) / bn);
+    const long long c = (tiles + sms - 1) / sms * (bn + 100);
+    if (best == 0 || c < cost) {
+      best = bn;
+      cost = c;
+    }
+  }
+  return best;
+}
+
 template <int KIND, int NPL, int OUT>
 cudaError_t launch_bn(const Operand& A, const Operand& B, const GemmOut& g, cudaStream_t s) {
-  switch (g.bn ? g.bn : default_bn(g.N)) {
+  switch (g.bn ? g.bn : pick_bn(g.M, g.N)) {
     case 32: return launch<KIND, NPL, 32, OUT, 0>(A, B, g, s);
     case 64: return launch<KIND, NPL, 64, OUT, 0>(A, B, g, s);
     case 128: return launch_pair<KIND, NPL, 128, OUT>(A, B, g, s);
@@ -820,7 +846,7 @@ bool own_device_memory(const void* p) {
   return a.type == cudaMemoryTypeDevice && a.device == dev;
 }
 
-int default_bn(int N) { return N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256; }
+int widest_bn(int N) { return N <= 32 ? 32 : N <= 64 ? 64 : N <= 128 ? 128 : 256; }
 
 cudaError_t gemm(int kind, int nplanes, const Operand& A, const Operand& B, const GemmOut& g,
                  cudaStream_t s) {

@@ -2241,23 +2241,51 @@ cudaError_t launch_prepare(const tpt_plan_s* p, const double* f, const MixedWork
   return cudaGetLastError();
 }
 
-// Tile width and segment length for Nz rows: 32-line tiles (16 segment slots)
-// up to Nz = 512, 16-line tiles (32 slots) above; M is the candidate whose
-// nseg = ceil(Nz / M) slots leave the fewest padding rows (ties: the smaller M).
-void thomas_shape(int nz, int* tlt, int* m_out) {
-  *tlt = nz <= 512 ? 32 : 16;
-  const int slots = kThomasThreads / *tlt;
+int sm_count(int dev) {
+  int sms = 152;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) cudaGetLastError();
+  return sms;
+}
+
+// Launch shape of thomas_tma_kernel: lines of a tile, threads of a CTA (512 / NT
+// CTAs per SM) and segment length for Nz rows and `lines` lines.
+struct ThomasShape {
+  int tlt, nt, m;
+};
+
+// A tile costs its CTA a fixed chain of barriers and reductions (~3 us) and a
+// serial sweep of its M-row segments (~0.1 us a row, padding rows included), so
+// with Nz small the 512-thread CTA spent its time on the chain, one tile at a
+// time (192x192x96 in tf32 35.5 us a step, 19.5 with four CTAs of 24-row
+// segments; 150x277x133 42.0 -> 30.4).  The shape is the one with the least rounds x (30 + M): 32-line tiles,
+// one, two or four CTAs per SM (16, 8 or 4 segments a line); 16-line tiles with
+// 32 segments above 512 rows.
+ThomasShape thomas_shape(int nz, long long lines, int sms) {
   static const int cand[] = {4, 8, 12, 16, 24, 32};
-  int best = 0, pad = 1 << 30;
-  for (int m : cand) {
-    const int nseg = (nz + m - 1) / m;
-    if (nseg > slots) continue;
-    if (nseg * m - nz < pad) {
-      pad = nseg * m - nz;
-      best = m;
+  ThomasShape best{32, kThomasThreads, 0};
+  if (nz > 512) best.tlt = 16;
+  long long cost = -1;
+  for (int nt = kThomasThreads; nt >= (nz > 512 ? kThomasThreads : 128); nt /= 2) {
+    const int slots = nt / best.tlt;
+    int m = 0, pad = 1 << 30;            // the fewest padding rows (ties: the smaller M)
+    for (int c : cand) {
+      const int nseg = (nz + c - 1) / c;
+      if (nseg > slots || (nt < kThomasThreads && c < 12)) continue;
+      if (nseg * c - nz < pad) {
+        pad = nseg * c - nz;
+        m = c;
+      }
+    }
+    if (m == 0) continue;
+    const long long tiles = (lines + best.tlt - 1) / best.tlt, per = static_cast<long long>(sms) * (kThomasThreads / nt);
+    const long long c = (tiles + per - 1) / per * (30 + m);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best.nt = nt;
+      best.m = m;
     }
   }
-  *m_out = best;
+  return best;
 }
 
 // Stage geometry and ring size of thomas_tma_kernel; false when the shared
@@ -2288,7 +2316,9 @@ cudaError_t launch_thomas_m(const tpt_plan_s* p, const MixedWork& w, cudaStream_
   if (ntiles <= 0) return cudaSuccess;
   if (lines + TLT > 0x7fffffffLL) return cudaErrorInvalidValue;   // int line indices and TMA coordinates
   ThomasGeom geo;
-  if (!thomas_geom(nz, M, TLT, O::NPL, O::EB, &geo, kThomasSmemBudget / kPerSm)) return cudaErrorInvalidConfiguration;
+  // several CTAs per SM: each also holds its static arrays and the system's share
+  const int budget = kThomasSmemBudget / kPerSm - (kPerSm > 1 ? 2048 : 0);
+  if (!thomas_geom(nz, M, TLT, O::NPL, O::EB, &geo, budget)) return cudaErrorInvalidConfiguration;
   CUtensorMap mi, mo0, mo1;
   if (!tc::make_plain_map(&mi, w.B[0], 4, lines, nz, lines * 4, TLT, geo.rb)) return cudaErrorInvalidValue;
   if (!tc::make_plain_map(&mo0, w.A[0], O::EB, lines, nz, lines * O::EB, TLT, geo.rb)) return cudaErrorInvalidValue;
@@ -2428,8 +2458,10 @@ cudaError_t launch_thomas2_m(const tpt_plan_s* p, const MixedWork& w, cudaStream
 
 // Thomas kernel for a plan: 1 one line per thread (thomas_tma_kernel), 2 two
 // lines per thread (thomas2_kernel); `variant` 0 picks the two-line kernel
-// where its segments are at least 8 rows long (Nz from 193 to 512), where it
-// has work for all but a few of its threads.
+// where its segments are at least 8 rows long (Nz from 193 to 512; 256^3 41.8
+// against 46.1 us).  Below, its tiles are as fast (64^3 5.9 against 6.8 us) but
+// on a singular problem its block-wide null line takes 19 us (64^3 24.6 in all)
+// where the one-warp kernel beside thomas_tma_kernel takes 10.
 int thomas_variant(int nz, int variant) {
   if (variant == 1) return 1;
   const int m2 = thomas2_m(nz);
@@ -2461,8 +2493,7 @@ cudaError_t launch_thomas(const tpt_plan_s* p, const MixedWork& w, cudaStream_t 
     if (e != cudaSuccess) return e;
   }
   cudaError_t e = cudaErrorInvalidConfiguration;
-  int tlt = 0, mm = 0;
-  thomas_shape(nz, &tlt, &mm);
+  const ThomasShape sh = thomas_shape(nz, static_cast<long long>(m.ldy) * p->n[0], sm_count(p->dev));
   if (two) {
     switch (thomas2_m(nz)) {
       case 4: e = launch_thomas2_m<FMT, 4>(p, w, s); break;
@@ -2471,8 +2502,24 @@ cudaError_t launch_thomas(const tpt_plan_s* p, const MixedWork& w, cudaStream_t 
       case 16: e = launch_thomas2_m<FMT, 16>(p, w, s); break;
       default: break;
     }
-  } else if (tlt == 32) {
-    switch (mm) {
+  } else if (sh.nt == 128) {
+    switch (sh.m) {
+      case 12: e = launch_thomas_m<FMT, 12, 32, 128>(p, w, s); break;
+      case 16: e = launch_thomas_m<FMT, 16, 32, 128>(p, w, s); break;
+      case 24: e = launch_thomas_m<FMT, 24, 32, 128>(p, w, s); break;
+      case 32: e = launch_thomas_m<FMT, 32, 32, 128>(p, w, s); break;
+      default: break;
+    }
+  } else if (sh.nt == 256) {
+    switch (sh.m) {
+      case 12: e = launch_thomas_m<FMT, 12, 32, 256>(p, w, s); break;
+      case 16: e = launch_thomas_m<FMT, 16, 32, 256>(p, w, s); break;
+      case 24: e = launch_thomas_m<FMT, 24, 32, 256>(p, w, s); break;
+      case 32: e = launch_thomas_m<FMT, 32, 32, 256>(p, w, s); break;
+      default: break;
+    }
+  } else if (sh.tlt == 32) {
+    switch (sh.m) {
       case 4: e = launch_thomas_m<FMT, 4, 32>(p, w, s); break;
       case 8: e = launch_thomas_m<FMT, 8, 32>(p, w, s); break;
       case 12: e = launch_thomas_m<FMT, 12, 32>(p, w, s); break;
@@ -2482,7 +2529,7 @@ cudaError_t launch_thomas(const tpt_plan_s* p, const MixedWork& w, cudaStream_t 
       default: break;
     }
   } else {
-    switch (mm) {
+    switch (sh.m) {
       case 24: e = launch_thomas_m<FMT, 24, 16>(p, w, s); break;
       case 32: e = launch_thomas_m<FMT, 32, 16>(p, w, s); break;
       default: break;
@@ -2496,12 +2543,6 @@ BRows rows_of(const float* t, int n) {
   return BRows{t, t + n, t + 2 * n, t + 3 * n, t + 4 * n, t + 5 * n};
 }
 
-int sm_count(int dev) {
-  int sms = 152;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) cudaGetLastError();
-  return sms;
-}
-
 // Planes of a residual block.  A plane costs a block ~0.6 us (one dependent
 // float-pair chain) however empty the chip is, and a block another ~6 planes'
 // worth of halo and start-up, so the segment is the one with the fewest planes
@@ -2512,7 +2553,7 @@ template <typename Blocks>
 int res_kseg(Blocks blocks, long long slots) {
   int best = kResKseg;
   long long cost = -1;
-  for (int k = kResKseg; k >= 4; k /= 2) {
+  for (int k = kResKseg; k >= 4; --k) {
     const long long c = (blocks(k) + slots - 1) / slots * (k + 6);
     if (cost < 0 || c < cost) {
       cost = c;
@@ -3818,7 +3859,7 @@ int autotune_gemms(tpt_plan_s* p, void* work, cudaStream_t s) {
   for (int i = 0; i < 4 && status == TPT_OK; ++i) {
     if (p->xform[stage_dir(i)] == TPT_XFORM_FFT) continue;   // no GEMM to tune
     const StageGemm t = stage_gemm(p, w, i, false);
-    const int top = tc::default_bn(t.g.N);
+    const int top = tc::widest_bn(t.g.N);
     // the operand common to neighbouring tiles: the transform matrix, which
     // is B for the x forward and y inverse stages and A for the other two
     const int share = (i == 0 || i == 2) ? 1 : 2;

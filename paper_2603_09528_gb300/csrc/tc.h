@@ -34,7 +34,7 @@ struct GemmOut {
   int accumulate;   // float-pair and float64 modes: add into the output instead of writing
   int n_fastest;    // tile order: n fastest (A tile reused by consecutive CTAs)
   int* err;         // device flag for timed-out waits (may be null)
-  int bn = 0;       // column tile width 32/64/128/256; 0 picks the smallest >= N
+  int bn = 0;       // column tile width 32/64/128/256; 0: chosen from M and N
   int max_ctas = 0; // cap on the persistent CTAs; 0 = one per SM
   int pair = 0;     // two-CTA clusters sharing an operand tile by TMA multicast:
                     // 1 = pairs of m-tiles share B, 2 = pairs of n-tiles share A
@@ -64,8 +64,8 @@ struct GemmJob {
 // a pair (TMA multicast) is used only when every operand plane passes.
 bool own_device_memory(const void* p);
 
-// Column tile width used when GemmOut::bn is 0.
-int default_bn(int N);
+// Widest useful column tile: the smallest of 32..256 covering N, at most 256.
+int widest_bn(int N);
 
 // Unswizzled 2D tensor map over `outer` rows of `inner` elements (2-byte
 // bf16 or 4-byte float32), row stride in bytes, box of box_inner x
