@@ -111,11 +111,13 @@ size_t region_bytes(const tpt_plan_s* p) {
 }
 
 // One correction solve: out (=|+=) Q_x Q_y (Thomas) Q_y^{-1} Q_x^{-1} rhs.
+// pivots (may be null: t1 serves) keeps the reciprocal pivots for the solve's
+// later corrections, which find them there (kept).
 int inner_fp64(const tpt_plan_s* p, const double* rhs, double* out, bool accumulate, double* t1,
-               double* t2, double* defect, void* rs, int* err, cudaStream_t s) {
+               double* t2, double* pivots, bool kept, double* defect, void* rs, int* err, cudaStream_t s) {
   TPT_TRY(apply_transform(p, 0, false, rhs, t1, false, rs, err, s));      // step 2.1
   TPT_TRY(apply_transform(p, 1, false, t1, t2, false, rs, err, s));       // step 2.2
-  TPT_CUDA(tpt::thomas_fp64(p, t2, t2, t1, defect, s));                   // step 2.3
+  TPT_CUDA(tpt::thomas_fp64(p, t2, t2, pivots ? pivots : t1, defect, s, pivots && kept));   // step 2.3
   TPT_TRY(apply_transform(p, 1, true, t2, t1, false, rs, err, s));        // step 2.4
   TPT_TRY(apply_transform(p, 0, true, t1, out, accumulate, rs, err, s));  // step 2.5
   return TPT_OK;
@@ -169,7 +171,8 @@ int fp64_solve(tpt_plan_s* p, const double* f, double* phi, void* work, cudaStre
   TPT_CUDA(tpt::field_sums(p, fu, ds + 5, s));
   void* rs = w + 4 * rb;   // scratch of the tensor-core transforms after fcopy
   int* gemm_err = reinterpret_cast<int*>(ds + 10);
-  TPT_TRY(inner_fp64(p, fu, phi, false, t1, t2, ds + 4, rs, gemm_err, s));
+  double* pivots = fu == f ? fcopy : nullptr;   // the region of f's copy is free unless phi overwrites f
+  TPT_TRY(inner_fp64(p, fu, phi, false, t1, t2, pivots, false, ds + 4, rs, gemm_err, s));
   int iters = 1;
   const double np = static_cast<double>(tpt::npts(p));
   double fn2 = -1.0, rel = -1.0;
@@ -198,7 +201,7 @@ int fp64_solve(tpt_plan_s* p, const double* f, double* phi, void* work, cudaStre
       }
     }
     if (iters >= corrections) break;
-    TPT_TRY(inner_fp64(p, r, phi, true, t1, t2, ds, rs, gemm_err, s));
+    TPT_TRY(inner_fp64(p, r, phi, true, t1, t2, pivots, true, ds, rs, gemm_err, s));
     ++iters;
   }
   // the canonical gauge: phi shifted to zero volume-weighted mean in physical

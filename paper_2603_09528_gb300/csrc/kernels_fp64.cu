@@ -10,6 +10,7 @@
 
 #include <cmath>
 
+#include "df.h"
 #include "tpt_internal.h"
 
 namespace tpt {
@@ -79,32 +80,43 @@ dgemm_cm_kernel(int M, int N, int K, const double* __restrict__ A, int lda, long
   }
 }
 
-// 1 / m in float64 without a division: the float32 reciprocal as the seed
-// (relative error below 2^-21) and two Newton steps r <- r + r (1 - m r), each
-// of which squares the relative error (2^-42, then below the float64
-// rounding).  Pivots outside the float32 range take the division.
+// 1 / m in float64 without a division: the float32 reciprocal of the leading 24
+// bits as the seed r0 (relative error below 2^-21) and one third-order step
+// r0 (1 + e + e^2), e = 1 - m r0, whose error e^3 is below the float64 rounding.
+// The seed's conversions are integer operations, so a reciprocal costs the
+// float64 pipe three FMAs.  Pivots outside the float32 range take the division.
 __device__ __forceinline__ double recip_fp64(double m) {
-  const float rf = __fdividef(1.0f, static_cast<float>(m));
-  if (!(fabsf(rf) < 1.0e37f && fabsf(rf) > 1.0e-37f)) return 1.0 / m;
-  double r = static_cast<double>(rf);
-  r = fma(r, fma(-m, r, 1.0), r);
-  return fma(r, fma(-m, r, 1.0), r);
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(m));
+  const unsigned e = static_cast<unsigned>(b >> 52) & 0x7ffu;
+  if (e - 900u > 240u) return 1.0 / m;
+  const float fm = __uint_as_float((static_cast<unsigned>(b >> 63) << 31) | ((e - 896u) << 23) |
+                                   (static_cast<unsigned>(b >> 29) & 0x7fffffu));
+  const double r0 = f2d_int(__fdividef(1.0f, fm));
+  const double d = fma(-m, r0, 1.0);
+  return fma(r0, fma(d, d, d), r0);
 }
 
-// One thread per (i, j) line.  Forward elimination keeps c' in `scratch`
-// and d' in `out`; back substitution overwrites `out`.  The singular line
-// (null_i, null_j) is first projected to compatible form (its dz-weighted
-// mean removed, recorded in *defect), its last modal unknown is set to zero,
-// and the result is shifted to zero dz-weighted mean.  The beta-scaled z rows
-// are staged in shared memory once per block (3 Nz doubles, dynamic) when
-// ROWS is set; the pipe that bounds the kernel is GB300's float64 pipe, so
-// the per-point work is kept to two DFMA, the reciprocal and two multiplies
-// forward and one DFMA back.  f may alias out (each element is read before
-// the same thread writes it).
-template <bool ROWS>
+// One thread per (i, j) line.  Forward elimination keeps the reciprocal pivots
+// in `inv` and d' in `out`; back substitution overwrites `out`.  With KEPT the
+// reciprocal pivots are already in `inv` (from an earlier call with the same
+// coefficients and sizes) and are only read.  The singular line (null_i,
+// null_j) is first projected to compatible form (its dz-weighted mean removed,
+// recorded in *defect), its last modal unknown is set to zero, and the result
+// is shifted to zero dz-weighted mean.  The beta-scaled z rows are staged in
+// shared memory once per block (3 Nz doubles, dynamic) when ROWS is set.  f may
+// alias out (each element is read before the same thread writes it).
+//
+// GB300's float64 pipe (2 FMA a cycle per SM) bounds large fields: 10 operations
+// a point, 5 with KEPT, where the loads (24 B a point) come near the pipe.
+// Small ones are bound by the chain along a line, so rows are read kAhead at a
+// time, one group ahead of the sweep (the loads of a row waited for the row
+// before: 2300 cycles a row), and the blocks are small enough to reach every SM.
+// 512^3 3.53 -> 2.73 ms, 1.31 with KEPT; 61x97x75 83 -> 45 and 25 us.
+constexpr int kAhead = 8;
+template <bool ROWS, bool KEPT>
 __global__ void __launch_bounds__(128)
 thomas_fp64_kernel(int nx, int ny, int nz, const double* f, double* out,
-                   double* __restrict__ scratch, const double* __restrict__ lamx,
+                   double* __restrict__ inv, const double* __restrict__ lamx,
                    const double* __restrict__ lamy, const double* __restrict__ az,
                    const double* __restrict__ bz, const double* __restrict__ cz,
                    const double* __restrict__ dz, double alpha, double beta, int null_i,
@@ -137,38 +149,82 @@ thomas_fp64_kernel(int nx, int ny, int nz, const double* f, double* out,
     fshift = s / w;
     if (defect) *defect = fshift * null_scale;
   }
-  double cp = 0.0, dp = 0.0;
-  for (int k = 0; k < nz; ++k) {
-    const long long o = line + k * lines;
-    const double sub = ra(k);
-    const double m = fma(-sub, cp, rb(k) + shift);
-    double fo = f[o];
-    if (is_null) fo -= fshift;
-    const double rhs = fma(-sub, dp, fo);
-    if (is_null && k == nz - 1) {
-      dp = 0.0;   // vanishing final pivot: the modal unknown is set to zero
-    } else {
-      const double inv = recip_fp64(m);
-      cp = rc(k) * inv;
-      dp = rhs * inv;
+  const double* fl = f + line;
+  double* ol = out + line;
+  double* il = inv + line;
+  double fv[kAhead], iv[kAhead];       // rows of the coming group
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int k = k0 + u;
+      fv[u] = k < nz ? fl[k * lines] : 0.0;
+      if (KEPT) iv[u] = k < nz ? il[k * lines] : 0.0;
     }
-    scratch[o] = cp;
-    out[o] = dp;
+  };
+  double cp = 0.0, dp = 0.0;
+  fetch(0);
+  for (int k0 = 0; k0 < nz; k0 += kAhead) {
+    double fc[kAhead], ic[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      fc[u] = fv[u];
+      ic[u] = KEPT ? iv[u] : 0.0;
+    }
+    fetch(k0 + kAhead);
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int k = k0 + u;
+      if (k < nz) {
+        const double sub = ra(k);
+        const double fo = is_null ? fc[u] - fshift : fc[u];
+        const double rhs = fma(-sub, dp, fo);
+        if (!KEPT) {
+          ic[u] = recip_fp64(fma(-sub, cp, rb(k) + shift));
+          if (is_null && k == nz - 1) ic[u] = 0.0;   // vanishing final pivot: the modal unknown is set to zero
+          cp = rc(k) * ic[u];
+          il[k * lines] = ic[u];
+        }
+        dp = rhs * ic[u];
+        ol[k * lines] = dp;
+      }
+    }
   }
+  // back substitution x_k = d'_k - c_k inv_k x_{k+1}, from the last row up
   double x = dp;
-  for (int k = nz - 2; k >= 0; --k) {
-    const long long o = line + k * lines;
-    x = fma(-scratch[o], x, out[o]);
-    out[o] = x;
+  auto fetch_back = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int k = k0 - u;
+      fv[u] = k >= 0 ? ol[k * lines] : 0.0;
+      iv[u] = k >= 0 ? il[k * lines] : 0.0;
+    }
+  };
+  fetch_back(nz - 2);
+  for (int k0 = nz - 2; k0 >= 0; k0 -= kAhead) {
+    double fc[kAhead], ic[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      fc[u] = fv[u];
+      ic[u] = iv[u];
+    }
+    fetch_back(k0 - kAhead);
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int k = k0 - u;
+      if (k >= 0) {
+        x = fma(-(rc(k) * ic[u]), x, fc[u]);
+        ol[k * lines] = x;
+      }
+    }
   }
   if (is_null) {
     double xs = 0.0, w = 0.0;
     for (int k = 0; k < nz; ++k) {
-      xs = fma(dz[k], out[line + k * lines], xs);
+      xs = fma(dz[k], ol[k * lines], xs);
       w += dz[k];
     }
     const double mean = xs / w;
-    for (int k = 0; k < nz; ++k) out[line + k * lines] -= mean;
+    for (int k = 0; k < nz; ++k) ol[k * lines] -= mean;
   }
 }
 
@@ -438,10 +494,13 @@ cudaError_t dgemm_cm(int M, int N, int K, const double* A, int lda, long long sA
 }
 
 cudaError_t thomas_fp64(const tpt_plan_s* p, const double* fhat, double* phihat, double* scratch,
-                        double* defect, cudaStream_t s) {
+                        double* defect, cudaStream_t s, bool kept) {
   const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
   const long long lines = static_cast<long long>(nx) * ny;
-  const int bs = 128;
+  int sms = 152;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->dev);
+  int bs = 128;
+  while (bs > 32 && lines < 2LL * sms * bs) bs /= 2;   // two blocks per SM, down to a warp
   const long long nb = (lines + bs - 1) / bs;
   const double* rz = p->d_rows[2];
   // f-hat of the null line equals (g_x g_y) times the physical constant
@@ -449,7 +508,8 @@ cudaError_t thomas_fp64(const tpt_plan_s* p, const double* fhat, double* phihat,
   const size_t rows_bytes = 3 * static_cast<size_t>(nz) * sizeof(double);
   const bool rows = rows_bytes <= 48 * 1024;   // within the default dynamic limit
   note_launch();
-  auto kern = rows ? thomas_fp64_kernel<true> : thomas_fp64_kernel<false>;
+  auto kern = rows ? (kept ? thomas_fp64_kernel<true, true> : thomas_fp64_kernel<true, false>)
+                   : (kept ? thomas_fp64_kernel<false, true> : thomas_fp64_kernel<false, false>);
   kern<<<static_cast<unsigned>(nb), bs, rows ? rows_bytes : 0, s>>>(
       nx, ny, nz, fhat, phihat, scratch, p->ddir[0].lam, p->ddir[1].lam, rz, rz + nz, rz + 2 * nz,
       p->d_dxf[2], p->alpha, p->beta, p->singular ? p->null_i : -1, p->singular ? p->null_j : -1,

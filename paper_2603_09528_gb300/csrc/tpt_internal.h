@@ -248,8 +248,10 @@ struct FftMixedArgs {
 };
 cudaError_t fft_mixed(const FftMixedArgs& a, cudaStream_t s);
 
+// scratch receives the reciprocal pivots (Nx*Ny*Nz doubles); with `kept` it
+// holds them already, from a call with the same coefficients.
 cudaError_t thomas_fp64(const tpt_plan_s* p, const double* fhat, double* phihat, double* scratch,
-                        double* defect, cudaStream_t s);
+                        double* defect, cudaStream_t s, bool kept = false);
 
 // out += in over n values
 cudaError_t add_fp64(long long n, const double* in, double* out, cudaStream_t s);
