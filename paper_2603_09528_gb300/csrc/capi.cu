@@ -168,7 +168,9 @@ int fp64_solve(tpt_plan_s* p, const double* f, double* phi, void* work, cudaStre
     fu = fcopy;
   }
   TPT_CUDA(cudaMemsetAsync(ds, 0, 16 * sizeof(double), s));
-  TPT_CUDA(tpt::field_sums(p, fu, ds + 5, s));
+  // the norm of f and the residual's: only where someone reads them
+  const bool report = adaptive || info || enqueue_only;
+  if (report) TPT_CUDA(tpt::field_sums(p, fu, ds + 5, s));
   void* rs = w + 4 * rb;   // scratch of the tensor-core transforms after fcopy
   int* gemm_err = reinterpret_cast<int*>(ds + 10);
   double* pivots = fu == f ? fcopy : nullptr;   // the region of f's copy is free unless phi overwrites f
@@ -189,10 +191,9 @@ int fp64_solve(tpt_plan_s* p, const double* f, double* phi, void* work, cudaStre
   int status = TPT_OK;
   bool converged = false;
   for (;;) {
-    const bool need_residual = (iters < corrections) || adaptive || info || enqueue_only;
-    if (!need_residual) break;
-    TPT_CUDA(cudaMemsetAsync(ds + 1, 0, 3 * sizeof(double), s));
-    TPT_CUDA(tpt::residual_fp64(p, fu, phi, r, ds + 1, p->singular ? ds + 4 : nullptr, s));
+    if (iters >= corrections && !report) break;
+    if (iters > 1) TPT_CUDA(cudaMemsetAsync(ds + 1, 0, 3 * sizeof(double), s));
+    TPT_CUDA(tpt::residual_fp64(p, fu, phi, r, report ? ds + 1 : nullptr, p->singular ? ds + 4 : nullptr, s));
     if (adaptive) {
       TPT_TRY(read_residual());
       if (rel <= p->rtol) {

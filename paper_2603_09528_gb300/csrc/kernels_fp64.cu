@@ -235,7 +235,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // r = (f - fshift) - (alpha phi + beta (Lx + Ly + Lz) phi); one thread per
-// (i, j) marching along k.  End couplings of non-periodic directions are zero,
+// (i, j) marching along kseg planes (blockIdx.z picks them).  End couplings of non-periodic directions are zero,
 // so wrapped neighbour indices only ever meet a zero coefficient.  The
 // beta-scaled rows are formed once (x and y per thread, z per block in shared
 // memory when ROWS, with alpha folded into the z diagonal), so that a point
@@ -251,11 +251,12 @@ residual_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ f,
                      const double* __restrict__ rz, const double* __restrict__ dxf,
                      const double* __restrict__ dyf, const double* __restrict__ dzf,
                      double alpha, double beta, const double* __restrict__ fshift_p,
-                     double* sums) {
+                     double* sums, int kseg) {
   extern __shared__ double zrow[];   // beta a_k, beta b_k + alpha, beta c_k (ROWS)
+  const int k0 = blockIdx.z * kseg, k1 = min(nz, k0 + kseg);
   if (ROWS) {
     const int tid = threadIdx.x + blockDim.x * threadIdx.y, nt = blockDim.x * blockDim.y;
-    for (int k = tid; k < nz; k += nt) {
+    for (int k = k0 + tid; k < k1; k += nt) {
       zrow[k] = beta * rz[k];
       zrow[nz + k] = fma(beta, rz[nz + k], alpha);
       zrow[2 * nz + k] = beta * rz[2 * nz + k];
@@ -275,9 +276,9 @@ residual_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ f,
     const double bxy = beta * (rx[nx + i] + ry[ny + j]);
     const double fshift = fshift_p ? *fshift_p : 0.0;
     const double vxy = ALL ? dxf[i] * dyf[j] : 0.0;
-    double pm = phi[base + sz * (nz - 1)];   // wrap partner, multiplied by a_0 = 0
-    double p0 = phi[base];
-    for (int k = 0; k < nz; ++k) {
+    double pm = phi[base + sz * (k0 == 0 ? nz - 1 : k0 - 1)];   // k = 0: wrap partner, multiplied by a_0 = 0
+    double p0 = phi[base + sz * k0];
+    for (int k = k0; k < k1; ++k) {
       const long long o = base + sz * k;
       const double pp = phi[base + sz * ((k == nz - 1) ? 0 : k + 1)];
       const double az = ROWS ? zrow[k] : beta * rz[k];
@@ -317,36 +318,53 @@ residual_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ f,
   }
 }
 
-// sums[0] += sum f^2, sums[1] += sum f, sums[2] += sum vol*f  (grid-stride)
+// sums[0] += sum f^2 and, with ALL, sums[1] += sum f, sums[2] += sum vol*f: one
+// warp per x-line (its weight dy_j dz_k once a line), one atomic per block and
+// sum.  One float64 operation a point, three with ALL; the pipe bounds it.
+template <bool ALL>
 __global__ void __launch_bounds__(256)
-field_sums_kernel(int nx, int ny, int nz, const double* __restrict__ f, const double* __restrict__ dxf,
+field_sums_kernel(int nx, int ny, long long lines, const double* __restrict__ f, const double* __restrict__ dxf,
                   const double* __restrict__ dyf, const double* __restrict__ dzf, double* sums) {
-  const long long n = static_cast<long long>(nx) * ny * nz;
+  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
   double s2 = 0.0, s1 = 0.0, sv = 0.0;
-  for (long long o = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; o < n;
-       o += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int i = static_cast<int>(o % nx);
-    const long long jk = o / nx;
-    const int j = static_cast<int>(jk % ny), k = static_cast<int>(jk / ny);
-    const double v = f[o];
-    s2 = fma(v, v, s2);
-    s1 += v;
-    sv = fma(dxf[i] * dyf[j] * dzf[k], v, sv);
+  for (long long L = blockIdx.x * 8LL + warp; L < lines; L += gridDim.x * 8LL) {
+    const double* row = f + L * nx;
+    double sl = 0.0;
+    for (int i = lane; i < nx; i += 32) {
+      const double v = row[i];
+      s2 = fma(v, v, s2);
+      if (ALL) {
+        s1 += v;
+        sl = fma(dxf[i], v, sl);
+      }
+    }
+    if (ALL) sv = fma(dyf[L % ny] * dzf[L / ny], sl, sv);
   }
+  __shared__ double sh[3][8];
   s2 = warp_sum(s2);
-  s1 = warp_sum(s1);
-  sv = warp_sum(sv);
-  if (threadIdx.x % 32 == 0) {
-    atomicAdd(&sums[0], s2);
-    atomicAdd(&sums[1], s1);
-    atomicAdd(&sums[2], sv);
+  if (ALL) {
+    s1 = warp_sum(s1);
+    sv = warp_sum(sv);
+  }
+  if (lane == 0) {
+    sh[0][warp] = s2;
+    sh[1][warp] = s1;
+    sh[2][warp] = sv;
+  }
+  __syncthreads();
+  if (threadIdx.x < (ALL ? 3 : 1)) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += sh[threadIdx.x][w];
+    atomicAdd(&sums[threadIdx.x], t);
   }
 }
 
-// Canonical gauge (reading R4): the volume-weighted mean of phi, summed
-// with error-free additions (TwoSum) so that the mean is exact to a few ulps
+// Canonical gauge (reading R4): the volume-weighted mean of phi to a few ulps
 // of the sum of |vol phi| whatever the cancellation, in two deterministic
-// levels: block partial sums as (hi, lo) pairs, then one block over them.
+// levels: a warp sums an x-line with FMAs (Nx / 32 terms a lane) and the lines
+// with error-free additions (TwoSum), block partial sums as (hi, lo) pairs,
+// then one block over them.  (TwoSum at every point cost ten operations of the
+// float64 pipe: 512^3 2.21 ms, now 0.38.)
 __device__ __forceinline__ void two_sum_d(double a, double b, double& s, double& e) {
   s = a + b;
   const double bb = s - a;
@@ -363,18 +381,17 @@ __global__ void __launch_bounds__(256)
 wsum_partial_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ phi, const double* __restrict__ dxf,
                          const double* __restrict__ dyf, const double* __restrict__ dzf, double2* partial) {
   const long long lines = static_cast<long long>(ny) * nz;
+  const int lane = threadIdx.x % 32;
   double hi = 0.0, lo = 0.0;
-  for (long long L = blockIdx.x; L < lines; L += gridDim.x) {   // x-line (j, k) = L
-    const int j = static_cast<int>(L % ny), k = static_cast<int>(L / ny);
-    const double wyz = dyf[j] * dzf[k];
+  for (long long L = blockIdx.x * 8LL + threadIdx.x / 32; L < lines; L += gridDim.x * 8LL) {   // x-line (j, k)
     const double* row = phi + static_cast<long long>(nx) * L;
-    for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-      const double v = (dxf[i] * wyz) * row[i];
-      double s, e;
-      two_sum_d(hi, v, s, e);
-      hi = s;
-      lo += e;
-    }
+    double sl = 0.0;
+    for (int i = lane; i < nx; i += 32) sl = fma(dxf[i], row[i], sl);
+    const double v = (dyf[L % ny] * dzf[L / ny]) * sl;
+    double s, e;
+    two_sum_d(hi, v, s, e);
+    hi = s;
+    lo += e;
   }
   __shared__ double sh[2][256];
   sh[0][threadIdx.x] = hi;
@@ -447,7 +464,7 @@ cudaError_t remove_weighted_mean(const tpt_plan_s* p, double* phi, void* scratch
   long long cap = static_cast<long long>(scratch_bytes / sizeof(double2));
   if (cap > 4LL * dev_sms) cap = 4LL * dev_sms;
   if (cap < 1) return cudaErrorInvalidValue;
-  const int nb = static_cast<int>(lines < cap ? lines : cap);
+  const int nb = static_cast<int>((lines + 7) / 8 < cap ? (lines + 7) / 8 : cap);
   double2* partial = static_cast<double2*>(scratch);
   note_launch(3);
   wsum_partial_fp64_kernel<<<nb, 256, 0, s>>>(p->n[0], p->n[1], p->n[2], phi, p->d_dxf[0], p->d_dxf[1],
@@ -463,12 +480,13 @@ cudaError_t remove_weighted_mean(const tpt_plan_s* p, double* phi, void* scratch
 cudaError_t field_sums(const tpt_plan_s* p, const double* f, double* sums, cudaStream_t s) {
   int dev_sms = 152;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, p->dev);
-  const long long n = static_cast<long long>(p->n[0]) * p->n[1] * p->n[2];
-  long long nb = (n + 255) / 256;
+  const long long lines = static_cast<long long>(p->n[1]) * p->n[2];
+  long long nb = (lines + 7) / 8;
   if (nb > 8LL * dev_sms) nb = 8LL * dev_sms;
   note_launch();
-  field_sums_kernel<<<static_cast<unsigned>(nb), 256, 0, s>>>(p->n[0], p->n[1], p->n[2], f, p->d_dxf[0],
-                                                              p->d_dxf[1], p->d_dxf[2], sums);
+  auto kern = p->singular ? field_sums_kernel<true> : field_sums_kernel<false>;   // only then are the others read
+  kern<<<static_cast<unsigned>(nb), 256, 0, s>>>(p->n[0], p->n[1], lines, f, p->d_dxf[0], p->d_dxf[1], p->d_dxf[2],
+                                                 sums);
   return cudaGetLastError();
 }
 
@@ -522,6 +540,16 @@ cudaError_t residual_fp64(const tpt_plan_s* p, const double* f, const double* ph
   const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
   dim3 block(32, 4);
   dim3 grid((nx + 31) / 32, (ny + 3) / 4);
+  // planes of a block: as many as leave eight blocks per SM (a plane is a
+  // dependent chain of loads and float64 operations, ~0.7 us), at least four;
+  // 61x97x75 51 -> 15 us, 32^3 27 -> 8.5 us
+  int sms = 152;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->dev);
+  const long long tiles = static_cast<long long>(grid.x) * grid.y;
+  long long segs = (8LL * sms + tiles - 1) / tiles;
+  if (segs > (nz + 3) / 4) segs = (nz + 3) / 4;
+  const int kseg = static_cast<int>((nz + segs - 1) / segs);
+  grid.z = (nz + kseg - 1) / kseg;
   const size_t rows_bytes = 3 * static_cast<size_t>(nz) * sizeof(double);
   const bool rows = rows_bytes <= 48 * 1024;   // within the default dynamic limit
   auto kern = rows ? (all_sums ? residual_fp64_kernel<true, true> : residual_fp64_kernel<true, false>)
@@ -529,7 +557,7 @@ cudaError_t residual_fp64(const tpt_plan_s* p, const double* f, const double* ph
   note_launch();
   kern<<<grid, block, rows ? rows_bytes : 0, s>>>(nx, ny, nz, f, phi, r, p->d_rows[0], p->d_rows[1], p->d_rows[2],
                                                  p->d_dxf[0], p->d_dxf[1], p->d_dxf[2], p->alpha, p->beta,
-                                                 fshift, sums);
+                                                 fshift, sums, kseg);
   return cudaGetLastError();
 }
 
