@@ -31,9 +31,9 @@
 // of the K steps (relative 2-norm error of one transform of noise, K = 512: 9e-17
 // against 7.5e-16; K = 64: 9e-17 against 2.6e-16).
 //
-// Measured (GB300, one transform of 512^3 points): 3.3 ms along x, 4.1 ms along
-// y, where the float64 FMA GEMM, at that pipe's peak, takes 109.7 ms; 256^3 0.33
-// / 0.35 ms against 6.9.
+// Measured (GB300, one transform of 512^3 points): 3.0 ms along x, 3.1 ms along
+// y (GEMM 2.0, slicing 1.0 and 1.1), where the float64 FMA GEMM, at that pipe's
+// peak, takes 109.7 ms; 256^3 0.30 ms against 6.9.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -93,26 +93,31 @@ __device__ __forceinline__ void limbs(long long X, float (&l)[4]) {
 
 __device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
 
-// Residues of two neighbouring values (limbs as pairs) for every modulus:
-// v = 2^k X mod p up to a multiple of p, from the digits times 2^(k + 14 j) mod p
-// (|v| <= 2^23, exact), r = v - p rint(v / p), stored as two bf16 at dst + i * Kp for modulus i.  Paired float32
-// instructions; v / p is an odd multiple of 1/(2p) away from a tie by more
-// than the error of v * (1/p), so |r| <= p / 2 exactly.
-__device__ __forceinline__ void store_residues(const SliceConst& sc, int k, const float (&a)[4],
-                                               const float (&b)[4], __nv_bfloat16* dst, int Kp) {
-  const float2 l0 = make_float2(a[0], b[0]), l1 = make_float2(a[1], b[1]);
-  const float2 l2 = make_float2(a[2], b[2]), l3 = make_float2(a[3], b[3]);
+// Residues of four values, two neighbouring pairs (limbs l[j] as pairs), for
+// every modulus: v = 2^k X mod p up to a multiple of p, from the digits times
+// 2^(k + 14 j) mod p (|v| <= 2^23, exact), r = v - p rint(v / p), stored as two
+// bf16 at dst + i * Kp for modulus i (and dst + 64 + i * Kp for the second pair
+// when `two`).  Paired float32 instructions, and the constants of a modulus
+// loaded once for both pairs; v / p is an odd multiple of 1/(2p) away from a tie
+// by more than the error of v * (1/p), so |r| <= p / 2 exactly.
+__device__ __forceinline__ void store_residues(const SliceConst& sc, int k, const float2 (&l)[2][4], bool two,
+                                               __nv_bfloat16* dst, int Kp) {
   const float2 mg = both(kMagic), nmg = both(-kMagic);
 #pragma unroll 2
   for (int i = 0; i < sc.nm; ++i) {
     const float4 c = sc.c[k][i];
-    float2 v = __fmul2_rn(l0, both(c.x));
-    v = __ffma2_rn(l1, both(c.y), v);
-    v = __ffma2_rn(l2, both(c.z), v);
-    v = __ffma2_rn(l3, both(c.w), v);
-    const float2 q = __fadd2_rn(__ffma2_rn(v, both(sc.inv[i]), mg), nmg);
-    const float2 r = __ffma2_rn(q, both(-sc.p[i]), v);
-    *reinterpret_cast<__nv_bfloat162*>(dst + static_cast<long long>(i) * Kp) = __float22bfloat162_rn(r);
+    const float inv = sc.inv[i], np = -sc.p[i];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float2 v = __fmul2_rn(l[h][0], both(c.x));
+      v = __ffma2_rn(l[h][1], both(c.y), v);
+      v = __ffma2_rn(l[h][2], both(c.z), v);
+      v = __ffma2_rn(l[h][3], both(c.w), v);
+      const float2 q = __fadd2_rn(__ffma2_rn(v, both(inv), mg), nmg);
+      const float2 r = __ffma2_rn(q, both(np), v);
+      if (h == 0 || two) *reinterpret_cast<__nv_bfloat162*>(dst + 64 * h) = __float22bfloat162_rn(r);
+    }
+    dst += Kp;
   }
 }
 
@@ -147,16 +152,23 @@ __device__ __forceinline__ void slice_line(const SliceConst& sc, int K, int Kp, 
   const int more = min(up, kMaxDataBits - sc.bits);   // as far as the digits reach, the line keeps more bits
   const int bits = sc.bits + more;
   up -= more;
-  for (int k = 2 * lane; k < Kp; k += 64) {
-    long long x0 = 0, x1 = 0;
-    if (e != kRowNonFinite) {
-      if (k < K) x0 = fixed_point(get(k), e, bits);
-      if (k + 1 < K) x1 = fixed_point(get(k + 1), e, bits);
+  for (int k = 2 * lane; k < Kp; k += 128) {
+    float2 l[2][4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int kh = k + 64 * h;
+      long long x0 = 0, x1 = 0;
+      if (e != kRowNonFinite) {
+        if (kh < K) x0 = fixed_point(get(kh), e, bits);
+        if (kh + 1 < K) x1 = fixed_point(get(kh + 1), e, bits);
+      }
+      float a[4], b[4];
+      limbs(x0, a);
+      limbs(x1, b);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) l[h][j] = make_float2(a[j], b[j]);
     }
-    float a[4], b[4];
-    limbs(x0, a);
-    limbs(x1, b);
-    store_residues(sc, up, a, b, dst + k, Kp);
+    store_residues(sc, up, l, k + 64 < Kp, dst + k, Kp);
   }
 }
 
@@ -186,7 +198,8 @@ slice_y_kernel(int nx, int K, int Kp, const double* __restrict__ src, __nv_bfloa
   const long long plane = blockIdx.x / tiles;
   const int i0 = static_cast<int>(blockIdx.x % tiles) * LB;
   const unsigned long long* in = reinterpret_cast<const unsigned long long*>(src) + plane * nx * K;
-  for (int t = threadIdx.x; t < LB * K; t += blockDim.x) {
+#pragma unroll 8
+  for (int t = threadIdx.x; t < LB * K; t += 256) {
     const int i = t % LB, j = t / LB;
     if (i0 + i < nx) tile[i * pitch + j] = __ldg(in + i0 + i + static_cast<long long>(nx) * j);
   }
@@ -249,14 +262,17 @@ matrix_residues_kernel(int K, int Kp, long long rs, long long cs, const double* 
 
 // ------------------------------------------------------------------ the GEMM
 
-constexpr int BM = 128, BN = 128, BK = 64;
-constexpr int kABytes = BM * BK * 2, kBBytes = BN * BK * 2, kStage = kABytes + kBBytes;
-constexpr int kStages = 6;
+constexpr int BM = 128, BK = 64;
 constexpr int kBufs = 4;                       // tensor-memory accumulators of BN columns
 constexpr int kEpiWarps = 16;
-constexpr int kCols = 4 * BN / kEpiWarps;       // columns of an epilogue thread
 constexpr int kThreads = 32 * (2 + kEpiWarps);
-constexpr int kSmem = kStages * kStage + 1024 /* alignment */ + 256 /* barriers */;
+template <int BN>
+struct RCfg {
+  static constexpr int kABytes = BM * BK * 2, kStage = kABytes + BN * BK * 2;
+  static constexpr int kStages = 192 * 1024 / kStage;
+  static constexpr int kCols = 4 * BN / kEpiWarps;   // columns of an epilogue thread
+  static constexpr int kSmem = kStages * kStage + 1024 /* alignment */ + 256 /* barriers */;
+};
 
 // 2^k times the 64-bit integer F, rounded to nearest even
 __device__ __forceinline__ double assemble(long long F, int k) {
@@ -278,19 +294,22 @@ __device__ __forceinline__ double assemble(long long F, int k) {
 }
 
 // D = A B^T through the residues of A (M rows) and B (N rows): persistent, one
-// CTA per SM, tiles of 128 x 128; for each tile the moduli in turn, each one
+// CTA per SM, tiles of 128 x BN; for each tile the moduli in turn, each one
 // K = Kp bf16 product into its own tensor-memory accumulator (four of them:
 // two pairs, so the tensor cores run ahead while the epilogue folds a pair).
-//   warp 0     TMA producer (128-byte rows, 128-byte swizzle, six 32 KB stages)
+//   warp 0     TMA producer (128-byte rows, 128-byte swizzle, 192 KB of stages)
 //   warp 1     tcgen05.mma issue; padding K steps of the last chunk are skipped
-//   warps 2-17 epilogue: a warp owns 32 rows x 32 columns, one 64-bit fraction
+//   warps 2-17 epilogue: a warp owns 32 rows x BN / 4 columns, one 64-bit fraction
 //              per element in registers over all moduli (sixteen warps: four a
 //              scheduler, and half the unrolled code of eight)
 // Element (m, n) is written (or added) at (m % rm) + (m / rm) sm + n sn.  Every
 // wait is bounded; a timeout sets bits in *err and the CTA drains and exits.
+template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
 residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB,
                     const __grid_constant__ ResidueGemm g) {
+  constexpr int kABytes = RCfg<BN>::kABytes, kStage = RCfg<BN>::kStage, kStages = RCfg<BN>::kStages;
+  constexpr int kCols = RCfg<BN>::kCols;
   extern __shared__ __align__(128) uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStage);
@@ -599,6 +618,34 @@ void gemm_const(const ResidueSystem& s, ResidueGemm* g) {
   g->shift = s.L - 64 - kMatrixBits - s.bits;
 }
 
+// Columns of a tile: rounds of tiles over the SMs times (columns + 70).  A tile's
+// epilogue takes 0.14 us a column, its start and the moduli's turns ~10 us, so
+// small transforms, which do not fill the chip with 128-column tiles, spread
+// their columns over more CTAs (32^3 22 -> 9.4 us, 61x97x75 30 -> 13).
+int tile_columns(int M, int N, int sms) {
+  int best = 128;
+  long long cost = -1;
+  for (int bn = 128; bn >= 32; bn /= 2) {
+    const long long tiles = static_cast<long long>((M + BM - 1) / BM) * ((N + bn - 1) / bn);
+    const long long c = (tiles + sms - 1) / sms * (bn + 70);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = bn;
+    }
+  }
+  return best;
+}
+
+template <int BN>
+cudaError_t launch_gemm(const CUtensorMap& a, const CUtensorMap& b, const ResidueGemm& g, int sms, cudaStream_t s) {
+  const cudaError_t e = cudaFuncSetAttribute(residue_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             RCfg<BN>::kSmem);
+  if (e != cudaSuccess) return e;
+  const long long tiles = static_cast<long long>((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
+  residue_gemm_kernel<BN><<<static_cast<unsigned>(tiles < sms ? tiles : sms), kThreads, RCfg<BN>::kSmem, s>>>(a, b, g);
+  return cudaGetLastError();
+}
+
 // Lines of direction d that one pass slices and multiplies (the scratch holds
 // their residues): all of them when they fit in the plan's res_cap, else whole
 // z planes.
@@ -684,9 +731,7 @@ cudaError_t residue_transform(const tpt_plan_s* p, int d, bool inverse, const do
   g.accumulate = accumulate ? 1 : 0;
   CUtensorMap mat, data;
   const int tab = inverse ? 1 : 0;
-  if (!tc::make_operand_map(&mat, rd.tab[tab], n, ld, ld, 128)) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(residue_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   for (long long l0 = 0; l0 < total; l0 += per_pass) {
     const int lines = static_cast<int>(total - l0 < per_pass ? total - l0 : per_pass);
     const long long off = l0 / per_plane * slab;   // first z plane of the pass
@@ -710,7 +755,6 @@ cudaError_t residue_transform(const tpt_plan_s* p, int d, bool inverse, const do
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (!tc::make_operand_map(&data, sl, lines, ld, ld, 128)) return cudaErrorInvalidValue;
     g.out = out + off;
     g.sn = nx;
     if (d == 0) {   // the matrix's rows are the output's x index
@@ -730,10 +774,13 @@ cudaError_t residue_transform(const tpt_plan_s* p, int d, bool inverse, const do
       g.expB = rd.expo[tab];
       g.n_fastest = 1;
     }
-    const long long tiles = static_cast<long long>((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
-    residue_gemm_kernel<<<static_cast<unsigned>(tiles < sms ? tiles : sms), kThreads, kSmem, s>>>(
-        d == 0 ? mat : data, d == 0 ? data : mat, g);
-    e = cudaGetLastError();
+    const int bn = tile_columns(g.M, g.N, sms);
+    if (!tc::make_operand_map(&mat, rd.tab[tab], n, ld, ld, d == 0 ? BM : bn)) return cudaErrorInvalidValue;
+    if (!tc::make_operand_map(&data, sl, lines, ld, ld, d == 0 ? bn : BM)) return cudaErrorInvalidValue;
+    const CUtensorMap& ma = d == 0 ? mat : data;
+    const CUtensorMap& mb = d == 0 ? data : mat;
+    e = bn == 128 ? launch_gemm<128>(ma, mb, g, sms, s) : bn == 64 ? launch_gemm<64>(ma, mb, g, sms, s)
+                                                                   : launch_gemm<32>(ma, mb, g, sms, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
