@@ -74,11 +74,19 @@ void free_plan(tpt_plan_s* p) {
 bool on_device(const tpt_plan_s* p) { return p && p->dev >= 0 && p->d_scal; }
 
 // Whether direction d of a float64 plan takes the tensor-core transform.  Per
-// transform (GB300, x; float64 FMA GEMM / residues): 16^3 21 / 30 us, 24^3 38 /
-// 31, 64^3 71 / 35, 256^3 6885 / 332, 512^3 109,690 / 3297: the FMA GEMM needs
-// 1.1 us per K step of a wave of tiles, the residue kernel ~25 us for its first
-// tile, so the line lies at 24 points whatever the other sizes.
-bool residue_pays(const tpt_plan_s* p, int d) { return p->n[d] >= 24 && p->n[d] <= tpt::kResidueMaxK; }
+// transform (GB300, x; float64 FMA GEMM / residues): 16^3 21 / 18 us, 16x128x128
+// 38 / 46, 24^3 37 / 19, 64^3 71 / 22, 256^3 6885 / 303, 512^3 109,690 / 3000: the
+// FMA GEMM needs 1.1 us per K step of a wave of tiles, the residue kernels ~17 us
+// for the smallest field, so the line lies at 24 points whatever the other sizes.
+// The float64 FFT / DCT of a uniform direction is bound by the same pipe and has
+// the same line against it up to 1024 points (per transform, FFT / residues: 32^3
+// 18 / 15 us, 64^3 32 / 22, 256^3 770 / 303, 512x512x64 840 / 380; solves of
+// 1024x64x64 2185 / 1494, 1024x1024x16 8815 / 6047), where the GEMM's work has
+// caught up: twice as much a point at 2048, the FFT's 10 % more.
+bool residue_pays(const tpt_plan_s* p, int d) {
+  if (p->xform[d] == TPT_XFORM_FFT) return p->n[d] >= 32 && p->n[d] <= 1024;
+  return p->n[d] >= 24 && p->n[d] <= tpt::kResidueMaxK;
+}
 
 int apply_transform(const tpt_plan_s* p, int d, bool inverse, const double* in, double* out,
                     bool accumulate, void* scratch, int* err, cudaStream_t s) {
@@ -87,9 +95,9 @@ int apply_transform(const tpt_plan_s* p, int d, bool inverse, const double* in, 
                                                         cudaMemcpyDeviceToDevice, s));
     return cuda_status(tpt::add_fp64(static_cast<long long>(tpt::npts(p)), in, out, s));
   }
-  if (p->xform[d] == TPT_XFORM_FFT) return cuda_status(tpt::fft_fp64(p, d, inverse, in, out, accumulate, s));
   if (p->res[d].ready && scratch)
     return cuda_status(tpt::residue_transform(p, d, inverse, in, out, accumulate, scratch, err, s));
+  if (p->xform[d] == TPT_XFORM_FFT) return cuda_status(tpt::fft_fp64(p, d, inverse, in, out, accumulate, s));
   const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
   const double* mat = inverse ? p->ddir[d].inv : p->ddir[d].fwd;
   if (d == 0) {
@@ -373,9 +381,10 @@ int create_plan_impl(const tpt_desc* desc, int cuda_device, tpt::BasisCache* cac
   }
   p->ozaki = desc->precision == TPT_PREC_FP64_OZAKI;
   for (int d = 0; d < 2 && p->precision == TPT_PREC_FP64; ++d) {   // residues of the transform matrices
-    if (p->dir[d].excluded() || p->xform[d] != TPT_XFORM_GEMM) continue;
-    if (p->ozaki && p->n[d] > tpt::kOzakiMaxK) return fail(TPT_ERR_UNSUPPORTED);
-    if (!p->ozaki && !residue_pays(p, d)) continue;
+    if (p->dir[d].excluded()) continue;
+    const bool gemm = p->xform[d] == TPT_XFORM_GEMM;
+    if (p->ozaki && gemm && p->n[d] > tpt::kOzakiMaxK) return fail(TPT_ERR_UNSUPPORTED);
+    if (!(p->ozaki && gemm) && !residue_pays(p, d)) continue;
     st = tpt::residue_setup(p, d);
     if (st != TPT_OK) return fail(st);
   }
@@ -694,9 +703,10 @@ int tpt_solve_host(tpt_plan p, const double* f_host, double* phi_host, double* f
 int tpt_transform(tpt_plan p, int dir, int inverse, const double* in, double* out, void* stream) {
   if (!on_device(p) || !in || !out || in == out || (dir != 0 && dir != 1)) return TPT_ERR_INVALID_ARG;
   DeviceGuard guard(p->dev);
-  if (p->ozaki && p->res[dir].ready && !p->res_scratch)   // this entry point's own scratch, kept by the plan
+  const bool residues = p->ozaki && p->xform[dir] == TPT_XFORM_GEMM && p->res[dir].ready;
+  if (residues && !p->res_scratch)   // this entry point's own scratch, kept by the plan
     TPT_CUDA(cudaMalloc(&p->res_scratch, tpt::residue_scratch_bytes(p)));
-  return apply_transform(p, dir, inverse != 0, in, out, false, p->res_scratch, nullptr,
+  return apply_transform(p, dir, inverse != 0, in, out, false, residues ? p->res_scratch : nullptr, nullptr,
                          static_cast<cudaStream_t>(stream));
 }
 

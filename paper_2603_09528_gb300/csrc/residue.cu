@@ -78,7 +78,8 @@ __device__ __forceinline__ long long fixed_point(unsigned long long bits, int e,
   return static_cast<long long>(bits) < 0 ? -X : X;
 }
 
-// X in balanced base-2^14 digits as floats: X = l0 + 2^14 l1 + 2^28 l2 + 2^42 l3.
+// X, |X| <= 2^57, in balanced base-2^14 digits as floats: X = l0 + 2^14 l1 + 2^28
+// l2 + 2^42 l3, |l3| <= 2^15.
 __device__ __forceinline__ void limbs(long long X, float (&l)[4]) {
   const unsigned long long Y = static_cast<unsigned long long>(X) + ((1ull << 13) + (1ull << 27) + (1ull << 41));
   const uint32_t lo = static_cast<uint32_t>(Y);
@@ -95,7 +96,7 @@ __device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
 
 // Residues of four values, two neighbouring pairs (limbs l[j] as pairs), for
 // every modulus: v = 2^k X mod p up to a multiple of p, from the digits times
-// 2^(k + 14 j) mod p (|v| <= 2^23, exact), r = v - p rint(v / p), stored as two
+// 2^(k + 14 j) mod p (|v| < 2^24, exact), r = v - p rint(v / p), stored as two
 // bf16 at dst + i * Kp for modulus i (and dst + 64 + i * Kp for the second pair
 // when `two`).  Paired float32 instructions, and the constants of a modulus
 // loaded once for both pairs; v / p is an odd multiple of 1/(2p) away from a tie
@@ -213,18 +214,51 @@ slice_y_kernel(int nx, int K, int Kp, const double* __restrict__ src, __nv_bfloa
   }
 }
 
-// Transform-matrix table: rows x K (element (r, k) at src[r rs + k cs]), row r
-// rounded to X_A = round(a 2^(54 - e) G / 2^64) and stored as the residues of
-// X_A y_i; one block per row.
+// Rows of a float64 transform matrix on the device: element (r, k) at
+// src[r rs + k cs].
+struct DenseRows {
+  const double* src;
+  long long rs, cs;
+  __device__ __forceinline__ double operator()(int r, int k) const { return src[r * rs + k * cs]; }
+};
+
+// Rows of the real DFT (kind 0, half-complex mode order) or DCT-II (kind 1) of n
+// points, a power of two, or of their exact inverses; tab holds cos(2 pi m / n)
+// and sin(2 pi m / n), m < n, or cos(2 pi m / 4n), m < 4n.
+struct FourierRows {
+  const double* tab;
+  int n, kind, inverse;
+  __device__ __forceinline__ double operator()(int r, int k) const {
+    const int mode = inverse ? k : r, point = inverse ? r : k;
+    double v;
+    if (kind == 1) {
+      v = tab[static_cast<int>(static_cast<long long>(mode) * (2 * point + 1) & (4 * n - 1))];
+    } else if (mode == 0) {
+      v = 1.0;
+    } else if (mode == n - 1) {
+      v = point % 2 ? -1.0 : 1.0;
+    } else {
+      const int m = static_cast<int>(static_cast<long long>((mode + 1) / 2) * point & (n - 1));
+      v = mode % 2 ? tab[m] : tab[n + m];
+    }
+    if (inverse) v *= (mode == 0 || (kind == 0 && mode == n - 1) ? 1.0 : 2.0) / n;
+    return v;
+  }
+};
+
+// Transform-matrix table: row r of K values rounded to X_A = round(a 2^(54 - e)
+// G / 2^64) and stored as the residues of X_A y_i; one block per row.
+template <typename Rows>
 __global__ void __launch_bounds__(256)
-matrix_residues_kernel(int K, int Kp, long long rs, long long cs, const double* __restrict__ src,
-                       __nv_bfloat16* __restrict__ dst, int* __restrict__ expo,
-                       const __grid_constant__ MatrixConst mc) {
+matrix_residues_kernel(int K, int Kp, const Rows rows, __nv_bfloat16* __restrict__ dst,
+                       int* __restrict__ expo, const __grid_constant__ MatrixConst mc) {
   __shared__ unsigned long long wmax[8];
   const long long r = blockIdx.x;
-  const unsigned long long* row = reinterpret_cast<const unsigned long long*>(src) + r * rs;
+  auto get = [&](int k) {
+    return static_cast<unsigned long long>(__double_as_longlong(rows(static_cast<int>(r), k)));
+  };
   unsigned long long m = 0;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) m = max(m, row[k * cs] & 0x7fffffffffffffffull);
+  for (int k = threadIdx.x; k < K; k += blockDim.x) m = max(m, get(k) & 0x7fffffffffffffffull);
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   if (threadIdx.x % 32 == 0) wmax[threadIdx.x / 32] = m;
   __syncthreads();
@@ -234,7 +268,7 @@ matrix_residues_kernel(int K, int Kp, long long rs, long long cs, const double* 
   for (int k = threadIdx.x; k < Kp; k += blockDim.x) {
     long long X = 0;
     if (k < K && e != kRowNonFinite) {
-      const unsigned long long bits = row[k * cs];
+      const unsigned long long bits = get(k);
       const int ex = static_cast<int>((bits >> 52) & 0x7ff);
       if (ex != 0) {
         const unsigned long long mant = (bits & ((1ull << 52) - 1)) | (1ull << 52);
@@ -675,20 +709,38 @@ int residue_setup(tpt_plan_s* p, int d) {
     mc.p[i] = rd.sys.p[i];
     mc.y[i] = rd.sys.y[i];
   }
+  void* tab_d = nullptr;   // angles of a Fourier-transformed direction
+  std::vector<double> angles;
+  if (p->xform[d] == TPT_XFORM_FFT) {
+    const long double pi2 = 6.283185307179586476925286766559005768L;
+    const int m = p->fft[d].kind == 1 ? 4 * n : n;
+    for (int k = 0; k < m; ++k) angles.push_back(static_cast<double>(std::cos(pi2 * k / m)));
+    if (p->fft[d].kind == 0)
+      for (int k = 0; k < n; ++k) angles.push_back(static_cast<double>(std::sin(pi2 * k / n)));
+    const int st = p->arena.upload(angles.data(), angles.size() * sizeof(double), &tab_d);
+    if (st != TPT_OK) return st;
+  }
   for (int inv = 0; inv < 2; ++inv) {
     void* t = nullptr;
     int st = p->arena.alloc(al256(tab) + static_cast<size_t>(n) * sizeof(int), &t);
     if (st != TPT_OK) return st;
     rd.tab[inv] = t;
     rd.expo[inv] = reinterpret_cast<int*>(static_cast<char*>(t) + al256(tab));
-    // rows = output modes: x transforms read A[r][k] = mat[r + n k], y
-    // transforms B[r][k] = mat[k + n r]
-    const double* src = inv ? p->ddir[d].inv : p->ddir[d].fwd;
     note_launch(1);
-    matrix_residues_kernel<<<n, 256, 0, p->arena.stream>>>(n, rd.kp, d == 0 ? 1 : n, d == 0 ? n : 1, src,
-                                                           static_cast<__nv_bfloat16*>(t), rd.expo[inv], mc);
+    if (tab_d) {
+      const FourierRows rows{static_cast<const double*>(tab_d), n, p->fft[d].kind, inv};
+      matrix_residues_kernel<<<n, 256, 0, p->arena.stream>>>(n, rd.kp, rows, static_cast<__nv_bfloat16*>(t),
+                                                             rd.expo[inv], mc);
+    } else {
+      // rows = output modes: x transforms read A[r][k] = mat[r + n k], y
+      // transforms B[r][k] = mat[k + n r]
+      const DenseRows rows{inv ? p->ddir[d].inv : p->ddir[d].fwd, d == 0 ? 1 : n, d == 0 ? n : 1};
+      matrix_residues_kernel<<<n, 256, 0, p->arena.stream>>>(n, rd.kp, rows, static_cast<__nv_bfloat16*>(t),
+                                                             rd.expo[inv], mc);
+    }
     if (cudaGetLastError() != cudaSuccess) return TPT_ERR_CUDA;
   }
+  if (tab_d && cudaStreamSynchronize(p->arena.stream) != cudaSuccess) return TPT_ERR_CUDA;   // angles dies here
   rd.ready = true;
   return TPT_OK;
 }

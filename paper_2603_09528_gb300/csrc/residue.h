@@ -10,7 +10,7 @@ namespace tpt {
 constexpr int kMaxModuli = 18;
 constexpr int kMatrixBits = 54;       // transform-matrix rows: |X| <= 2^54
 constexpr int kDataBits = 53;         // lines of the field: at least 53 bits of the line's maximum
-constexpr int kMaxDataBits = 55;      // (four 14-bit digits)
+constexpr int kMaxDataBits = 57;      // (14-bit digits, the top one of 15 bits and a sign)
 constexpr int kResidueMaxK = 2048;    // contraction length (shared-memory tile of the y slicing)
 constexpr int kOzakiMaxK = 576;       // contraction length a TPT_PREC_FP64_OZAKI plan accepts
 // Residues of one pass of a transform; larger fields go in passes of whole z

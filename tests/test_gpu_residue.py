@@ -151,3 +151,21 @@ def test_a_tight_server_budget_still_takes_a_float64_request(spare):
         assert (ph - ref.cpu()).abs().max().item() <= 1e-12 * ref.abs().max().item()
     finally:
         srv.close()
+
+
+# a uniform direction in a float64 solve takes its transform's matrix from 32 to
+# 1024 points, the FFT outside that range: both ends, periodic and Neumann, in
+# x and in y, against the oracle at the float64 bar
+@pytest.mark.parametrize("n,bcs", [((32, 24, 20), [(0, 0), (1, 1), (1, 1)]), ((1024, 16, 6), [(1, 1)] * 3),
+                                   ((24, 64, 20), [(1, 1), (0, 0), (2, 1)]), ((128, 128, 10), [(0, 0), (1, 1), (1, 1)]),
+                                   ((16, 2048, 3), [(1, 1), (1, 1), (2, 2)])])
+def test_uniform_directions_match_the_oracle(n, bcs):
+    dirs = [O.Direction(*O.uniform_grid(n[a]), bcs[a]) if a < 2 else O.Direction(*O.tanh_grid(n[a], 1.0, 1.5), bcs[a])
+            for a in range(3)]
+    f = S.uniform_rhs(n, 4)
+    if O.is_singular(dirs, 0.0):
+        f = S.remove_weighted_mean(f, [d.dxf for d in dirs])
+    plan = tpt.Plan(n, [d.dxf for d in dirs], [d.dxc for d in dirs], bcs, precision=L.TPT_PREC_FP64, max_refine=1)
+    phi, _ = plan.solve(tpt.field_to_device(f))
+    ref, _ = O.solve_tensor(f, dirs, 0.0, 1.0)
+    assert np.abs(tpt.field_to_host(phi, n) - ref).max() <= 1e-12 * np.abs(ref).max()
