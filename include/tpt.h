@@ -354,7 +354,7 @@ int tpt_plan_set_residual_kernel(tpt_plan plan, int variant);
  * 2.3 / Algorithm 1 step 5 in float32, by the partition method): 0
  * automatic, 1 one modal line per thread (segments of up to 32 rows, 16 per
  * line), 2 two neighbouring lines per thread (segments of up to 16 rows, 32
- * per line; Nz <= 512).  Automatic takes 2 for 192 < Nz <= 512.  The two
+ * per line; Nz <= 512).  Automatic takes 2 for 112 < Nz <= 512.  The two
  * partition the lines differently, so results agree to float32 rounding,
  * not to the bit.  For kernel tests and measurements.  INVALID_ARG for
  * another value; a no-op on float64 plans.                                 */

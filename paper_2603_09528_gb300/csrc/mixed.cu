@@ -502,9 +502,15 @@ thomas_tma_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_const
 // column reads are free of bank conflicts.  The second forward pass keeps its
 // values in registers for the back substitution instead of rewriting the
 // input tile.
-constexpr int kT2Slots = 32;                    // segment slots per line
-constexpr int kT2Pitch = kT2Slots + 1;          // row pitch of the reduced-system buffer
-constexpr int kT2SmemBudget = 209 * 1024;       // dynamic shared memory (17.1 KB static beside it)
+// A CTA of NT threads has NT / 16 segment slots per line: 32 (NT = 512, one CTA
+// per SM) above 256 rows, 16 (NT = 256, two per SM) up to 256, where the fixed
+// chain of barriers and the reduced system, not the sweeps, fill a tile's time
+// and two tiles in turn hide each other's (256^3 41.8 -> 30.4 us a launch,
+// 256x256x192 39.5 -> 25.9).
+constexpr int kT2Pitch = 33;                    // row pitch of the reduced-system buffer (32 lines)
+__host__ __device__ constexpr int t2_threads(int nz) { return nz <= 256 ? 256 : kThomasThreads; }
+// dynamic shared memory of a CTA (17.1 or 9.1 KB static beside it)
+__host__ __device__ constexpr int t2_smem_budget(int nt) { return (nt == kThomasThreads ? 209 : 103) * 1024; }
 
 // Elements i and i + 1 (i even) of an output tile in the T3 format.
 template <int FMT>
@@ -535,10 +541,12 @@ __device__ __forceinline__ float2 p_fma(float2 a, float2 b, float2 c) { return _
 __device__ __forceinline__ float2 p_dup(float v) { return make_float2(v, v); }
 
 // Row of thomas2_kernel's shared table with each coefficient duplicated for
-// the thread's two lines: -beta a_k, beta b_k, beta c_k and the shift factor.
+// the thread's two lines: -beta a_k, beta b_k, beta c_k.  A padding row has
+// a = c = 0 and a diagonal that no modal shift cancels.
 struct RowCoef2 {
-  float2 na, b, c, m;
+  float2 na, b, c;
 };
+constexpr float kT2PadDiag = 1e30f;
 
 // The data of one instance for thomas2_kernel: tensor maps of T2 (in) and
 // T3 (out planes), its stage geometry, sizes, tables and flags.  A grouped
@@ -576,18 +584,20 @@ struct ThomasJob {
 template <int FMT>
 __device__ void null_line_block(const ThomasJob& J, void* o0, void* o1, double* scr) {
   constexpr int TLT = 32;
-  const int k = threadIdx.x, lane = k % 32, warp = k / 32, nw = blockDim.x / 32;
   const int nz = J.nz;
+  const int k = threadIdx.x, lane = k % 32, warp = k / 32, nw = (nz + 31) / 32;   // warps that hold rows
   const bool row = k < nz, elim = k < nz - 1;
   const double f = row ? static_cast<double>(J.t2[static_cast<long long>(k) * J.nstride]) : 0.0;
   const double dzk = row ? J.ndz[k] : 0.0;
   // block sums, the same in every thread
   auto sum2 = [&](double a, double b, double& sa, double& sb) {
-    a = warp_sum_d(a);
-    b = warp_sum_d(b);
-    if (lane == 0) {
-      scr[warp] = a;
-      scr[32 + warp] = b;
+    if (warp < nw) {
+      a = warp_sum_d(a);
+      b = warp_sum_d(b);
+      if (lane == 0) {
+        scr[warp] = a;
+        scr[32 + warp] = b;
+      }
     }
     __syncthreads();
     sa = 0.0;
@@ -602,7 +612,7 @@ __device__ void null_line_block(const ThomasJob& J, void* o0, void* o1, double* 
   // returns this row's composed map applied to the value entering the line (0)
   auto scan = [&](double A, double B, bool up) -> double {
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
+    for (int d = 1; d < 32 && warp < nw; d <<= 1) {
       const double Ap = up ? __shfl_up_sync(0xffffffffu, A, d) : __shfl_down_sync(0xffffffffu, A, d);
       const double Bp = up ? __shfl_up_sync(0xffffffffu, B, d) : __shfl_down_sync(0xffffffffu, B, d);
       if (up ? lane >= d : lane + d < 32) {
@@ -610,7 +620,7 @@ __device__ void null_line_block(const ThomasJob& J, void* o0, void* o1, double* 
         A *= Ap;
       }
     }
-    if (lane == (up ? 31 : 0)) {         // the map of the whole warp
+    if (warp < nw && lane == (up ? 31 : 0)) {   // the map of the whole warp
       scr[warp] = A;
       scr[32 + warp] = B;
     }
@@ -639,13 +649,14 @@ __device__ void null_line_block(const ThomasJob& J, void* o0, void* o1, double* 
 
 // lg: the shared-memory layout of the launch (stage count and the largest
 // stage, output tile and row table over its instances).
-template <int FMT, int M, int MULTI>
-__global__ void __launch_bounds__(kThomasThreads, 1)
+template <int FMT, int M, int MULTI, int NT>
+__global__ void __launch_bounds__(NT, kThomasThreads / NT)
 thomas2_kernel(const __grid_constant__ ThomasJob job0, ThomasGeom lg, int* next_tile, int total_tiles,
                const ThomasJob* __restrict__ jobs, int njobs) {
   if (!MULTI && job0.skip && *job0.skip) return;   // the refinement has stopped
   using O = T3Fmt<FMT>;
   constexpr int TLT = 32;
+  constexpr int SLOTS = NT / 16;         // segment slots per line
   static_assert(M >= 2 && M <= 16, "segments of 2 to 16 rows");
   extern __shared__ __align__(128) uint8_t dsm_raw[];
   uint8_t* dsm = dsm_raw + ((1024u - (ptx::smem_u32(dsm_raw) & 1023u)) & 1023u);
@@ -656,7 +667,7 @@ thomas2_kernel(const __grid_constant__ ThomasJob job0, ThomasGeom lg, int* next_
   // the interface row of segment s (A, B, C, D; D overwritten by the interface
   // value y_s) in slot s + 1.  The thread of segment s is the only reader of
   // slot s + 1 before it writes it, so no barrier separates the two uses.
-  __shared__ __align__(16) float X[4][(kT2Slots + 1) * kT2Pitch];
+  __shared__ __align__(16) float X[4][(SLOTS + 1) * kT2Pitch];
   __shared__ __align__(8) uint64_t full[kThomasMaxStages];
   __shared__ int tile_of[kThomasMaxStages];
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
@@ -751,14 +762,13 @@ thomas2_kernel(const __grid_constant__ ThomasJob job0, ThomasGeom lg, int* next_
     if (jid != cur) {                    // this instance's beta-scaled z rows into the table
       if (cur >= 0) __syncthreads();     // the previous tile is done with them
       for (int k = tid; k < J.geo.sr; k += blockDim.x) {
-        float a = 0.0f, b = 1.0f, c = 0.0f, m = 0.0f;   // padding rows: identity
+        float a = 0.0f, b = kT2PadDiag, c = 0.0f;   // padding rows
         if (k < J.nz) {
           a = k > 0 ? J.beta * J.az[k] : 0.0f;
           b = J.beta * J.bz[k];
           c = k < J.nz - 1 ? J.beta * J.cz[k] : 0.0f;
-          m = 1.0f;
         }
-        coef[k] = {p_dup(-a), p_dup(b), p_dup(c), p_dup(m)};
+        coef[k] = {p_dup(-a), p_dup(b), p_dup(c)};
       }
       cur = jid;
       __syncthreads();
@@ -797,7 +807,7 @@ thomas2_kernel(const __grid_constant__ ThomasJob job0, ThomasGeom lg, int* next_
       for (int t = 0; t < M - 1; ++t) {
         const RowCoef2 rc = coef[s0 + t];
         const float2 d = *reinterpret_cast<const float2*>(in + (s0 + t) * TLT + l0);
-        const float2 m = p_fma(rc.na, cprev, p_fma(rc.m, sh, rc.b));
+        const float2 m = p_fma(rc.na, cprev, p_add(sh, rc.b));
         const float2 iv = make_float2(__fdividef(1.0f, m.x), __fdividef(1.0f, m.y));
         const float2 cp = p_mul(rc.c, iv);
         const float2 g = p_mul(p_fma(rc.na, gprev, d), iv);
@@ -838,15 +848,15 @@ thomas2_kernel(const __grid_constant__ ThomasJob job0, ThomasGeom lg, int* next_
     if (active) {
       const int k = s0 + M - 1;
       const RowCoef2 rc = coef[k];
-      const float a = -rc.na.x, b = rc.b.x, c = rc.c.x, mf = rc.m.x;
+      const float a = -rc.na.x, b = rc.b.x, c = rc.c.x;
       const float2 d = *reinterpret_cast<const float2*>(in + k * TLT + l0);
       const float cpr[2] = {cprev.x, cprev.y}, gpr[2] = {gprev.x, gprev.y}, upr[2] = {uprev.x, uprev.y};
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         ra[j] = a * upr[j];
-        rb[j] = fmaf(-a, cpr[j], fmaf(mf, shift[j], b));
+        rb[j] = fmaf(-a, cpr[j], shift[j] + b);
         rd[j] = fmaf(-a, gpr[j], j ? d.y : d.x);
-        if (s + 1 < kT2Slots) {
+        if (s + 1 < SLOTS) {
           const int on = xo + kT2Pitch + j;
           rb[j] = fmaf(c, X[1][on], rb[j]);
           rcc[j] = c * X[2][on];
@@ -862,22 +872,24 @@ thomas2_kernel(const __grid_constant__ ThomasJob job0, ThomasGeom lg, int* next_
       X[3][xo + kT2Pitch + j] = rd[j];
     }
     __syncthreads();
-    // reduced systems: warp w takes lines 2w (lanes 0-15) and 2w + 1 (lanes
-    // 16-31); lane q of a half holds interface rows 2q and 2q + 1, scaled to a
-    // unit diagonal (a x_{r-1} + x_r + c x_{r+1} = d).  One odd-even step
-    // eliminates the odd rows from the even ones (the odd row below comes from
-    // lane q - 1), parallel cyclic reduction solves the 16 even rows, and each
-    // odd row is then recovered from its two even neighbours.  Eliminating both
+    // reduced systems: QL = SLOTS / 2 neighbouring lanes take a line (a warp of
+    // 32-slot CTAs the lines 2w and 2w + 1); lane q of them holds interface rows
+    // 2q and 2q + 1, scaled to a unit diagonal (a x_{r-1} + x_r + c x_{r+1} =
+    // d).  One odd-even step eliminates the odd rows from the even ones (the
+    // odd row below comes from lane q - 1), parallel cyclic reduction solves the
+    // QL even rows, and each odd row is then recovered from its two even
+    // neighbours.  Eliminating both
     // neighbours at distance d gives
     //   a' = -a a_{r-d},  c' = -c c_{r+d},  b' = 1 - a c_{r-d} - c a_{r+d},
     //   d' = d - a d_{r-d} - c d_{r+d},  then the row is scaled by 1 / b'.
-    // Row 0 has a = 0 and row 31 has c = 0, and that stays so for every row
+    // Row 0 has a = 0 and the last row c = 0, and that stays so for every row
     // whose neighbour at distance d lies outside (its a or c is a product
     // with such a zero), so the shuffles that fall off an end of a half (which
     // return the lane's own values) are always multiplied by zero.
     {
-      const int q = lane % 16;
-      const int col = 2 * warp + lane / 16;
+      constexpr int QL = SLOTS / 2;
+      const int q = lane % QL;
+      const int col = tid / QL;
       const int ie = (2 * q + 1) * kT2Pitch + col, io = ie + kT2Pitch;   // rows 2q, 2q + 1
       float ae, ce, de, ao, co, dO;
       {
@@ -891,8 +903,8 @@ thomas2_kernel(const __grid_constant__ ThomasJob job0, ThomasGeom lg, int* next_
       }
       {
         // the odd row 2q - 1 (lane q - 1) and 2q + 1 (this lane)
-        const float am = __shfl_up_sync(0xffffffffu, ao, 1, 16), cm = __shfl_up_sync(0xffffffffu, co, 1, 16);
-        const float dm = __shfl_up_sync(0xffffffffu, dO, 1, 16);
+        const float am = __shfl_up_sync(0xffffffffu, ao, 1, QL), cm = __shfl_up_sync(0xffffffffu, co, 1, QL);
+        const float dm = __shfl_up_sync(0xffffffffu, dO, 1, QL);
         const float b = fmaf(-ae, cm, fmaf(-ce, ao, 1.0f));
         const float d = fmaf(-ae, dm, fmaf(-ce, dO, de));
         const float ib = __fdividef(1.0f, b);
@@ -901,11 +913,11 @@ thomas2_kernel(const __grid_constant__ ThomasJob job0, ThomasGeom lg, int* next_
         de = d * ib;
       }
 #pragma unroll
-      for (int dlt = 1; dlt < 16; dlt <<= 1) {
-        const float Am = __shfl_up_sync(0xffffffffu, ae, dlt, 16), Cm = __shfl_up_sync(0xffffffffu, ce, dlt, 16);
-        const float Dm = __shfl_up_sync(0xffffffffu, de, dlt, 16);
-        const float Ap = __shfl_down_sync(0xffffffffu, ae, dlt, 16), Cp = __shfl_down_sync(0xffffffffu, ce, dlt, 16);
-        const float Dp = __shfl_down_sync(0xffffffffu, de, dlt, 16);
+      for (int dlt = 1; dlt < QL; dlt <<= 1) {
+        const float Am = __shfl_up_sync(0xffffffffu, ae, dlt, QL), Cm = __shfl_up_sync(0xffffffffu, ce, dlt, QL);
+        const float Dm = __shfl_up_sync(0xffffffffu, de, dlt, QL);
+        const float Ap = __shfl_down_sync(0xffffffffu, ae, dlt, QL), Cp = __shfl_down_sync(0xffffffffu, ce, dlt, QL);
+        const float Dp = __shfl_down_sync(0xffffffffu, de, dlt, QL);
         const float b = fmaf(-ae, Cm, fmaf(-ce, Ap, 1.0f));
         const float d = fmaf(-ae, Dm, fmaf(-ce, Dp, de));
         const float ib = __fdividef(1.0f, b);
@@ -914,7 +926,7 @@ thomas2_kernel(const __grid_constant__ ThomasJob job0, ThomasGeom lg, int* next_
         de = d * ib;
       }
       // de = x_{2q}; the odd row from x_{2q} and x_{2q+2} (lane q + 1)
-      const float xn = __shfl_down_sync(0xffffffffu, de, 1, 16);
+      const float xn = __shfl_down_sync(0xffffffffu, de, 1, QL);
       X[3][ie] = de;
       X[3][io] = fmaf(-ao, de, fmaf(-co, xn, dO));
     }
@@ -2351,14 +2363,14 @@ cudaError_t launch_thomas_m(const tpt_plan_s* p, const MixedWork& w, cudaStream_
 }
 
 // Segment length of thomas2_kernel for Nz rows: the candidate M <= 16 whose
-// ceil(Nz / M) <= 32 segments leave the fewest padding rows (ties: the
-// smaller M); 0 when Nz > 512.
+// ceil(Nz / M) segments fit the CTA's slots and leave the fewest padding rows
+// (ties: the smaller M); 0 when Nz > 512.
 int thomas2_m(int nz) {
   static const int cand[] = {4, 8, 12, 16};
   int best = 0, pad = 1 << 30;
   for (int m : cand) {
     const int nseg = (nz + m - 1) / m;
-    if (nseg > kT2Slots) continue;
+    if (nseg > t2_threads(nz) / 16) continue;
     if (nseg * m - nz < pad) {
       pad = nseg * m - nz;
       best = m;
@@ -2390,8 +2402,9 @@ bool thomas2_job(const tpt_plan_s* p, const MixedWork& w, int first, ThomasJob* 
   const int nz = p->n[2];
   if (lines + TLT > 0x7fffffffLL) return false;   // int line indices and TMA coordinates
   std::memset(J, 0, sizeof(*J));
-  if (!thomas_geom(nz, M, TLT, O::NPL, O::EB, &J->geo, kT2SmemBudget, static_cast<int>(sizeof(RowCoef2))) ||
-      J->geo.nseg > kT2Slots)
+  if (!thomas_geom(nz, M, TLT, O::NPL, O::EB, &J->geo, t2_smem_budget(t2_threads(nz)),
+                   static_cast<int>(sizeof(RowCoef2))) ||
+      J->geo.nseg > t2_threads(nz) / 16)
     return false;
   if (!tc::make_plain_map(&J->map_in, w.B[0], 4, lines, nz, lines * 4, TLT, J->geo.rb)) return false;
   if (!tc::make_plain_map(&J->map_o0, w.A[0], O::EB, lines, nz, lines * O::EB, TLT, J->geo.rb)) return false;
@@ -2434,7 +2447,7 @@ size_t thomas2_smem(const ThomasGeom& g) {
          static_cast<size_t>(g.out_bytes);
 }
 
-template <int FMT, int M>
+template <int FMT, int M, int NT>
 cudaError_t launch_thomas2_m(const tpt_plan_s* p, const MixedWork& w, cudaStream_t s) {
   ThomasJob J;
   if (!thomas2_job<FMT, M>(p, w, 0, &J)) return cudaErrorInvalidValue;
@@ -2443,30 +2456,35 @@ cudaError_t launch_thomas2_m(const tpt_plan_s* p, const MixedWork& w, cudaStream
   cudaError_t e = cudaMemsetAsync(next_tile, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   const size_t smem = thomas2_smem(J.geo);
-  auto kern = thomas2_kernel<FMT, M, 0>;
+  auto kern = thomas2_kernel<FMT, M, 0, NT>;
   // a fixed cap (see launch_thomas_m)
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kT2SmemBudget);
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, t2_smem_budget(NT));
   if (e != cudaSuccess) return e;
-  if (smem > static_cast<size_t>(kT2SmemBudget)) return cudaErrorInvalidConfiguration;
-  int sms = 152;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->dev);
-  const int grid = J.ntiles < sms ? J.ntiles : sms;
+  if (smem > static_cast<size_t>(t2_smem_budget(NT))) return cudaErrorInvalidConfiguration;
+  const int slots = sm_count(p->dev) * (kThomasThreads / NT);
+  const int grid = J.ntiles < slots ? J.ntiles : slots;
   note_launch(1);
-  kern<<<static_cast<unsigned>(grid), kThomasThreads, smem, s>>>(J, J.geo, next_tile, J.ntiles, nullptr, 0);
+  kern<<<static_cast<unsigned>(grid), NT, smem, s>>>(J, J.geo, next_tile, J.ntiles, nullptr, 0);
   return cudaGetLastError();
 }
 
+template <int FMT, int M>
+cudaError_t launch_thomas2_nt(const tpt_plan_s* p, const MixedWork& w, cudaStream_t s) {
+  return t2_threads(p->n[2]) == 256 ? launch_thomas2_m<FMT, M, 256>(p, w, s)
+                                    : launch_thomas2_m<FMT, M, kThomasThreads>(p, w, s);
+}
+
 // Thomas kernel for a plan: 1 one line per thread (thomas_tma_kernel), 2 two
-// lines per thread (thomas2_kernel); `variant` 0 picks the two-line kernel
-// where its segments are at least 8 rows long (Nz from 193 to 512; 256^3 41.8
-// against 46.1 us).  Below, its tiles are as fast (64^3 5.9 against 6.8 us) but
-// on a singular problem its block-wide null line takes 19 us (64^3 24.6 in all)
-// where the one-warp kernel beside thomas_tma_kernel takes 10.
+// lines per thread (thomas2_kernel); `variant` 0 picks the two-line kernel above
+// 112 rows (per launch, one-line / two-line: 256^3 45.7 / 30.4 us, 150x277x133
+// 26.1 / 19.0, 128^3 11.2 / 10.1; 192x192x96 15.4 / 16.0, 300x200x40 15.4 /
+// 18.3).  Up to there a singular problem also keeps its null line off the
+// block-wide scans of the two-line kernel.
 int thomas_variant(int nz, int variant) {
   if (variant == 1) return 1;
   const int m2 = thomas2_m(nz);
   if (variant == 2) return m2 > 0 ? 2 : 1;
-  return (m2 >= 8 && nz > 192) ? 2 : 1;
+  return (m2 > 0 && nz > 112) ? 2 : 1;
 }
 
 // Step 2.3: T3 = modal Thomas solve of T2 (float32, in B) into A.  The null
@@ -2496,10 +2514,10 @@ cudaError_t launch_thomas(const tpt_plan_s* p, const MixedWork& w, cudaStream_t 
   const ThomasShape sh = thomas_shape(nz, static_cast<long long>(m.ldy) * p->n[0], sm_count(p->dev));
   if (two) {
     switch (thomas2_m(nz)) {
-      case 4: e = launch_thomas2_m<FMT, 4>(p, w, s); break;
-      case 8: e = launch_thomas2_m<FMT, 8>(p, w, s); break;
-      case 12: e = launch_thomas2_m<FMT, 12>(p, w, s); break;
-      case 16: e = launch_thomas2_m<FMT, 16>(p, w, s); break;
+      case 4: e = launch_thomas2_nt<FMT, 4>(p, w, s); break;
+      case 8: e = launch_thomas2_nt<FMT, 8>(p, w, s); break;
+      case 12: e = launch_thomas2_nt<FMT, 12>(p, w, s); break;
+      case 16: e = launch_thomas2_nt<FMT, 16>(p, w, s); break;
       default: break;
     }
   } else if (sh.nt == 128) {
@@ -3441,7 +3459,7 @@ struct GroupSolve {
   tc::GemmJob* d_gemm[5] = {};
   long long gemm_units[5] = {};
   bool gemm_tma[5] = {};
-  struct TGroup { int m = 0; int njobs = 0; int tiles = 0; ThomasGeom lg{}; ThomasJob* d = nullptr; };
+  struct TGroup { int m = 0, nt = 0; int njobs = 0; int tiles = 0; ThomasGeom lg{}; ThomasJob* d = nullptr; };
   std::vector<TGroup> tg;
   struct RGroup { int code = 0; int njobs = 0; int blocks = 0; ResJob* d = nullptr; };
   std::vector<RGroup> rg;
@@ -3483,27 +3501,34 @@ cudaError_t launch_res_code(const GroupSolve::RGroup& r, cudaStream_t s) {
   }
 }
 
-template <int M>
+template <int M, int NT>
 cudaError_t launch_thomas_group(const GroupSolve::TGroup& t, int* counter, int dev, cudaStream_t s) {
-  auto kern = thomas2_kernel<kFmtSplit, M, 1>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kT2SmemBudget);
+  auto kern = thomas2_kernel<kFmtSplit, M, 1, NT>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, t2_smem_budget(NT));
   if (e != cudaSuccess) return e;
-  int sms = 152;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int grid = t.tiles < sms ? t.tiles : sms;
+  const int slots = sm_count(dev) * (kThomasThreads / NT);
+  const int grid = t.tiles < slots ? t.tiles : slots;
   ThomasJob none;
   std::memset(&none, 0, sizeof(none));
   note_launch(1);
-  kern<<<grid, kThomasThreads, thomas2_smem(t.lg), s>>>(none, t.lg, counter, t.tiles, t.d, t.njobs);
+  kern<<<grid, NT, thomas2_smem(t.lg), s>>>(none, t.lg, counter, t.tiles, t.d, t.njobs);
   return cudaGetLastError();
 }
 
 cudaError_t launch_thomas_m_group(const GroupSolve::TGroup& t, int* counter, int dev, cudaStream_t s) {
   switch (t.m) {
-    case 4: return launch_thomas_group<4>(t, counter, dev, s);
-    case 8: return launch_thomas_group<8>(t, counter, dev, s);
-    case 12: return launch_thomas_group<12>(t, counter, dev, s);
-    case 16: return launch_thomas_group<16>(t, counter, dev, s);
+    case 4:
+      return t.nt == 256 ? launch_thomas_group<4, 256>(t, counter, dev, s)
+                         : launch_thomas_group<4, kThomasThreads>(t, counter, dev, s);
+    case 8:
+      return t.nt == 256 ? launch_thomas_group<8, 256>(t, counter, dev, s)
+                         : launch_thomas_group<8, kThomasThreads>(t, counter, dev, s);
+    case 12:
+      return t.nt == 256 ? launch_thomas_group<12, 256>(t, counter, dev, s)
+                         : launch_thomas_group<12, kThomasThreads>(t, counter, dev, s);
+    case 16:
+      return t.nt == 256 ? launch_thomas_group<16, 256>(t, counter, dev, s)
+                         : launch_thomas_group<16, kThomasThreads>(t, counter, dev, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -3555,12 +3580,13 @@ void group_destroy(GroupSolve* g) {
 }
 
 size_t group_table_bytes(const GroupSolve* g) {
-  // an upper bound of group_prepare's layout: at most 4 Thomas groups (one per
-  // segment length) and 5 residual variants, each rounded up to 256 bytes
+  // an upper bound of group_prepare's layout: at most 8 Thomas groups (one per
+  // segment length and CTA size) and 5 residual variants, each rounded up to
+  // 256 bytes
   const size_t n = g ? static_cast<size_t>(g->n) : 0;
   return align256(sizeof(InstJob) * n) + 5 * align256(sizeof(tc::GemmJob) * n) + sizeof(ThomasJob) * n +
-         4 * 256 + sizeof(ResJob) * n + 5 * 256 + align256(sizeof(int) * std::max<size_t>(1, n)) +
-         align256(sizeof(int) * 4 * 64);
+         8 * 256 + sizeof(ResJob) * n + 5 * 256 + align256(sizeof(int) * std::max<size_t>(1, n)) +
+         align256(sizeof(int) * 8 * 64);
 }
 
 void group_set_memory(GroupSolve* g, void* mem, size_t bytes) {
@@ -3672,10 +3698,12 @@ int group_prepare(GroupSolve* g, const double* const* f, double* const* phi, voi
     const tpt_plan_s* p = g->plans[i];
     const int m = thomas2_m(p->n[2]);
     size_t k = 0;
-    while (k < tg.size() && tg[k].m != m) ++k;
+    const int nt = t2_threads(p->n[2]);
+    while (k < tg.size() && (tg[k].m != m || tg[k].nt != nt)) ++k;
     if (k == tg.size()) {
       tg.push_back(GroupSolve::TGroup{});
       tg[k].m = m;
+      tg[k].nt = nt;
       tg[k].lg.stages = 2;
       tj.emplace_back();
     }
@@ -3710,7 +3738,7 @@ int group_prepare(GroupSolve* g, const double* const* f, double* const* phi, voi
     rj[r].push_back(R);
   }
   for (auto& t : tg) {   // as many stages as the budget holds beside the output tile and rows
-    const long long room = static_cast<long long>(kT2SmemBudget) - 1024 - t.lg.coef_bytes - t.lg.out_bytes;
+    const long long room = static_cast<long long>(t2_smem_budget(t.nt)) - 1024 - t.lg.coef_bytes - t.lg.out_bytes;
     t.lg.stages = static_cast<int>(std::min<long long>(kThomasMaxStages, room / std::max(1, t.lg.in_bytes)));
     if (t.lg.stages < 2) return TPT_ERR_UNSUPPORTED;
     t.njobs = 0;
