@@ -288,6 +288,9 @@ thomas_tma_kernel(const __grid_constant__ CUtensorMap map_in, const __grid_const
     ++issued;
     if (tile >= ntiles) {                // none left: complete the phase without data
       exhausted = true;
+      // every CTA claims past the end once: the last of them leaves the counter
+      // at zero for the next launch
+      if (tile == ntiles + static_cast<int>(gridDim.x) - 1) *next_tile = 0;
       tile_of[st] = -1;
       ptx::mbar_arrive(bar);
       return;
@@ -712,6 +715,7 @@ thomas2_kernel(const __grid_constant__ ThomasJob job0, ThomasGeom lg, int* next_
     ++issued;
     if (tile >= total_tiles) {
       exhausted = true;
+      if (tile == total_tiles + static_cast<int>(gridDim.x) - 1) *next_tile = 0;   // as in thomas_tma_kernel
       tile_of[st] = -1;
       ptx::mbar_arrive(bar);
       return;
@@ -1077,6 +1081,62 @@ struct BRows {
   const float *ah, *al, *ch, *cl, *wh, *wl;
 };
 
+// Device-side stopping test of the adaptive refinement (Sec. 4.1), run after
+// each correction's residual: scal[8] (as int) becomes 1 once ||r|| / ||f||
+// <= rtol (norm of f projected to compatible form for a singular problem, as
+// proj_norm2 computes it), 2 for a non-finite norm and 3 after a timed-out
+// wait, and from then on every kernel of a later correction returns at entry;
+// scal[8] + 4 bytes counts the corrections applied; scal[11], scal[12] keep
+// the last r^2 and f^2 sums; otherwise r's sum is cleared for the next residual.
+__device__ __forceinline__ void converge_body(double* scal, double npts, double vol, int singular, double rtol) {
+  int* flags = reinterpret_cast<int*>(scal + 8);
+  if (flags[0]) return;
+  flags[1] += 1;
+  scal[2] = 0.0;   // the gauge sum of an output that may follow
+  const double r2 = __ldcg(scal + 1);
+  double fn2 = scal[5];
+  if (singular) {
+    const double c = scal[7] / vol;
+    fn2 = scal[5] - 2.0 * c * scal[6] + npts * c * c;
+  }
+  scal[11] = r2;
+  scal[12] = fn2;
+  if (*reinterpret_cast<volatile const int*>(scal + 15)) {
+    flags[0] = 3;
+    return;
+  }
+  if (!isfinite(r2) || !isfinite(fn2)) {
+    flags[0] = 2;
+    return;
+  }
+  const double rel = fn2 > 0.0 ? sqrt(r2 / fn2) : sqrt(r2);
+  if (rel <= rtol) {
+    flags[0] = 1;
+    return;
+  }
+  scal[1] = 0.0;
+  scal[2] = 0.0;
+}
+
+// The stopping test as the last act of a residual: the warp that arrives last at
+// the counter (scal[13]) has every warp's share of sum r^2 before it.  scal null:
+// no test.
+struct Conv {
+  double* scal;
+  double npts, vol, rtol;
+  int singular;
+  unsigned total;   // warps that arrive
+};
+__device__ __forceinline__ void arrive_converge(const Conv& c) {
+  if (!c.scal) return;
+  __threadfence();
+  unsigned* count = reinterpret_cast<unsigned*>(c.scal + 13);
+  if (atomicAdd(count, 1u) != c.total - 1) return;
+  *count = 0;
+  __threadfence();
+  converge_body(c.scal, c.npts, c.vol, c.singular, c.rtol);
+}
+
 // r = (f - fshift) - alpha phi - beta L phi in float-pair arithmetic, written
 // to R (operand format, rows of ldx), and sum r^2 -> sums[0]; fshift (the
 // volume-weighted mean of f) only for a singular problem (SING).  Block (32, 4)
@@ -1090,7 +1150,7 @@ residual_df_kernel(int nx, int ny, int nz, int ldx, int kseg, const float* __res
                    const float* __restrict__ fl, const float* __restrict__ ph,
                    const float* __restrict__ pl, void* r0, void* r1, BRows RX, BRows RY, BRows RZ,
                    float alpha_h, float alpha_l, const double* __restrict__ fsums, double inv_vol,
-                   double* sums, const int* skip) {
+                   double* sums, const int* skip, const Conv conv) {
   if (skip && *skip) return;   // the refinement has stopped
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1155,7 +1215,10 @@ residual_df_kernel(int nx, int ny, int nz, int ldx, int kseg, const float* __res
     }
   }
   double s2 = warp_sum_d(static_cast<double>(acc2));
-  if ((threadIdx.x + blockDim.x * threadIdx.y) % 32 == 0) atomicAdd(&sums[0], s2);
+  if ((threadIdx.x + blockDim.x * threadIdx.y) % 32 == 0) {
+    atomicAdd(&sums[0], s2);
+    arrive_converge(conv);
+  }
 }
 
 // exact difference x - y of float pairs (hi parts by TwoSum, lo parts added)
@@ -1310,7 +1373,7 @@ residual_df2_kernel(int nx, int ny, int nz, int ldx, int kseg, const float* __re
                     const float* __restrict__ fl, const float* __restrict__ ph,
                     const float* __restrict__ pl, void* r0, void* r1, BRows RX, BRows RY, BRows RZ,
                     float alpha_h, float alpha_l, const double* __restrict__ fsums, double inv_vol,
-                    double* sums, const int* skip) {
+                    double* sums, const int* skip, const Conv conv) {
   if (skip && *skip) return;   // the refinement has stopped
   const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x);   // points i and i + 1
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
@@ -1387,7 +1450,10 @@ residual_df2_kernel(int nx, int ny, int nz, int ldx, int kseg, const float* __re
     }
   }
   double s2 = warp_sum_d(static_cast<double>(acc2));
-  if ((threadIdx.x + blockDim.x * threadIdx.y) % 32 == 0) atomicAdd(&sums[0], s2);
+  if ((threadIdx.x + blockDim.x * threadIdx.y) % 32 == 0) {
+    atomicAdd(&sums[0], s2);
+    arrive_converge(conv);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1560,6 +1626,7 @@ struct ResJob {
   int* err;
   const int* skip;
   int first, tx, ty, tz;   // first block and tile counts of the instance
+  Conv conv;
   int kseg;                // planes of a block
 };
 
@@ -1728,7 +1795,10 @@ __device__ __forceinline__ void residual_tma_body(const ResJob& J, int bx, int b
     }
   }
   double s2 = warp_sum_d(static_cast<double>(acc2));
-  if (lane == 0) atomicAdd(&sums[0], s2);
+  if (lane == 0) {
+    atomicAdd(&sums[0], s2);
+    arrive_converge(J.conv);
+  }
 }
 
 template <int FMT, int HAS_ALPHA, int WX, int WY, int WZ, int SING>
@@ -1805,7 +1875,9 @@ wsum_df_kernel(int nx, int ny, int nz, const float* __restrict__ h, const float*
 // pair is converted with integer operations and one float64 add.
 __global__ void __launch_bounds__(256)
 df_to_f64_kernel(long long n, const float* __restrict__ h, const float* __restrict__ l,
-                 const double* __restrict__ wsum, double inv_vol, double* out) {
+                 const double* __restrict__ wsum, double inv_vol, double* out,
+                 const double* __restrict__ scal, double* host) {
+  if (host && blockIdx.x == 0 && threadIdx.x < 16) host[threadIdx.x] = scal[threadIdx.x];
   const df shift = df_from_double(wsum ? *wsum * inv_vol : 0.0);
   constexpr int U = 4;
   const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
@@ -2031,7 +2103,9 @@ __device__ __forceinline__ void df_to_f64_v4_body(int bx, int G, long long n4, c
 
 __global__ void __launch_bounds__(256)
 df_to_f64_v4_kernel(long long n4, const float4* __restrict__ h, const float4* __restrict__ l,
-                    const double* __restrict__ wsum, double inv_vol, double2* out) {
+                    const double* __restrict__ wsum, double inv_vol, double2* out,
+                    const double* __restrict__ scal, double* host) {
+  if (host && blockIdx.x == 0 && threadIdx.x < 16) host[threadIdx.x] = scal[threadIdx.x];
   df_to_f64_v4_body(blockIdx.x, gridDim.x, n4, h, l, wsum, inv_vol, out);
 }
 
@@ -2341,15 +2415,14 @@ cudaError_t launch_thomas_m(const tpt_plan_s* p, const MixedWork& w, cudaStream_
     mo1 = mo0;
   }
   int* next_tile = reinterpret_cast<int*>(w.scal + 14);
-  cudaError_t e = cudaMemsetAsync(next_tile, 0, sizeof(int), s);
-  if (e != cudaSuccess) return e;
   const size_t smem = 1024 + static_cast<size_t>(geo.coef_bytes) + static_cast<size_t>(geo.stages) * geo.in_bytes +
                       static_cast<size_t>(geo.out_bytes);
   auto kern = thomas_tma_kernel<FMT, M, TLT, NT>;
   // The cap is the kernel's fixed budget, never the size of this launch:
   // threads that launch the same kernel for different Nz (the server's slots)
   // would otherwise lower each other's cap between setting it and launching.
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kThomasSmemBudget / kPerSm);
+  const cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kThomasSmemBudget / kPerSm);
   if (e != cudaSuccess) return e;
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->dev);
@@ -2453,12 +2526,10 @@ cudaError_t launch_thomas2_m(const tpt_plan_s* p, const MixedWork& w, cudaStream
   if (!thomas2_job<FMT, M>(p, w, 0, &J)) return cudaErrorInvalidValue;
   if (J.ntiles <= 0) return cudaSuccess;
   int* next_tile = reinterpret_cast<int*>(w.scal + 14);
-  cudaError_t e = cudaMemsetAsync(next_tile, 0, sizeof(int), s);
-  if (e != cudaSuccess) return e;
   const size_t smem = thomas2_smem(J.geo);
   auto kern = thomas2_kernel<FMT, M, 0, NT>;
   // a fixed cap (see launch_thomas_m)
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, t2_smem_budget(NT));
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, t2_smem_budget(NT));
   if (e != cudaSuccess) return e;
   if (smem > static_cast<size_t>(t2_smem_budget(NT))) return cudaErrorInvalidConfiguration;
   const int slots = sm_count(p->dev) * (kThomasThreads / NT);
@@ -2634,12 +2705,16 @@ bool res_maps(const tpt_plan_s* p, const MixedWork& w, CUtensorMap m[4]) {
 }
 
 template <int FMT, int HA, int WX, int WY, int WZ, int SING>
-cudaError_t launch_res(const tpt_plan_s* p, const MixedWork& w, cudaStream_t s) {
+cudaError_t launch_res(const tpt_plan_s* p, const MixedWork& w, bool test, cudaStream_t s) {
   const int nx = p->n[0], ny = p->n[1], nz = p->n[2];
   const int kseg = 32;
   dim3 block(32, 4), grid((nx + 31) / 32, (ny + 3) / 4, (nz + kseg - 1) / kseg);
   const float ah = static_cast<float>(p->alpha);
   const float al = static_cast<float>(p->alpha - static_cast<double>(ah));
+  auto conv_of = [&](const dim3& g, int warps) {
+    return Conv{test ? w.scal : nullptr, static_cast<double>(npts(p)), p->vol, p->rtol, p->singular ? 1 : 0,
+                g.x * g.y * g.z * static_cast<unsigned>(warps)};
+  };
   note_launch(1);
   if (nx % 4 == 0 && p->mixed.res_kernel != 1) {   // TMA-staged tiles (rows of 16-byte multiples)
     CUtensorMap m[4];
@@ -2654,7 +2729,8 @@ cudaError_t launch_res(const tpt_plan_s* p, const MixedWork& w, cudaStream_t s) 
       if (e != cudaSuccess) return e;
       // the kernel's blocks per SM (its launch bounds): three on a problem without walls or alpha
       const long long slots = ((WX || WY || WZ || HA) ? 2LL : 3LL) * sm_count(p->dev);
-      const ResJob J = res_job(p, w, m, res_kseg([&](int k) { return res_blocks(p, k); }, slots), 0);
+      ResJob J = res_job(p, w, m, res_kseg([&](int k) { return res_blocks(p, k); }, slots), 0);
+      J.conv = conv_of(dim3(J.tx, J.ty, J.tz), kResTY);
       kern<<<dim3(J.tx, J.ty, J.tz), kResThreads, kResSmem, s>>>(J);
       return cudaGetLastError();
     }
@@ -2664,31 +2740,32 @@ cudaError_t launch_res(const tpt_plan_s* p, const MixedWork& w, cudaStream_t s) 
     residual_df2_kernel<FMT, HA, WX, WY, WZ, SING><<<grid2, block, 0, s>>>(
         nx, ny, nz, p->mixed.ldx, kseg, w.fh, w.fl, w.ph, w.pl, w.R[0], w.R[1],
         rows_of(p->mixed.dfrows[0], nx), rows_of(p->mixed.dfrows[1], ny), rows_of(p->mixed.dfrows[2], nz),
-        ah, al, w.scal + 5, 1.0 / p->vol, w.scal + 1, w.skip);
+        ah, al, w.scal + 5, 1.0 / p->vol, w.scal + 1, w.skip, conv_of(grid2, 4));
     return cudaGetLastError();
   }
   residual_df_kernel<FMT, HA, WX, WY, WZ, SING><<<grid, block, 0, s>>>(
       nx, ny, nz, p->mixed.ldx, kseg, w.fh, w.fl, w.ph, w.pl, w.R[0], w.R[1],
       rows_of(p->mixed.dfrows[0], nx), rows_of(p->mixed.dfrows[1], ny), rows_of(p->mixed.dfrows[2], nz),
-      ah, al, w.scal + 5, 1.0 / p->vol, w.scal + 1, w.skip);
+      ah, al, w.scal + 5, 1.0 / p->vol, w.scal + 1, w.skip, conv_of(grid, 4));
   return cudaGetLastError();
 }
 
+// test: followed by the stopping test (converge_body)
 template <int FMT>
-cudaError_t launch_residual(const tpt_plan_s* p, const MixedWork& w, cudaStream_t s) {
+cudaError_t launch_residual(const tpt_plan_s* p, const MixedWork& w, cudaStream_t s, bool test = false) {
   const int* hw = p->mixed.has_w;
   const int code = (p->alpha != 0.0 ? 8 : 0) | (hw[0] ? 4 : 0) | (hw[1] ? 2 : 0) | (hw[2] ? 1 : 0);
   // a singular problem (alpha = 0, every direction periodic or Neumann-Neumann)
   // has no wall with a diagonal remainder, so code is 0 there
-  if (p->singular) return launch_res<FMT, 0, 0, 0, 0, 1>(p, w, s);
+  if (p->singular) return launch_res<FMT, 0, 0, 0, 0, 1>(p, w, test, s);
   switch (code) {
-    case 0: return launch_res<FMT, 0, 0, 0, 0, 0>(p, w, s);
-    case 8: return launch_res<FMT, 1, 0, 0, 0, 0>(p, w, s);
+    case 0: return launch_res<FMT, 0, 0, 0, 0, 0>(p, w, test, s);
+    case 8: return launch_res<FMT, 1, 0, 0, 0, 0>(p, w, test, s);
     default: break;
   }
   // walls with a diagonal remainder (Dirichlet): one general instantiation
-  if (p->alpha != 0.0) return launch_res<FMT, 1, 1, 1, 1, 0>(p, w, s);
-  return launch_res<FMT, 0, 1, 1, 1, 0>(p, w, s);
+  if (p->alpha != 0.0) return launch_res<FMT, 1, 1, 1, 1, 0>(p, w, test, s);
+  return launch_res<FMT, 0, 1, 1, 1, 0>(p, w, test, s);
 }
 
 // Operands and output of transform stage i of one correction (Algorithm 1
@@ -2820,52 +2897,6 @@ int correction(tpt_plan_s* p, const MixedWork& w, bool accumulate, cudaStream_t 
   return TPT_OK;
 }
 
-// Device-side stopping test of the adaptive refinement (Sec. 4.1), run after
-// each correction's residual: scal[8] (as int) becomes 1 once ||r|| / ||f||
-// <= rtol (norm of f projected to compatible form for a singular problem, as
-// proj_norm2 computes it), 2 for a non-finite norm and 3 after a timed-out
-// wait, and from then on every kernel of a later correction returns at entry;
-// scal[8] + 4 bytes counts the corrections applied; scal[11], scal[12] keep
-// the last r^2 and f^2 sums; otherwise r's sum is cleared for the next residual.
-__device__ __forceinline__ void converge_body(double* scal, double npts, double vol, int singular, double rtol) {
-  int* flags = reinterpret_cast<int*>(scal + 8);
-  if (flags[0]) return;
-  flags[1] += 1;
-  const double r2 = scal[1];
-  double fn2 = scal[5];
-  if (singular) {
-    const double c = scal[7] / vol;
-    fn2 = scal[5] - 2.0 * c * scal[6] + npts * c * c;
-  }
-  scal[11] = r2;
-  scal[12] = fn2;
-  if (*reinterpret_cast<const int*>(scal + 15)) {
-    flags[0] = 3;
-    return;
-  }
-  if (!isfinite(r2) || !isfinite(fn2)) {
-    flags[0] = 2;
-    return;
-  }
-  const double rel = fn2 > 0.0 ? sqrt(r2 / fn2) : sqrt(r2);
-  if (rel <= rtol) {
-    flags[0] = 1;
-    return;
-  }
-  scal[1] = 0.0;
-  scal[2] = 0.0;
-}
-
-__global__ void converge_kernel(double* scal, double npts, double vol, int singular, double rtol) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  converge_body(scal, npts, vol, singular, rtol);
-}
-
-// The 16 workspace scalars into a pinned, device-mapped host slot.
-__global__ void scal_to_host_kernel(const double* __restrict__ scal, double* host) {
-  if (threadIdx.x < 16) host[threadIdx.x] = scal[threadIdx.x];
-}
-
 // ------------------------------------------------------- grouped launches
 // The per-instance data of the grouped stage kernels of a batch: each of
 // those kernels runs once over all instances, a block (or thread) finding its
@@ -2960,10 +2991,14 @@ void add_stage_times(tpt_plan_s* p, float* ms, bool with_residual) {
 // no host synchronisation (capturable in a CUDA graph); the sums stay in the
 // workspace scalars for mixed_info().
 // Gauge sum (singular problems) and float64 output of the float-pair phi.
-cudaError_t launch_output(const tpt_plan_s* p, const MixedWork& w, double* phi, cudaStream_t s) {
+// clear: the gauge sum may hold an earlier one (the stopping test clears it
+// otherwise); host: device address of a pinned slot for the 16 scalars, or null
+// (written by the output kernel: a copy engine's queue would hold them up).
+cudaError_t launch_output(const tpt_plan_s* p, const MixedWork& w, double* phi, cudaStream_t s, bool clear,
+                          double* host) {
   const long long n = static_cast<long long>(npts(p));
   if (p->singular) {
-    cudaError_t e0 = cudaMemsetAsync(w.scal + 2, 0, sizeof(double), s);
+    cudaError_t e0 = clear ? cudaMemsetAsync(w.scal + 2, 0, sizeof(double), s) : cudaSuccess;
     if (e0 != cudaSuccess) return e0;
     note_launch(1);
     if (p->n[0] % 4 == 0)   // four points per thread
@@ -2982,10 +3017,10 @@ cudaError_t launch_output(const tpt_plan_s* p, const MixedWork& w, double* phi, 
   if (n % 4 == 0 && reinterpret_cast<uintptr_t>(phi) % 16 == 0)
     df_to_f64_v4_kernel<<<grid_for(n / 4, 256, p->dev), 256, 0, s>>>(
         n / 4, reinterpret_cast<const float4*>(w.ph), reinterpret_cast<const float4*>(w.pl),
-        p->singular ? w.scal + 2 : nullptr, 1.0 / p->vol, reinterpret_cast<double2*>(phi));
+        p->singular ? w.scal + 2 : nullptr, 1.0 / p->vol, reinterpret_cast<double2*>(phi), w.scal, host);
   else
     df_to_f64_kernel<<<grid_for(n, 256, p->dev), 256, 0, s>>>(n, w.ph, w.pl, p->singular ? w.scal + 2 : nullptr,
-                                                              1.0 / p->vol, phi);
+                                                              1.0 / p->vol, phi, w.scal, host);
   return cudaGetLastError();
 }
 
@@ -3006,16 +3041,10 @@ int enqueue_adaptive(tpt_plan_s* p, const MixedWork& w, const double* f, double*
   }
   for (int c = first; c < last; ++c) {
     MX_TRY(correction<FMT>(p, w, c > 0, s));
-    MX_CUDA(launch_residual<FMT>(p, w, s));
-    note_launch(1);
-    converge_kernel<<<1, 32, 0, s>>>(w.scal, np, p->vol, p->singular ? 1 : 0, p->rtol);
-    MX_CUDA(cudaGetLastError());
+    MX_CUDA(launch_residual<FMT>(p, w, s, true));
   }
-  MX_CUDA(launch_output(p, w, phi, s));
-  if (!d_hdst) return TPT_OK;   // the caller gathers the scalars itself
-  note_launch(1);
-  scal_to_host_kernel<<<1, 32, 0, s>>>(w.scal, d_hdst);   // no copy engine: see pinned_slot_acquire
-  return cudaGetLastError() == cudaSuccess ? TPT_OK : TPT_ERR_CUDA;
+  MX_CUDA(launch_output(p, w, phi, s, false, d_hdst));   // no slot: the caller gathers the scalars itself
+  return TPT_OK;
 }
 
 // The first `planned` corrections as a CUDA graph (captured on the plan's own
@@ -3220,7 +3249,7 @@ int solve_fmt(tpt_plan_s* p, const double* f, double* phi, void* work, cudaStrea
     if (iters >= corrections) break;
   }
   if (timing) cudaEventRecord(p->ev[10], s);
-  MX_CUDA(launch_output(p, w, phi, s));
+  MX_CUDA(launch_output(p, w, phi, s, true, nullptr));
   if (timing) {
     cudaEventRecord(p->ev[11], s);
     MX_CUDA(cudaEventSynchronize(p->ev[11]));
