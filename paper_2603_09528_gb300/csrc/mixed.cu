@@ -103,7 +103,7 @@ __device__ __forceinline__ void acc_mul(df& acc, float ch, float cl, df x) {
 // sums[0..2].  No float64 arithmetic per point.
 template <int FMT>
 __global__ void __launch_bounds__(256)
-prepare_kernel(int nx, int ny, int nz, int ldx, int nbi, const double* __restrict__ f, float* __restrict__ fh,
+prepare_kernel(int nx, int ny, int nz, int ldx, int ldf, int nbi, const double* __restrict__ f, float* __restrict__ fh,
                float* __restrict__ fl, void* r0, void* r1, const float* __restrict__ gx,
                const float* __restrict__ gy, const float* __restrict__ gz, double* sums) {
   // work item t covers x-line (j, k) = t / nbi, points (t % nbi) * 256 + 0..255;
@@ -133,7 +133,7 @@ prepare_kernel(int nx, int ny, int nz, int ldx, int nbi, const double* __restric
       const int i = ii[u];
       if (i < 0) continue;
       const int j = static_cast<int>(line[u] % ny), k = static_cast<int>(line[u] / ny);
-      const long long o = i + static_cast<long long>(nx) * line[u];
+      const long long o = i + static_cast<long long>(ldf) * line[u];
       const df d = split_double_int(v[u]);
       fh[o] = d.hi;
       fl[o] = d.lo;
@@ -1146,7 +1146,7 @@ __device__ __forceinline__ void arrive_converge(const Conv& c) {
 // zero coefficient).
 template <int FMT, int HAS_ALPHA, int WX, int WY, int WZ, int SING>
 __global__ void __launch_bounds__(128)
-residual_df_kernel(int nx, int ny, int nz, int ldx, int kseg, const float* __restrict__ fh,
+residual_df_kernel(int nx, int ny, int nz, int ldx, int ldf, int kseg, const float* __restrict__ fh,
                    const float* __restrict__ fl, const float* __restrict__ ph,
                    const float* __restrict__ pl, void* r0, void* r1, BRows RX, BRows RY, BRows RZ,
                    float alpha_h, float alpha_l, const double* __restrict__ fsums, double inv_vol,
@@ -1158,10 +1158,10 @@ residual_df_kernel(int nx, int ny, int nz, int ldx, int kseg, const float* __res
   const int k1 = min(nz, k0 + kseg);
   float acc2 = 0.0f;
   if (i < nx && j < ny && k0 < nz) {
-    const long long sz = static_cast<long long>(nx) * ny;
-    const long long base = i + static_cast<long long>(nx) * j;
+    const long long sz = static_cast<long long>(ldf) * ny;
+    const long long base = i + static_cast<long long>(ldf) * j;
     const int dxm = (i == 0) ? nx - 1 : -1, dxp = (i == nx - 1) ? -(nx - 1) : 1;
-    const int dym = (j == 0) ? (ny - 1) * nx : -nx, dyp = (j == ny - 1) ? -(ny - 1) * nx : nx;
+    const int dym = (j == 0) ? (ny - 1) * ldf : -ldf, dyp = (j == ny - 1) ? -(ny - 1) * ldf : ldf;
     const float axh = RX.ah[i], axl = RX.al[i], cxh = RX.ch[i], cxl = RX.cl[i];
     const float ayh = RY.ah[j], ayl = RY.al[j], cyh = RY.ch[j], cyl = RY.cl[j];
     df fshift = {0.0f, 0.0f};
@@ -1369,7 +1369,7 @@ __device__ __forceinline__ df fshift_of(const double* fsums, double inv_vol) {
 // k.  Used where the plane rows cannot be described by a tensor map.
 template <int FMT, int HAS_ALPHA, int WX, int WY, int WZ, int SING>
 __global__ void __launch_bounds__(128, 5)
-residual_df2_kernel(int nx, int ny, int nz, int ldx, int kseg, const float* __restrict__ fh,
+residual_df2_kernel(int nx, int ny, int nz, int ldx, int ldf, int kseg, const float* __restrict__ fh,
                     const float* __restrict__ fl, const float* __restrict__ ph,
                     const float* __restrict__ pl, void* r0, void* r1, BRows RX, BRows RY, BRows RZ,
                     float alpha_h, float alpha_l, const double* __restrict__ fsums, double inv_vol,
@@ -1381,11 +1381,11 @@ residual_df2_kernel(int nx, int ny, int nz, int ldx, int kseg, const float* __re
   const int k1 = min(nz, k0 + kseg);
   float acc2 = 0.0f;
   if (i < nx && j < ny && k0 < nz) {
-    const long long sz = static_cast<long long>(nx) * ny;
-    const long long base = i + static_cast<long long>(nx) * j;
+    const long long sz = static_cast<long long>(ldf) * ny;
+    const long long base = i + static_cast<long long>(ldf) * j;
     const int dxm = (i == 0) ? nx - 1 : -1;                    // from point i
     const int dxp = (i + 1 == nx - 1) ? -(nx - 2) : 2;         // from point i (to i + 2 or the wrap)
-    const int dym = (j == 0) ? (ny - 1) * nx : -nx, dyp = (j == ny - 1) ? -(ny - 1) * nx : nx;
+    const int dym = (j == 0) ? (ny - 1) * ldf : -ldf, dyp = (j == ny - 1) ? -(ny - 1) * ldf : ldf;
     const PairCoefs c = pair_coefs<WX, WY>(RX, RY, i, j);
     const df fshift = SING ? fshift_of(fsums, inv_vol) : df{0.0f, 0.0f};
     const float* hk = ph + base + sz * k0;
@@ -1615,7 +1615,7 @@ constexpr int kResThreads = 32 * (kResTY + 1);
 // b - first of instance `job` (tiles x fastest, then y, then z segments).
 struct ResJob {
   CUtensorMap tPH, tPL, tFH, tFL;
-  int nx, ny, nz, ldx, px, py;
+  int nx, ny, nz, ldx, ldf, px, py;
   const float *ph, *pl;
   void *r0, *r1;
   BRows RX, RY, RZ;
@@ -1636,7 +1636,7 @@ __device__ __forceinline__ void residual_tma_body(const ResJob& J, int bx, int b
   const CUtensorMap& tPL = J.tPL;
   const CUtensorMap& tFH = J.tFH;
   const CUtensorMap& tFL = J.tFL;
-  const int nx = J.nx, ny = J.ny, nz = J.nz, ldx = J.ldx, px = J.px, py = J.py;
+  const int nx = J.nx, ny = J.ny, nz = J.nz, ldx = J.ldx, ldf = J.ldf, px = J.px, py = J.py;
   const float* __restrict__ ph = J.ph;
   const float* __restrict__ pl = J.pl;
   void* r0 = J.r0;
@@ -1719,7 +1719,7 @@ __device__ __forceinline__ void residual_tma_body(const ResJob& J, int bx, int b
   const float2 ach = p_dup(-alpha_h), anch = p_dup(alpha_h), ancl = p_dup(alpha_l);
   const int pc = (warp + 1) * kResPW + 4 + 2 * lane;          // centre of the pair in a phi stage
   const int fc = warp * kResTX + 2 * lane;
-  const long long sz = static_cast<long long>(nx) * ny;
+  const long long sz = static_cast<long long>(ldf) * ny;
   auto pair_at = [&](const uint8_t* st, int e) -> dfx2 {      // points e, e + 1 (e even)
     return {*reinterpret_cast<const float2*>(reinterpret_cast<const float*>(st) + e),
             *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(st + kResPBytes) + e)};
@@ -1760,15 +1760,15 @@ __device__ __forceinline__ void residual_tma_body(const ResJob& J, int bx, int b
     if (edge) {
       const long long plane = sz * k;
       if (px && i == 0) {
-        const long long o = plane + static_cast<long long>(nx) * j + (nx - 1);
+        const long long o = plane + static_cast<long long>(ldf) * j + (nx - 1);
         xm = {ph[o], pl[o]};
       }
       if (px && i + 2 == nx) {
-        const long long o = plane + static_cast<long long>(nx) * j;
+        const long long o = plane + static_cast<long long>(ldf) * j;
         xp = {ph[o], pl[o]};
       }
       if (py && j == 0) {
-        const long long o = plane + static_cast<long long>(nx) * (ny - 1) + i;
+        const long long o = plane + static_cast<long long>(ldf) * (ny - 1) + i;
         YM = {*reinterpret_cast<const float2*>(ph + o), *reinterpret_cast<const float2*>(pl + o)};
       }
       if (py && j == ny - 1) {
@@ -1833,7 +1833,7 @@ residual_tma_group_kernel(const ResJob* __restrict__ jobs, int njobs) {
 // sum of cell volume times phi (float pair) into *out, for the exact gauge;
 // work items are 256-point chunks of x-lines (one division per item)
 __global__ void __launch_bounds__(256)
-wsum_df_kernel(int nx, int ny, int nz, const float* __restrict__ h, const float* __restrict__ l,
+wsum_df_kernel(int nx, int ny, int nz, int ldf, const float* __restrict__ h, const float* __restrict__ l,
                const float* __restrict__ gx, const float* __restrict__ gy,
                const float* __restrict__ gz, double* out) {
   const int nbi = (nx + 255) / 256;
@@ -1851,7 +1851,7 @@ wsum_df_kernel(int nx, int ny, int nz, const float* __restrict__ h, const float*
       ii[u] = static_cast<int>(t % nbi) * 256 + threadIdx.x;
       const bool ok = t < items && ii[u] < nx;
       if (!ok) ii[u] = -1;
-      const long long o = ok ? ii[u] + static_cast<long long>(nx) * line[u] : 0;
+      const long long o = ok ? ii[u] + static_cast<long long>(ldf) * line[u] : 0;
       hh[u] = ok ? h[o] : 0.0f;
       ll[u] = ok ? l[o] : 0.0f;
     }
@@ -1899,13 +1899,48 @@ df_to_f64_kernel(long long n, const float* __restrict__ h, const float* __restri
   }
 }
 
+// The same from rows of stride ldf (Nx even, ldf > Nx): two points per thread,
+// blocks as line_block(nx, 2); out 16-byte aligned.
+__global__ void __launch_bounds__(256)
+df_rows_to_f64_kernel(int nx, long long lines, int ldf, const float* __restrict__ h, const float* __restrict__ l,
+                      const double* __restrict__ wsum, double inv_vol, double* out,
+                      const double* __restrict__ scal, double* host) {
+  if (host && blockIdx.x == 0 && threadIdx.x < 16 && threadIdx.y == 0) host[threadIdx.x] = scal[threadIdx.x];
+  const df shift = df_from_double(wsum ? *wsum * inv_vol : 0.0);
+  for (long long L = blockIdx.x * static_cast<long long>(blockDim.y) + threadIdx.y; L < lines;
+       L += static_cast<long long>(gridDim.x) * blockDim.y) {
+    for (int i = 2 * threadIdx.x; i < nx; i += 2 * blockDim.x) {
+      const float2 hh = *reinterpret_cast<const float2*>(h + L * ldf + i);
+      const float2 ll = *reinterpret_cast<const float2*>(l + L * ldf + i);
+      const df a = df_sub({hh.x, ll.x}, shift), b = df_sub({hh.y, ll.y}, shift);
+      *reinterpret_cast<double2*>(out + L * nx + i) =
+          make_double2(f2d_int(a.hi) + f2d_int(a.lo), f2d_int(b.hi) + f2d_int(b.lo));
+    }
+  }
+}
+
+// One point at a time from rows of stride ldf (any alignment of out).
+__global__ void __launch_bounds__(256)
+df_points_to_f64_kernel(int nx, long long n, int ldf, const float* __restrict__ h, const float* __restrict__ l,
+                        const double* __restrict__ wsum, double inv_vol, double* out,
+                        const double* __restrict__ scal, double* host) {
+  if (host && blockIdx.x == 0 && threadIdx.x < 16) host[threadIdx.x] = scal[threadIdx.x];
+  const df shift = df_from_double(wsum ? *wsum * inv_vol : 0.0);
+  for (long long o = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; o < n;
+       o += static_cast<long long>(gridDim.x) * blockDim.x) {
+    const long long q = o / nx * ldf + o % nx;
+    const df x = df_sub({h[q], l[q]}, shift);
+    out[o] = f2d_int(x.hi) + f2d_int(x.lo);
+  }
+}
+
 // Vectorised forms of prepare_kernel, wsum_df_kernel and df_to_f64_kernel for
 // the common aligned case (Nx a multiple of the vector width): each thread
 // moves 2 or 4 consecutive points of an x-line with 16-byte loads and stores,
 // and the per-line weights and index divisions are shared by those points.
 // Same operations per point as the scalar kernels.
 template <int FMT>
-__device__ __forceinline__ void prepare2_body(int bx, int G, int nx, int ny, int nz, int ldx,
+__device__ __forceinline__ void prepare2_body(int bx, int G, int nx, int ny, int nz, int ldx, int ldf,
                                               const double* __restrict__ f, float* __restrict__ fh,
                                               float* __restrict__ fl, void* r0, void* r1,
                                               const float* __restrict__ gx, const float* __restrict__ gy,
@@ -1943,7 +1978,7 @@ __device__ __forceinline__ void prepare2_body(int bx, int G, int nx, int ny, int
       for (int u = 0; u < U; ++u) {
         const int L = L0 + u * G * ty;
         if (L >= lines) break;
-        const long long o = i + static_cast<long long>(nx) * L;
+        const long long o = i + static_cast<long long>(ldf) * L;
         const df d0 = split_double_int(v[u].x), d1 = split_double_int(v[u].y);
         *reinterpret_cast<float2*>(fh + o) = make_float2(d0.hi, d1.hi);
         *reinterpret_cast<float2*>(fl + o) = make_float2(d0.lo, d1.lo);
@@ -2003,10 +2038,10 @@ __device__ __forceinline__ void prepare2_body(int bx, int G, int nx, int ny, int
 
 template <int FMT>
 __global__ void __launch_bounds__(256)
-prepare2_kernel(int nx, int ny, int nz, int ldx, const double* __restrict__ f, float* __restrict__ fh,
+prepare2_kernel(int nx, int ny, int nz, int ldx, int ldf, const double* __restrict__ f, float* __restrict__ fh,
                 float* __restrict__ fl, void* r0, void* r1, const float* __restrict__ gx,
                 const float* __restrict__ gy, const float* __restrict__ gz, double* sums) {
-  prepare2_body<FMT>(blockIdx.x, gridDim.x, nx, ny, nz, ldx, f, fh, fl, r0, r1, gx, gy, gz, sums);
+  prepare2_body<FMT>(blockIdx.x, gridDim.x, nx, ny, nz, ldx, ldf, f, fh, fl, r0, r1, gx, gy, gz, sums);
 }
 
 // sum of cell volume times phi, four points of an x-line per thread; lines
@@ -2225,11 +2260,17 @@ struct MixedSizes {
   size_t nf, nr, nab, eb, np;
 };
 
+// Row stride of the float-pair planes of f and phi: Nx, or Nx + 2 where that makes
+// rows of whole 16 bytes out of an even Nx (mixed_setup), which the TMA-staged
+// residual needs (150x277x133: 66 us a launch by direct loads, 45 staged; solve
+// 655 -> 613 us).  The two columns are never read.
+int row_stride(const tpt_plan_s* p) { return p->n[0] + p->mixed.row_pad; }
+
 MixedSizes sizes_of(const tpt_plan_s* p) {
   const MixedTables& m = p->mixed;
   const size_t nx = p->n[0], ny = p->n[1], nz = p->n[2];
   MixedSizes s;
-  s.nf = nx * ny * nz;
+  s.nf = static_cast<size_t>(row_stride(p)) * ny * nz;
   s.nr = static_cast<size_t>(m.ldx) * ny * nz;
   s.nab = std::max(static_cast<size_t>(m.ldy) * nx, static_cast<size_t>(m.ldx) * ny) * nz;
   s.eb = elem_bytes(m.fmt);
@@ -2317,12 +2358,12 @@ cudaError_t launch_prepare(const tpt_plan_s* p, const double* f, const MixedWork
     const long long lines = static_cast<long long>(p->n[1]) * p->n[2];
     const dim3 blk = line_block(p->n[0], 2);
     prepare2_kernel<FMT><<<grid_for(lines * blk.x, blk.x * blk.y, p->dev), blk, 0, s>>>(
-        p->n[0], p->n[1], p->n[2], p->mixed.ldx, f, w.fh, w.fl, w.R[0], w.R[1], p->mixed.dfgeom[0],
+        p->n[0], p->n[1], p->n[2], p->mixed.ldx, row_stride(p), f, w.fh, w.fl, w.R[0], w.R[1], p->mixed.dfgeom[0],
         p->mixed.dfgeom[1], p->mixed.dfgeom[2], w.scal + 5);
     return cudaGetLastError();
   }
   prepare_kernel<FMT><<<grid_for(items * 256, 256, p->dev), 256, 0, s>>>(
-      p->n[0], p->n[1], p->n[2], p->mixed.ldx, nbi, f, w.fh, w.fl, w.R[0], w.R[1], p->mixed.dfgeom[0],
+      p->n[0], p->n[1], p->n[2], p->mixed.ldx, row_stride(p), nbi, f, w.fh, w.fl, w.R[0], w.R[1], p->mixed.dfgeom[0],
       p->mixed.dfgeom[1], p->mixed.dfgeom[2], w.scal + 5);
   return cudaGetLastError();
 }
@@ -2671,6 +2712,7 @@ ResJob res_job(const tpt_plan_s* p, const MixedWork& w, const CUtensorMap m[4], 
   J.ny = ny;
   J.nz = nz;
   J.ldx = p->mixed.ldx;
+  J.ldf = row_stride(p);
   J.px = p->dir[0].periodic ? 1 : 0;
   J.py = p->dir[1].periodic ? 1 : 0;
   J.ph = w.ph;
@@ -2696,12 +2738,12 @@ ResJob res_job(const tpt_plan_s* p, const MixedWork& w, const CUtensorMap m[4], 
 }
 
 bool res_maps(const tpt_plan_s* p, const MixedWork& w, CUtensorMap m[4]) {
-  const int nx = p->n[0];
+  const int nx = p->n[0], ldf = row_stride(p);
   const long long rows = static_cast<long long>(p->n[1]) * p->n[2];
-  return nx % 4 == 0 && tc::make_plain_map(&m[0], w.ph, 4, nx, rows, 4LL * nx, kResPW, kResTY + 2) &&
-         tc::make_plain_map(&m[1], w.pl, 4, nx, rows, 4LL * nx, kResPW, kResTY + 2) &&
-         tc::make_plain_map(&m[2], w.fh, 4, nx, rows, 4LL * nx, kResTX, kResTY) &&
-         tc::make_plain_map(&m[3], w.fl, 4, nx, rows, 4LL * nx, kResTX, kResTY);
+  return ldf % 4 == 0 && tc::make_plain_map(&m[0], w.ph, 4, nx, rows, 4LL * ldf, kResPW, kResTY + 2) &&
+         tc::make_plain_map(&m[1], w.pl, 4, nx, rows, 4LL * ldf, kResPW, kResTY + 2) &&
+         tc::make_plain_map(&m[2], w.fh, 4, nx, rows, 4LL * ldf, kResTX, kResTY) &&
+         tc::make_plain_map(&m[3], w.fl, 4, nx, rows, 4LL * ldf, kResTX, kResTY);
 }
 
 template <int FMT, int HA, int WX, int WY, int WZ, int SING>
@@ -2716,14 +2758,9 @@ cudaError_t launch_res(const tpt_plan_s* p, const MixedWork& w, bool test, cudaS
                 g.x * g.y * g.z * static_cast<unsigned>(warps)};
   };
   note_launch(1);
-  if (nx % 4 == 0 && p->mixed.res_kernel != 1) {   // TMA-staged tiles (rows of 16-byte multiples)
+  if (p->mixed.res_kernel != 1) {   // TMA-staged tiles (rows of 16-byte multiples)
     CUtensorMap m[4];
-    const long long rows = static_cast<long long>(ny) * nz;
-    bool maps = tc::make_plain_map(&m[0], w.ph, 4, nx, rows, 4LL * nx, kResPW, kResTY + 2) &&
-                tc::make_plain_map(&m[1], w.pl, 4, nx, rows, 4LL * nx, kResPW, kResTY + 2) &&
-                tc::make_plain_map(&m[2], w.fh, 4, nx, rows, 4LL * nx, kResTX, kResTY) &&
-                tc::make_plain_map(&m[3], w.fl, 4, nx, rows, 4LL * nx, kResTX, kResTY);
-    if (maps) {
+    if (res_maps(p, w, m)) {
       auto kern = residual_tma_kernel<FMT, HA, WX, WY, WZ, SING>;
       cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
       if (e != cudaSuccess) return e;
@@ -2738,13 +2775,13 @@ cudaError_t launch_res(const tpt_plan_s* p, const MixedWork& w, bool test, cudaS
   if (nx % 2 == 0) {   // two points per thread
     dim3 grid2((nx / 2 + 31) / 32, (ny + 3) / 4, (nz + kseg - 1) / kseg);
     residual_df2_kernel<FMT, HA, WX, WY, WZ, SING><<<grid2, block, 0, s>>>(
-        nx, ny, nz, p->mixed.ldx, kseg, w.fh, w.fl, w.ph, w.pl, w.R[0], w.R[1],
+        nx, ny, nz, p->mixed.ldx, row_stride(p), kseg, w.fh, w.fl, w.ph, w.pl, w.R[0], w.R[1],
         rows_of(p->mixed.dfrows[0], nx), rows_of(p->mixed.dfrows[1], ny), rows_of(p->mixed.dfrows[2], nz),
         ah, al, w.scal + 5, 1.0 / p->vol, w.scal + 1, w.skip, conv_of(grid2, 4));
     return cudaGetLastError();
   }
   residual_df_kernel<FMT, HA, WX, WY, WZ, SING><<<grid, block, 0, s>>>(
-      nx, ny, nz, p->mixed.ldx, kseg, w.fh, w.fl, w.ph, w.pl, w.R[0], w.R[1],
+      nx, ny, nz, p->mixed.ldx, row_stride(p), kseg, w.fh, w.fl, w.ph, w.pl, w.R[0], w.R[1],
       rows_of(p->mixed.dfrows[0], nx), rows_of(p->mixed.dfrows[1], ny), rows_of(p->mixed.dfrows[2], nz),
       ah, al, w.scal + 5, 1.0 / p->vol, w.scal + 1, w.skip, conv_of(grid, 4));
   return cudaGetLastError();
@@ -2800,7 +2837,7 @@ StageGemm stage_gemm(const tpt_plan_s* p, const MixedWork& w, int i, bool accumu
     default:  // A = Q_x rows i, B = T4 rows (j,k) -> phi (float pair) (+)= result
       t.a = operand(m.q[0][1], nx, nx, m.ldx);
       t.b = operand(w.B, ny * nz, nx, m.ldx);
-      t.g = gout(nx, ny * nz, nx, kBig, 0, nx, w.ph, w.pl, tc::kOutDF, accumulate ? 1 : 0, 0, err);
+      t.g = gout(nx, ny * nz, nx, kBig, 0, row_stride(p), w.ph, w.pl, tc::kOutDF, accumulate ? 1 : 0, 0, err);
       break;
   }
   return t;
@@ -2933,7 +2970,7 @@ __global__ void group_clear_kernel(const InstJob* __restrict__ jobs) {
 template <int FMT>
 __global__ void __launch_bounds__(256) group_prepare_kernel(const InstJob* __restrict__ jobs, int njobs) {
   const InstJob& J = jobs[inst_of(jobs, njobs, 0, blockIdx.x)];
-  prepare2_body<FMT>(blockIdx.x - J.first[0], J.blocks[0], J.nx, J.ny, J.nz, J.ldx, J.f, J.fh, J.fl, J.r0, J.r1,
+  prepare2_body<FMT>(blockIdx.x - J.first[0], J.blocks[0], J.nx, J.ny, J.nz, J.ldx, J.nx, J.f, J.fh, J.fl, J.r0, J.r1,
                      J.gx, J.gy, J.gz, J.scal + 5);
 }
 
@@ -3007,14 +3044,25 @@ cudaError_t launch_output(const tpt_plan_s* p, const MixedWork& w, double* phi, 
                      line_block(p->n[0], 4), 0, s>>>(p->n[0], p->n[1], p->n[2], w.ph, w.pl, p->mixed.dfgeom[0],
                                                      p->mixed.dfgeom[1], p->mixed.dfgeom[2], w.scal + 2);
     else
-      wsum_df_kernel<<<grid_for(n, 256, p->dev), 256, 0, s>>>(p->n[0], p->n[1], p->n[2], w.ph, w.pl,
+      wsum_df_kernel<<<grid_for(n, 256, p->dev), 256, 0, s>>>(p->n[0], p->n[1], p->n[2], row_stride(p), w.ph, w.pl,
                                                               p->mixed.dfgeom[0], p->mixed.dfgeom[1],
                                                               p->mixed.dfgeom[2], w.scal + 2);
     e0 = cudaGetLastError();
     if (e0 != cudaSuccess) return e0;
   }
   note_launch(1);
-  if (n % 4 == 0 && reinterpret_cast<uintptr_t>(phi) % 16 == 0)
+  const double* wsum = p->singular ? w.scal + 2 : nullptr;
+  const bool aligned = reinterpret_cast<uintptr_t>(phi) % 16 == 0;
+  const int ldf = row_stride(p);
+  if (ldf != p->n[0] && aligned) {
+    const long long lines = static_cast<long long>(p->n[1]) * p->n[2];
+    const dim3 blk = line_block(p->n[0], 2);
+    df_rows_to_f64_kernel<<<grid_for(lines * blk.x, 256, p->dev), blk, 0, s>>>(
+        p->n[0], lines, ldf, w.ph, w.pl, wsum, 1.0 / p->vol, phi, w.scal, host);
+  } else if (ldf != p->n[0]) {
+    df_points_to_f64_kernel<<<grid_for(n, 256, p->dev), 256, 0, s>>>(p->n[0], n, ldf, w.ph, w.pl, wsum,
+                                                                      1.0 / p->vol, phi, w.scal, host);
+  } else if (n % 4 == 0 && aligned)
     df_to_f64_v4_kernel<<<grid_for(n / 4, 256, p->dev), 256, 0, s>>>(
         n / 4, reinterpret_cast<const float4*>(w.ph), reinterpret_cast<const float4*>(w.pl),
         p->singular ? w.scal + 2 : nullptr, 1.0 / p->vol, reinterpret_cast<double2*>(phi), w.scal, host);
@@ -3348,6 +3396,7 @@ int mixed_setup(tpt_plan_s* p) {
   m.fmt = fmt_of(p->precision);
   m.ldx = (p->n[0] + 7) & ~7;
   m.ldy = (p->n[1] + 7) & ~7;
+  m.row_pad = p->n[0] % 4 == 2 ? 2 : 0;
   for (int d = 0; d < 2; ++d) {
     if (p->xform[d] == TPT_XFORM_FFT) {   // no operand matrices: float32 twiddles
       MX_TRY(fft_tables_f32(p, d));

@@ -112,7 +112,8 @@ struct tpt_server_s {
       const size_t fields = 2 * r->npts * sizeof(double) + 3 * 256;
       if (st == TPT_OK && cfg.cuda_device >= 0 && fields + wb > cfg.memory_budget) {
         // a float64 request that only its transforms' scratch keeps out of the
-        // budget runs with less of it
+        // budget runs with less of it, a mixed one without padded rows
+        p->mixed.row_pad = 0;
         const size_t rest = fields + wb - tpt::residue_scratch_bytes(p);
         tpt::residue_limit(p, cfg.memory_budget > rest ? cfg.memory_budget - rest : 0);
         st = tpt_workspace_bytes(p, &wb);

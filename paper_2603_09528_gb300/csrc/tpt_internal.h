@@ -79,6 +79,7 @@ enum { kFmtSplit = 0, kFmtBF16 = 1, kFmtF32 = 2 };
 struct MixedTables {
   int fmt = kFmtSplit;
   int ldx = 0, ldy = 0;            // Nx, Ny rounded up to 8 (operand row strides)
+  int row_pad = 0;                 // columns added to the rows of f and phi (row_stride, mixed.cu)
   void* q[2][2][2] = {};           // [x|y][forward Q^{-1} | inverse Q][plane], row-major
   float* lam_f[2] = {nullptr, nullptr};
   float* zrows_f = nullptr;        // a|b|c of z in float32
