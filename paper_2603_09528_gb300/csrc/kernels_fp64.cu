@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <type_traits>
 
 #include "df.h"
 #include "tpt_internal.h"
@@ -96,49 +97,63 @@ __device__ __forceinline__ double recip_fp64(double m) {
   return fma(r0, fma(d, d, d), r0);
 }
 
-// One thread per (i, j) line.  Forward elimination keeps the reciprocal pivots
-// in `inv` and d' in `out`; back substitution overwrites `out`.  With KEPT the
-// reciprocal pivots are already in `inv` (from an earlier call with the same
-// coefficients and sizes) and are only read.  The singular line (null_i,
-// null_j) is first projected to compatible form (its dz-weighted mean removed,
-// recorded in *defect), its last modal unknown is set to zero, and the result
-// is shifted to zero dz-weighted mean.  The beta-scaled z rows are staged in
-// shared memory once per block (3 Nz doubles, dynamic) when ROWS is set.  f may
-// alias out (each element is read before the same thread writes it).
+// One thread per (i, j) line, or with SPLIT two (threadIdx.y), which eliminate from
+// its two ends and meet in the middle: the upper one rows 0 .. h-1 downwards, the lower one rows
+// nz-1 .. h upwards; the two rows that meet are solved as a 2 x 2 system and each
+// half is then substituted back outwards.  Elimination
+// keeps the reciprocal pivots in `inv` and d' in `out`; back substitution
+// overwrites `out`.  With KEPT the reciprocal pivots are already in `inv` (from
+// an earlier call with the same coefficients and sizes) and are only read.  The
+// singular line (null_i, null_j) is first projected to compatible form (its
+// dz-weighted mean removed, recorded in *defect), the unknown where its
+// elimination breaks down (the last, or row h) is set to zero, and the result is
+// shifted to zero dz-weighted mean.  The beta-scaled z rows are staged in shared memory once per
+// block (3 Nz doubles, dynamic) when ROWS is set.  f may alias out (each element
+// is read before the same thread writes it).
 //
-// GB300's float64 pipe (2 FMA a cycle per SM) bounds large fields: 10 operations
+// GB300's float64 pipe (2 FMA a cycle per SM) bounds large fields: 11 operations
 // a point, 5 with KEPT, where the loads (24 B a point) come near the pipe.
-// Small ones are bound by the chain along a line, so rows are read kAhead at a
-// time, one group ahead of the sweep (the loads of a row waited for the row
-// before: 2300 cycles a row), and the blocks are small enough to reach every SM.
-// 512^3 3.53 -> 2.73 ms, 1.31 with KEPT; 61x97x75 83 -> 45 and 25 us.
+// Small ones are bound by the chain along a line, which SPLIT halves; rows are
+// also read kAhead at a time, one group ahead of the sweep (the loads
+// of a row waited for the row before: 2300 cycles a row), and the blocks are
+// small enough to reach every SM.  512^3 3.53 -> 2.73
+// ms, 1.31 with KEPT; 61x97x75 83 -> 27 and 20 us (SPLIT).
 constexpr int kAhead = 8;
-template <bool ROWS, bool KEPT>
+template <bool ROWS, bool KEPT, bool SPLIT>
 __global__ void __launch_bounds__(128)
 thomas_fp64_kernel(int nx, int ny, int nz, const double* f, double* out,
-                   double* __restrict__ inv, const double* __restrict__ lamx,
+                   double* inv, const double* __restrict__ lamx,
                    const double* __restrict__ lamy, const double* __restrict__ az,
                    const double* __restrict__ bz, const double* __restrict__ cz,
                    const double* __restrict__ dz, double alpha, double beta, int null_i,
                    int null_j, double null_scale, double* defect) {
-  extern __shared__ double zrow[];   // beta a, beta b, beta c (ROWS)
+  extern __shared__ double zrow[];   // beta a, beta b, beta c (ROWS; plan tables)
+  __shared__ double meet[2][2][SPLIT ? 64 : 1];   // c' and d' of the rows that meet
   if (ROWS) {
-    for (int k = threadIdx.x; k < nz; k += blockDim.x) {
+    const int tid = threadIdx.x + blockDim.x * threadIdx.y, nt = blockDim.x * blockDim.y;
+    for (int k = tid; k < nz; k += nt) {
       zrow[k] = k > 0 ? beta * az[k] : 0.0;
       zrow[nz + k] = beta * bz[k];
       zrow[2 * nz + k] = k < nz - 1 ? beta * cz[k] : 0.0;
     }
     __syncthreads();
   }
+  const bool lower = SPLIT && threadIdx.y == 1;
+  const int h = SPLIT ? (nz + 1) / 2 : nz;
+  const int rows = lower ? nz - h : h;               // of this thread
+  const int first = lower ? nz - 1 : 0, dir = lower ? -1 : 1;
+  // coupling to the row before (in the sweep's direction), diagonal, and to the next
   auto ra = [&](int k) { return ROWS ? zrow[k] : (k > 0 ? beta * az[k] : 0.0); };
   auto rb = [&](int k) { return ROWS ? zrow[nz + k] : beta * bz[k]; };
   auto rc = [&](int k) { return ROWS ? zrow[2 * nz + k] : (k < nz - 1 ? beta * cz[k] : 0.0); };
+  auto before = [&](int k) { return lower ? rc(k) : ra(k); };
+  auto after = [&](int k) { return lower ? ra(k) : rc(k); };
   const long long lines = static_cast<long long>(nx) * ny;
   const long long line = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-  if (line >= lines) return;
+  const bool active = line < lines;
   const int i = static_cast<int>(line % nx), j = static_cast<int>(line / nx);
-  const bool is_null = (i == null_i && j == null_j);
-  const double shift = alpha + beta * (lamx[i] + lamy[j]);
+  const bool is_null = active && i == null_i && j == null_j;
+  const double shift = active ? alpha + beta * (lamx[i] + lamy[j]) : 1.0;
   double fshift = 0.0;
   if (is_null) {
     double s = 0.0, w = 0.0;
@@ -147,84 +162,102 @@ thomas_fp64_kernel(int nx, int ny, int nz, const double* f, double* out,
       w += dz[k];
     }
     fshift = s / w;
-    if (defect) *defect = fshift * null_scale;
+    if (defect && !lower) *defect = fshift * null_scale;
   }
+  if (SPLIT && null_i >= 0) __syncthreads();         // both threads have read the line before it is overwritten
   const double* fl = f + line;
   double* ol = out + line;
   double* il = inv + line;
   double fv[kAhead], iv[kAhead];       // rows of the coming group
-  auto fetch = [&](int k0) {
+  auto fetch = [&](int t0) {
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) {
-      const int k = k0 + u;
-      fv[u] = k < nz ? fl[k * lines] : 0.0;
-      if (KEPT) iv[u] = k < nz ? il[k * lines] : 0.0;
+      const bool ok = active && t0 + u < rows;
+      const long long o = static_cast<long long>(first + dir * (t0 + u)) * lines;
+      fv[u] = ok ? fl[o] : 0.0;
+      if (KEPT) iv[u] = ok ? il[o] : 0.0;
     }
   };
   double cp = 0.0, dp = 0.0;
   fetch(0);
-  for (int k0 = 0; k0 < nz; k0 += kAhead) {
+  for (int t0 = 0; t0 < rows; t0 += kAhead) {
     double fc[kAhead], ic[kAhead];
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) {
       fc[u] = fv[u];
       ic[u] = KEPT ? iv[u] : 0.0;
     }
-    fetch(k0 + kAhead);
+    fetch(t0 + kAhead);
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) {
-      const int k = k0 + u;
-      if (k < nz) {
-        const double sub = ra(k);
+      const int k = first + dir * (t0 + u);
+      if (active && t0 + u < rows) {
+        const double sub = before(k);
         const double fo = is_null ? fc[u] - fshift : fc[u];
         const double rhs = fma(-sub, dp, fo);
         if (!KEPT) {
           ic[u] = recip_fp64(fma(-sub, cp, rb(k) + shift));
-          if (is_null && k == nz - 1) ic[u] = 0.0;   // vanishing final pivot: the modal unknown is set to zero
-          cp = rc(k) * ic[u];
+          if (!SPLIT && is_null && k == nz - 1) ic[u] = 0.0;   // vanishing final pivot
           il[k * lines] = ic[u];
         }
+        if (!KEPT || (SPLIT && t0 + u == rows - 1)) cp = after(k) * ic[u];
         dp = rhs * ic[u];
         ol[k * lines] = dp;
       }
     }
   }
-  // back substitution x_k = d'_k - c_k inv_k x_{k+1}, from the last row up
+  // x_{h-1} = d' - c' x_h from above, x_h = d'' - c'' x_{h-1} from below
+  if (SPLIT) {
+    meet[threadIdx.y][0][threadIdx.x] = cp;
+    meet[threadIdx.y][1][threadIdx.x] = dp;
+    __syncthreads();
+  }
   double x = dp;
-  auto fetch_back = [&](int k0) {
+  if (SPLIT) {
+    const double co = meet[1 - threadIdx.y][0][threadIdx.x], dn = meet[1 - threadIdx.y][1][threadIdx.x];
+    if (is_null) x = lower ? 0.0 : dp;               // the determinant vanishes: x_h = 0
+    else if (active) x = fma(-cp, dn, dp) * recip_fp64(fma(-cp, co, 1.0));
+    if (active) ol[(first + dir * (rows - 1)) * lines] = x;
+  }
+  // back substitution x_k = d'_k - (after_k inv_k) x_next, outwards from the middle
+  auto fetch_back = [&](int t0) {
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) {
-      const int k = k0 - u;
-      fv[u] = k >= 0 ? ol[k * lines] : 0.0;
-      iv[u] = k >= 0 ? il[k * lines] : 0.0;
+      const bool ok = active && t0 - u >= 0;
+      const long long o = static_cast<long long>(first + dir * (t0 - u)) * lines;
+      fv[u] = ok ? ol[o] : 0.0;
+      iv[u] = ok ? il[o] : 0.0;
     }
   };
-  fetch_back(nz - 2);
-  for (int k0 = nz - 2; k0 >= 0; k0 -= kAhead) {
+  fetch_back(rows - 2);
+  for (int t0 = rows - 2; t0 >= 0; t0 -= kAhead) {
     double fc[kAhead], ic[kAhead];
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) {
       fc[u] = fv[u];
       ic[u] = iv[u];
     }
-    fetch_back(k0 - kAhead);
+    fetch_back(t0 - kAhead);
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) {
-      const int k = k0 - u;
-      if (k >= 0) {
-        x = fma(-(rc(k) * ic[u]), x, fc[u]);
+      const int k = first + dir * (t0 - u);
+      if (active && t0 - u >= 0) {
+        x = fma(-(after(k) * ic[u]), x, fc[u]);
         ol[k * lines] = x;
       }
     }
   }
-  if (is_null) {
-    double xs = 0.0, w = 0.0;
-    for (int k = 0; k < nz; ++k) {
-      xs = fma(dz[k], ol[k * lines], xs);
-      w += dz[k];
+  if (null_i >= 0) {
+    if (SPLIT) __syncthreads();                      // both halves of the null line are in place
+    if (is_null && !lower) {
+      double xs = 0.0, w = 0.0;
+      for (int k = 0; k < nz; ++k) {
+        xs = fma(dz[k], ol[k * lines], xs);
+        w += dz[k];
+      }
+      const double mean = xs / w;
+      for (int k = 0; k < nz; ++k) ol[k * lines] -= mean;
     }
-    const double mean = xs / w;
-    for (int k = 0; k < nz; ++k) ol[k * lines] -= mean;
   }
 }
 
@@ -521,7 +554,11 @@ cudaError_t thomas_fp64(const tpt_plan_s* p, const double* fhat, double* phihat,
   const long long lines = static_cast<long long>(nx) * ny;
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->dev);
-  int bs = 128;
+  // Two threads a line up to 128 lines per SM, where the chain bounds the kernel
+  // (61x97x75 45 -> 27 us and 25 -> 20); above, the float64 pipe does and the extra
+  // operations of the meeting cost (a 256^3 Helmholtz solve 3.45 -> 3.54 ms).
+  const bool split = nz > 1 && lines <= 128LL * sms;
+  int bs = split ? 64 : 128;
   while (bs > 32 && lines < 2LL * sms * bs) bs /= 2;   // two blocks per SM, down to a warp
   const long long nb = (lines + bs - 1) / bs;
   const double* rz = p->d_rows[2];
@@ -530,9 +567,13 @@ cudaError_t thomas_fp64(const tpt_plan_s* p, const double* fhat, double* phihat,
   const size_t rows_bytes = 3 * static_cast<size_t>(nz) * sizeof(double);
   const bool rows = rows_bytes <= 48 * 1024;   // within the default dynamic limit
   note_launch();
-  auto kern = rows ? (kept ? thomas_fp64_kernel<true, true> : thomas_fp64_kernel<true, false>)
-                   : (kept ? thomas_fp64_kernel<false, true> : thomas_fp64_kernel<false, false>);
-  kern<<<static_cast<unsigned>(nb), bs, rows ? rows_bytes : 0, s>>>(
+  auto pick = [&](auto r, auto k) {
+    return split ? thomas_fp64_kernel<decltype(r)::value, decltype(k)::value, true>
+                 : thomas_fp64_kernel<decltype(r)::value, decltype(k)::value, false>;
+  };
+  auto kern = rows ? (kept ? pick(std::true_type{}, std::true_type{}) : pick(std::true_type{}, std::false_type{}))
+                   : (kept ? pick(std::false_type{}, std::true_type{}) : pick(std::false_type{}, std::false_type{}));
+  kern<<<static_cast<unsigned>(nb), dim3(bs, split ? 2 : 1), rows ? rows_bytes : 0, s>>>(
       nx, ny, nz, fhat, phihat, scratch, p->ddir[0].lam, p->ddir[1].lam, rz, rz + nz, rz + 2 * nz,
       p->d_dxf[2], p->alpha, p->beta, p->singular ? p->null_i : -1, p->singular ? p->null_j : -1,
       null_scale, p->singular ? defect : nullptr);
