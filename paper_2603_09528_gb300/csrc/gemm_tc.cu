@@ -10,8 +10,8 @@
 // 128 x BN tiles) with a double-buffered tensor-memory accumulator:
 //   warp 0      TMA producer: A and B tiles of 128-byte rows, 128-byte swizzle,
 //               into a ring of shared-memory stages (mbarrier full/empty);
-//   warp 1      allocates BN tensor-memory columns and issues tcgen05.mma from
-//               one thread, committing each stage back to the producer;
+//   warp 1      allocates the tensor-memory columns and issues tcgen05.mma from
+//               one lane, committing each stage back to the producer;
 //   warps 2..5  epilogue: tcgen05.ld 32 columns at a time, convert, and store
 //               with addresses idx(m, n) = (m % rm) + (m / rm) * sm + n * sn, so
 //               consecutive lanes (consecutive m) write consecutive addresses.
@@ -60,7 +60,8 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   e = (a - (s - bb)) + (b - bb);
 }
 
-template <int KIND, int NPL, int BN>
+// CG2: one CTA's share of a pair that runs each MMA together (PAIR 3): half of B.
+template <int KIND, int NPL, int BN, bool CG2 = false>
 struct Cfg {
   static constexpr int EB = (KIND == kKindBF16) ? 2 : 4;     // element bytes
   // bytes of a K-row of a stage: 64 (64-byte swizzle) for the split-bf16
@@ -69,9 +70,10 @@ struct Cfg {
   static constexpr int BK = SW / EB;                          // elements per row
   static constexpr int KI = (KIND == kKindBF16) ? 16 : 8;     // K of one MMA instruction
   static constexpr int A_BYTES = BM * SW;                     // one plane of A per stage
-  static constexpr int B_BYTES = BN * SW;
+  static constexpr int B_BYTES = (CG2 ? BN / 2 : BN) * SW;
   static constexpr int STAGE = NPL * (A_BYTES + B_BYTES);
-  static constexpr int STAGES = (kSmemBudget / STAGE) > 4 ? 4 : (kSmemBudget / STAGE);
+  static constexpr int MAX_STAGES = CG2 ? 6 : 4;
+  static constexpr int STAGES = (kSmemBudget / STAGE) > MAX_STAGES ? MAX_STAGES : (kSmemBudget / STAGE);
   static constexpr int TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;   // two accumulator buffers
   static constexpr int SMEM = STAGES * STAGE + 1024 /* alignment */ + 256 /* barriers */;
   // TMA-store epilogue: per epilogue warp two 32 x 32 chunks of up to 8 bytes
@@ -170,13 +172,14 @@ __device__ __forceinline__ void tile_coords(const GemmOut& g, int num_m, int num
 // Tile of work unit q for CTA rank r of a pair.  PAIR 0: one CTA per tile
 // (q is the tile).  PAIR 1: the two CTAs of a cluster take the m-tiles 2mp and
 // 2mp + 1 of one n-tile and share its B tile; PAIR 2: the n-tiles 2np and
-// 2np + 1 of one m-tile, sharing its A tile.
+// 2np + 1 of one m-tile, sharing its A tile; PAIR 3: the tiles of PAIR 1, each
+// MMA run by both CTAs together (cta_group::2: M = 256).
 template <int BN, int PAIR>
 __device__ __forceinline__ void unit_coords(const GemmOut& g, int num_m, int num_n, long long q, int r, int& m0,
                                             int& n0) {
   if (PAIR == 0) {
     tile_coords<BN>(g, num_m, num_n, q, m0, n0);
-  } else if (PAIR == 1) {
+  } else if (PAIR == 1 || PAIR == 3) {
     const int num_mp = num_m / 2;
     const int nt = static_cast<int>(g.n_fastest ? q % num_n : q / num_mp);
     const int mp = static_cast<int>(g.n_fastest ? q / num_n : q % num_mp);
@@ -210,7 +213,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
                const GemmOut g, const GemmJob* __restrict__ jobs, int njobs, long long total_units) {
   static_assert(!MULTI || PAIR == 0, "grouped launches run one CTA per tile");
   if (!MULTI && g.skip && *g.skip) return;   // uniform over the grid: no barrier or TMEM is touched
-  using C = Cfg<KIND, NPL, BN>;
+  constexpr bool CG2 = PAIR == 3;
+  static_assert(!CG2 || KIND == kKindBF16, "pair MMAs are bf16");
+  using C = Cfg<KIND, NPL, BN, CG2>;
   static_assert(C::STAGES >= 2, "shared-memory ring needs two stages");
   extern __shared__ __align__(128) uint8_t smem_raw[];
   // 1024-byte aligned start, offset on the shared pointer itself so that the
@@ -271,18 +276,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
     for (int s = 0; s < C::STAGES; ++s) {
       ptx::mbar_init(ptx::smem_u32(&bars[s]), 1);
       // a stage is free once the MMA of every CTA that reads it has finished
-      ptx::mbar_init(ptx::smem_u32(&bars[C::STAGES + s]), PAIR ? 2 : 1);
+      // (CG2: one MMA for both CTAs)
+      ptx::mbar_init(ptx::smem_u32(&bars[C::STAGES + s]), PAIR && !CG2 ? 2 : 1);
     }
     for (int b = 0; b < 2; ++b) {
       ptx::mbar_init(ptx::smem_u32(&accf[b]), 1);
-      ptx::mbar_init(ptx::smem_u32(&acce[b]), EPI);
+      ptx::mbar_init(ptx::smem_u32(&acce[b]), CG2 ? 2 * EPI : EPI);
     }
     ptx::mbar_init(ptx::smem_u32(mdone), 1);
     ptx::fence_mbar_init();
   }
   if (warp == 1) {
-    ptx::tmem_alloc(ptx::smem_u32(tmem_slot), C::TMEM_COLS);
-    ptx::tmem_relinquish();
+    if (CG2) {
+      ptx::tmem_alloc2(ptx::smem_u32(tmem_slot), C::TMEM_COLS);
+      ptx::tmem_relinquish2();
+    } else {
+      ptx::tmem_alloc(ptx::smem_u32(tmem_slot), C::TMEM_COLS);
+      ptx::tmem_relinquish();
+    }
   }
   ptx::tc_fence_before();
   __syncthreads();
@@ -328,7 +339,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
         }
         uint8_t* st = smem + s * C::STAGE;
         const uint32_t full = ptx::smem_u32(&bars[s]);
-        ptx::mbar_arrive_expect_tx(full, C::STAGE);
+        if (!CG2) ptx::mbar_arrive_expect_tx(full, C::STAGE);
+        else if (rank == 0) ptx::mbar_arrive_expect_tx(full, 2 * C::STAGE);
         const int kx = kc * C::BK;
         if (PAIR == 1) {          // own A; half of the shared B tile, to both CTAs
           const int hb = BN / 2;
@@ -349,6 +361,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
                                 kPairMask);
             ptx::tma_load_2d(ptx::smem_u32(st + NPL * C::A_BYTES + C::B_BYTES), mB1, full, kx, n0);
           }
+        } else if (CG2) {         // own A, own half of B; the bytes count on the first CTA's barrier
+          const uint32_t pf = ptx::mapa(full, 0);
+          const int nb = n0 + rank * (BN / 2);
+          ptx::tma_load_2d_pair(ptx::smem_u32(st), mA0, pf, kx, m0);
+          ptx::tma_load_2d_pair(ptx::smem_u32(st + NPL * C::A_BYTES), mB0, pf, kx, nb);
+          if (NPL == 2) {
+            ptx::tma_load_2d_pair(ptx::smem_u32(st + C::A_BYTES), mA1, pf, kx, m0);
+            ptx::tma_load_2d_pair(ptx::smem_u32(st + NPL * C::A_BYTES + C::B_BYTES), mB1, pf, kx, nb);
+          }
         } else {
           ptx::tma_load_2d(ptx::smem_u32(st), mA0, full, kx, m0);
           ptx::tma_load_2d(ptx::smem_u32(st + NPL * C::A_BYTES), mB0, full, kx, n0);
@@ -362,18 +383,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
     // drain: every issued stage's copies have landed before the CTA may exit
     // (the same bound as the main waits; a timed-out drain is recorded in
     // g.err, and every caller then treats the output as invalid)
+    // A pair's second CTA has no barrier of its own copies: when the loop ended
+    // early it leaves them two milliseconds.
     const long long first = it > C::STAGES ? it - C::STAGES : 0;
+    if (CG2 && rank == 1) {
+      if (!ok || stop)
+        for (int t = 0; t < 2000; ++t) __nanosleep(1000);
+    } else
     for (long long k = first; k < it; ++k)
       ptx::mbar_wait(ptx::smem_u32(&bars[k % C::STAGES]), static_cast<uint32_t>((k / C::STAGES) & 1), last_err,
                      ptx::kErrWaitDrain, polls);
-  } else if (warp == 1) {
+  } else if (warp == 1 && !(CG2 && rank == 1)) {   // a pair's MMAs are issued by its first CTA
     // -------------------------------------------------------- MMA issuer
     // The whole warp runs the loop and one elected lane issues, so that
     // descriptors and barrier addresses stay in uniform registers: a lone
     // thread building them took ~170 cycles per MMA, more than the 128 of the
     // MMA itself (128 x 256 x 16).  512^3: x forward 0.294 -> 0.248 ms, y
     // forward 0.295 -> 0.260, x inverse 0.434 -> 0.354.
-    constexpr uint32_t idesc = ptx::instr_desc(KIND == kKindBF16 ? 1u : 2u, BM, BN);
+    constexpr uint32_t idesc = ptx::instr_desc(KIND == kKindBF16 ? 1u : 2u, CG2 ? 2 * BM : BM, BN);
     const uint32_t issue = ptx::elect_one();
     const uint64_t desc0 = ptx::smem_desc_k_sw<C::SW>(ptx::smem_u32(smem));
     const uint32_t bar0 = ptx::smem_u32(bars);
@@ -393,9 +420,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
       const uint32_t b = tcount & 1;
       const int use = tcount >> 1;
       ++tcount;
-      if (use > 0)
-        ok = ptx::mbar_wait_warp(bar0 + 8 * (2 * C::STAGES + 2 + b), static_cast<uint32_t>((use - 1) & 1), last_err,
-                                 ptx::kErrWaitAccum, polls);
+      if (use > 0) {
+        const uint32_t drained = bar0 + 8 * (2 * C::STAGES + 2 + b), dpar = static_cast<uint32_t>((use - 1) & 1);
+        ok = CG2 ? ptx::mbar_wait_warp_cluster(drained, dpar, last_err, ptx::kErrWaitAccum, polls)
+                 : ptx::mbar_wait_warp(drained, dpar, last_err, ptx::kErrWaitAccum, polls);
+      }
       if (!ok) break;
       ptx::tc_fence_after();
       const uint32_t d = tmem + b * BN;
@@ -413,23 +442,28 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
             const uint64_t pa = da + (p == 2 ? C::A_BYTES >> 4 : 0) + off;
             const uint64_t pb = db + (p == 1 ? C::B_BYTES >> 4 : 0) + off;
             const uint32_t acc = (kc > 0 || kk > 0 || p > 0) ? 1u : 0u;
-            if (KIND == kKindBF16) ptx::mma_bf16_if(issue, d, pa, pb, idesc, acc);
+            if (CG2) ptx::mma_bf16_pair_if(issue, d, pa, pb, idesc, acc);
+            else if (KIND == kKindBF16) ptx::mma_bf16_if(issue, d, pa, pb, idesc, acc);
             else ptx::mma_tf32_if(issue, d, pa, pb, idesc, acc);
           }
         }
         const uint32_t freed = bar0 + 8 * (C::STAGES + s);
-        if (PAIR) ptx::mma_commit_mc_if(issue, freed, kPairMask);   // frees the stage in both CTAs
+        if (CG2) ptx::mma_commit_pair_if(issue, freed, kPairMask);
+        else if (PAIR) ptx::mma_commit_mc_if(issue, freed, kPairMask);   // frees the stage in both CTAs
         else ptx::mma_commit_if(issue, freed);
         if (++s == C::STAGES) {
           s = 0;
           par ^= 1;
         }
       }
-      ptx::mma_commit_if(issue, bar0 + 8 * (2 * C::STAGES + b));   // accumulator b ready
+      const uint32_t ready = bar0 + 8 * (2 * C::STAGES + b);   // accumulator b
+      if (CG2) ptx::mma_commit_pair_if(issue, ready, kPairMask);
+      else ptx::mma_commit_if(issue, ready);
     }
     // every MMA this warp issued has completed before the tensor memory is
     // freed, also when a timed-out wait ended the loop early
-    ptx::mma_commit_if(issue, ptx::smem_u32(mdone));
+    if (CG2) ptx::mma_commit_pair_if(issue, ptx::smem_u32(mdone), 0x1);
+    else ptx::mma_commit_if(issue, ptx::smem_u32(mdone));
     ptx::mbar_wait_warp(ptx::smem_u32(mdone), 0u, last_err, ptx::kErrWaitDrain, polls);
   } else if (warp >= 2) {
     // ---------------------------------------------------------- epilogue
@@ -517,14 +551,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
       }
       ptx::tc_fence_before();
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(ptx::smem_u32(&acce[b]));   // buffer b may be refilled
+      if (lane == 0) {   // buffer b may be refilled (CG2: by the pair's first CTA)
+        if (CG2) ptx::mbar_arrive_cluster(ptx::mapa(ptx::smem_u32(&acce[b]), 0));
+        else ptx::mbar_arrive(ptx::smem_u32(&acce[b]));
+      }
     }
     if (TMAO && lane == 0) ptx::bulk_wait_all();   // staging buffers stay until the stores are done
   }
   ptx::tc_fence_before();
   __syncthreads();
   if (PAIR) ptx::cluster_sync();   // no CTA leaves while its peer may still signal it
-  if (warp == 1) ptx::tmem_dealloc(tmem, C::TMEM_COLS);
+  if (warp == 1) {
+    if (CG2) ptx::tmem_dealloc2(tmem, C::TMEM_COLS);
+    else ptx::tmem_dealloc(tmem, C::TMEM_COLS);
+  }
 }
 
 // ---------------------------------------------------------------- host side
@@ -587,7 +627,7 @@ bool make_out_map(CUtensorMap* map, void* base, int eb, const GemmOut& g) {
 
 template <int KIND, int NPL, int BN, int OUT, int PAIR, int TMAO = 0>
 cudaError_t launch(const Operand& A, const Operand& B, const GemmOut& g, cudaStream_t s) {
-  using C = Cfg<KIND, NPL, BN>;
+  using C = Cfg<KIND, NPL, BN, PAIR == 3>;
   CUtensorMap m[6];
   std::memset(m, 0, sizeof(m));
   if (TMAO) {
@@ -602,7 +642,7 @@ cudaError_t launch(const Operand& A, const Operand& B, const GemmOut& g, cudaStr
     }
   }
   // the shared operand of a pair is loaded in halves (one per CTA)
-  const int a_rows = PAIR == 2 ? BM / 2 : BM, b_rows = PAIR == 1 ? BN / 2 : BN;
+  const int a_rows = PAIR == 2 ? BM / 2 : BM, b_rows = PAIR == 1 || PAIR == 3 ? BN / 2 : BN;
   if (!make_map(&m[0], A.plane[0], KIND, A.rows, A.K, A.ld, a_rows, C::SW)) return cudaErrorInvalidValue;
   if (!make_map(&m[2], B.plane[0], KIND, B.rows, B.K, B.ld, b_rows, C::SW)) return cudaErrorInvalidValue;
   if (NPL == 2) {
@@ -656,6 +696,23 @@ cudaError_t launch(const Operand& A, const Operand& B, const GemmOut& g, cudaStr
   return cudaGetLastError();
 }
 
+// Whether a GEMM without an operand-sharing mode runs its 256-column tiles as
+// pairs of CTAs (PAIR 3): half of B per CTA relieves the shared memory that the
+// operand loads, the MMAs and the output staging share (without loads the MMAs
+// run at their peak).  512^3, best mode before / pairs: x forward 0.262 / 0.250
+// ms, y forward 0.272 / 0.246, y inverse 0.260 / 0.247; at K = 256 the same
+// (256^3 y forward 33.2 / 32.5 us, x forward 37.7 / 38.4), with an odd number of
+// m-tiles slower (320^3 62 / 74), and so is the float-pair x inverse, which HBM
+// bounds (0.421 / 0.427).
+bool pair_mma(const GemmOut& g, int num_m, int num_n) {
+  if (g.pair != 0 || g.max_ctas > 0 || g.drop_loads || g.K < 384 || num_m % 2 != 0) return false;
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    cudaGetLastError();
+  return static_cast<long long>(num_m) * num_n >= 2LL * sms;   // two rounds of tiles
+}
+
 // Pair mode g.pair when it applies (split bf16 operands, 128- or 256-column
 // tiles, an even number of m-tiles (pair 1) or n-tiles (pair 2), an output
 // mode instantiated for it, and both operands in the current device's own
@@ -676,6 +733,8 @@ cudaError_t launch_pair(const Operand& A, const Operand& B, const GemmOut& g, cu
   constexpr bool can1 = NPL == 2 && BN >= 128 &&
                         (OUT == kOutSplitBF16 || OUT == kOutBF16 || OUT == kOutF32 || OUT == kOutF64);
   constexpr bool can2 = NPL == 2 && BN >= 128 && (OUT == kOutF32 || OUT == kOutDF || OUT == kOutF64);
+  constexpr bool can3 = KIND == kKindBF16 && NPL == 2 && BN == 256 &&
+                        (OUT == kOutSplitBF16 || OUT == kOutF32);
   // TMA-store epilogue when the output is a plain block of rows or whole
   // 32-row chunks of rm-row blocks
   constexpr bool cant = OUT == kOutSplitBF16 || OUT == kOutBF16 || OUT == kOutF32;
@@ -686,6 +745,9 @@ cudaError_t launch_pair(const Operand& A, const Operand& B, const GemmOut& g, cu
   if (g.pair == 2 && can2 && num_n % 2 == 0)
     return tma ? launch<KIND, NPL, BN, OUT, can2 ? 2 : 0, cant ? 1 : 0>(A, B, g, s)
                : launch<KIND, NPL, BN, OUT, can2 ? 2 : 0>(A, B, g, s);
+  if (can3 && pair_mma(g, num_m, num_n))
+    return tma ? launch<KIND, NPL, BN, OUT, can3 ? 3 : 0, cant ? 1 : 0>(A, B, g, s)
+               : launch<KIND, NPL, BN, OUT, can3 ? 3 : 0>(A, B, g, s);
   if (tma) return launch<KIND, NPL, BN, OUT, 0, cant ? 1 : 0>(A, B, g, s);
   return launch<KIND, NPL, BN, OUT, 0>(A, B, g, s);
 }
