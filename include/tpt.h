@@ -337,7 +337,8 @@ int tpt_plan_get_tiles(tpt_plan plan, int* tiles_out);
  * m-tiles share the B tile, 2 pairs of n-tiles share the A tile, through
  * TMA multicast in a cluster of two): chosen by tpt_plan_autotune, or set
  * here (each 0, 1 or 2, else INVALID_ARG; a mode that does not apply to a
- * GEMM falls back to one CTA per tile).                                     */
+ * GEMM falls back to 0).  With 0, split-bf16 GEMMs of at least 384 terms and
+ * two rounds of tiles run their MMAs over pairs of CTAs.                    */
 int tpt_plan_set_pairing(tpt_plan plan, const int* pairs);
 int tpt_plan_get_pairing(tpt_plan plan, int* pairs_out);
 

@@ -278,10 +278,11 @@ __device__ __forceinline__ double warp_sum(double v) {
 // read (SUMS).  Diagonals last: taken first they leave up to 1.4 times the
 // rounding error on noise.  With the terms summed before they leave f, the sums
 // always and each plane loaded when it is used, a 256^3 Poisson solve took
-// 3734 us (now 3655) and 512^3 33.5 ms (32.9).  The three diagonals are applied one by one: rounding their sum, the
-// same at every point of a uniform direction, shifted the refined solution by
-// eps times the condition number (6e-12 on 1024 uniform points).  sums[0] += sum r^2; with ALL also sums[1] += sum r and sums[2] +=
-// sum vol*r.
+// 3734 us (now 3655) and 512^3 33.5 ms (32.9).  The three diagonals are applied
+// one by one: rounding their sum, the same at every point of a uniform direction,
+// shifted the refined solution by eps times the condition number (6e-12 on 1024
+// uniform points).  sums[0] += sum r^2; with ALL also sums[1] += sum r and
+// sums[2] += sum vol*r.
 template <bool ROWS, bool SUMS, bool ALL>
 __global__ void __launch_bounds__(128)
 residual_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ f,

@@ -3073,9 +3073,9 @@ cudaError_t launch_output(const tpt_plan_s* p, const MixedWork& w, double* phi, 
 }
 
 // Adaptive refinement without a host round trip per correction: the
-// corrections and their residuals are enqueued back to back, each followed by
-// converge_kernel, whose flag makes the kernels of corrections past
-// convergence return at entry.  As many corrections as the plan's previous
+// corrections and their residuals are enqueued back to back, each ending with
+// the stopping test (converge_body), whose flag makes the kernels of corrections
+// past convergence return at entry.  As many corrections as the plan's previous
 // solve needed are enqueued first, with the output conversion behind them,
 // and the stream is synchronised once; should they not have converged, the
 // remaining corrections and the output conversion are enqueued again.
@@ -4036,7 +4036,7 @@ int autotune_gemms(tpt_plan_s* p, void* work, cudaStream_t s) {
 int mixed_info(const tpt_plan_s* p, const double* h, tpt_info* info) {
   int flags[2] = {0, 0};
   std::memcpy(flags, &h[8], sizeof(flags));
-  if (flags[1] > 0) {   // decided on the device (converge_kernel): its count and sums
+  if (flags[1] > 0) {   // decided on the device (converge_body): its count and sums
     const double rel = h[12] > 0.0 ? std::sqrt(h[11] / h[12]) : std::sqrt(h[11]);
     if (info) {
       std::memset(info, 0, sizeof(*info));

@@ -37,7 +37,8 @@ struct GemmOut {
   int bn = 0;       // column tile width 32/64/128/256; 0: chosen from M and N
   int max_ctas = 0; // cap on the persistent CTAs; 0 = one per SM
   int pair = 0;     // two-CTA clusters sharing an operand tile by TMA multicast:
-                    // 1 = pairs of m-tiles share B, 2 = pairs of n-tiles share A
+                    // 1 = pairs of m-tiles share B, 2 = pairs of n-tiles share A;
+                    // 0: none (large split-bf16 GEMMs run CTA pairs on one MMA)
   int tma_out = 1;  // TMA-store epilogue where the output layout allows (split bf16,
                     // bf16 or float32 out, 128/256-column tiles, one CTA per tile)
   const int* skip = nullptr;   // device flag: the kernel returns at entry when it is nonzero
