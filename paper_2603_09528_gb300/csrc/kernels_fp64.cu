@@ -119,6 +119,7 @@ __device__ __forceinline__ double recip_fp64(double m) {
 // small enough to reach every SM.  512^3 3.53 -> 2.73
 // ms, 1.31 with KEPT; 61x97x75 83 -> 27 and 20 us (SPLIT).
 constexpr int kAhead = 8;
+constexpr size_t kRowsSmem = 48 * 1024;   // largest z rows staged in shared memory (2048 points)
 template <bool ROWS, bool KEPT, bool SPLIT>
 __global__ void __launch_bounds__(128)
 thomas_fp64_kernel(int nx, int ny, int nz, const double* f, double* out,
@@ -580,7 +581,7 @@ cudaError_t thomas_fp64(const tpt_plan_s* p, const double* fhat, double* phihat,
   // f-hat of the null line equals (g_x g_y) times the physical constant
   const double null_scale = p->singular ? 1.0 / (p->null_g[0] * p->null_g[1]) : 0.0;
   const size_t rows_bytes = 3 * static_cast<size_t>(nz) * sizeof(double);
-  const bool rows = rows_bytes <= 48 * 1024;   // within the default dynamic limit
+  const bool rows = rows_bytes <= kRowsSmem;
   note_launch();
   auto pick = [&](auto r, auto k) {
     return split ? thomas_fp64_kernel<decltype(r)::value, decltype(k)::value, true>
@@ -588,6 +589,13 @@ cudaError_t thomas_fp64(const tpt_plan_s* p, const double* fhat, double* phihat,
   };
   auto kern = rows ? (kept ? pick(std::true_type{}, std::true_type{}) : pick(std::true_type{}, std::false_type{}))
                    : (kept ? pick(std::false_type{}, std::true_type{}) : pick(std::false_type{}, std::false_type{}));
+  if (rows && split) {
+    // without it static and dynamic memory together may take 48 KB, which the
+    // 2 KB of `meet` leave short of the rows from 1963 points on
+    const cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kRowsSmem));
+    if (e != cudaSuccess) return e;
+  }
   kern<<<static_cast<unsigned>(nb), dim3(bs, split ? 2 : 1), rows ? rows_bytes : 0, s>>>(
       nx, ny, nz, fhat, phihat, scratch, p->ddir[0].lam, p->ddir[1].lam, rz, rz + nz, rz + 2 * nz,
       p->d_dxf[2], p->alpha, p->beta, p->singular ? p->null_i : -1, p->singular ? p->null_j : -1,
@@ -611,7 +619,7 @@ cudaError_t residual_fp64(const tpt_plan_s* p, const double* f, const double* ph
   const int kseg = static_cast<int>((nz + segs - 1) / segs);
   grid.z = (nz + kseg - 1) / kseg;
   const size_t rows_bytes = 3 * static_cast<size_t>(nz) * sizeof(double);
-  const bool rows = rows_bytes <= 48 * 1024;   // within the default dynamic limit
+  const bool rows = rows_bytes <= kRowsSmem;   // within the default dynamic limit: no static memory here
   auto pick = [&](auto ro) {
     constexpr bool R = decltype(ro)::value;
     return !sums ? residual_fp64_kernel<R, false, false>
