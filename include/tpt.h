@@ -156,7 +156,9 @@ int tpt_workspace_bytes(tpt_plan plan, size_t* bytes);
  * NOT_CONVERGED (phi holds the last iterate), NONFINITE (a NaN or Inf in f
  * or in a residual; the float64 path reports it as a status when rtol > 0,
  * otherwise as a non-finite info->rel_residual once `stream` is
- * synchronised), TIMEOUT.                                                  */
+ * synchronised), TIMEOUT (a bounded device-side wait ran out; a float64 solve
+ * with rtol = 0 returns before it can know: phi then holds NaN and
+ * info->rel_residual is NaN).                                              */
 int tpt_solve(tpt_plan plan, const double* f_dev, double* phi_dev, void* work_dev,
               void* stream, tpt_info* info);
 
@@ -540,6 +542,12 @@ int tpt_test_fail_allocations(long long after);
  * context stays usable.  work_dev: at least 1 MiB of device scratch.  The
  * paper has no counterpart.                                                */
 int tpt_test_gemm_timeout(unsigned polls, void* work_dev, size_t work_bytes, void* stream);
+
+/* on = 1: from now on the tensor-core transforms in this float64 plan's
+ * solves issue no loads, with waits of about 0.1 ms: each runs out, sets the
+ * solve's flag and leaves NaN.  0 turns it off.  INVALID_ARG for a plan
+ * without such transforms.  The paper has no counterpart.                  */
+int tpt_test_transform_timeout(tpt_plan plan, int on);
 
 /* Name of a cudaError_t value as reported in tpt_result.cuda_error.        */
 const char* tpt_cuda_error_name(int cuda_error);

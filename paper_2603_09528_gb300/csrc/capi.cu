@@ -152,6 +152,9 @@ void CUDART_CB fill_info(void* arg) {
   cb->info->iters = cb->iters;
   cb->info->compat_defect = h[4];
   cb->info->rel_residual = (fn2 > 0.0) ? std::sqrt(h[1]) / std::sqrt(fn2) : std::sqrt(h[1]);
+  int gemm_err;   // a bounded GEMM wait ran out
+  std::memcpy(&gemm_err, h + 10, sizeof(gemm_err));
+  if (gemm_err) cb->info->rel_residual = NAN;
   delete cb;
 }
 
@@ -234,7 +237,7 @@ int fp64_solve(tpt_plan_s* p, const double* f, double* phi, void* work, cudaStre
       }
       double* slot = p->h_ring + static_cast<size_t>(p->ring_next) * kSlot;
       p->ring_next = (p->ring_next + 1) % kRingSlots;
-      TPT_CUDA(cudaMemcpyAsync(slot, ds, 8 * sizeof(double), cudaMemcpyDeviceToHost, s));
+      TPT_CUDA(cudaMemcpyAsync(slot, ds, kSlot * sizeof(double), cudaMemcpyDeviceToHost, s));
       InfoCallback* cb = new (std::nothrow) InfoCallback{info, slot, np, p->vol, iters, p->singular};
       if (!cb) return TPT_ERR_OOM;
       TPT_CUDA(cudaLaunchHostFunc(s, fill_info, cb));
@@ -439,6 +442,15 @@ int solve_enqueue(tpt_plan_s* p, const double* f, double* phi, void* work, cudaS
   return fp64_solve(p, f, phi, work, s, nullptr, true);
 }
 
+int fp64_wait_status(const tpt_plan_s* p, const void* work, cudaStream_t s) {
+  if (p->precision != TPT_PREC_FP64) return TPT_OK;
+  int gemm_err = 0;
+  TPT_CUDA(cudaMemcpyAsync(&gemm_err, static_cast<const double*>(work) + 10, sizeof(gemm_err),
+                           cudaMemcpyDeviceToHost, s));
+  TPT_CUDA(cudaStreamSynchronize(s));
+  return gemm_err ? TPT_ERR_TIMEOUT : TPT_OK;
+}
+
 int solve_info(const tpt_plan_s* p, const double* h, tpt_info* info) {
   if (p->precision != TPT_PREC_FP64) return mixed_info(p, h, info);
   const double np = static_cast<double>(npts(p));
@@ -493,6 +505,13 @@ int tpt_test_gemm_timeout(unsigned polls, void* work_dev, size_t work_bytes, voi
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return cuda_status(cudaGetLastError());
   return tpt::gemm_timeout_test(polls, work_dev, dev, static_cast<cudaStream_t>(stream));
+}
+
+int tpt_test_transform_timeout(tpt_plan p, int on) {
+  if (!on_device(p) || !(p->res[0].ready || p->res[1].ready)) return TPT_ERR_INVALID_ARG;
+  p->res_drop_loads = on != 0;
+  ++p->generation;   // recorded graphs hold the old setting
+  return TPT_OK;
 }
 
 const char* tpt_cuda_error_name(int cuda_error) {
@@ -697,6 +716,7 @@ int tpt_solve_host(tpt_plan p, const double* f_host, double* phi_host, double* f
   if (st != TPT_OK && st != TPT_ERR_NOT_CONVERGED) return st;
   TPT_CUDA(cudaMemcpyAsync(phi_host, phi_dev, bytes, cudaMemcpyDeviceToHost, s));
   TPT_CUDA(cudaStreamSynchronize(s));
+  TPT_TRY(tpt::fp64_wait_status(p, work, s));
   return st;
 }
 

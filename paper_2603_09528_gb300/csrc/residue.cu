@@ -305,7 +305,7 @@ struct RCfg {
   static constexpr int kABytes = BM * BK * 2, kStage = kABytes + BN * BK * 2;
   static constexpr int kStages = 192 * 1024 / kStage;
   static constexpr int kCols = 4 * BN / kEpiWarps;   // columns of an epilogue thread
-  static constexpr int kSmem = kStages * kStage + 1024 /* alignment */ + 256 /* barriers */;
+  static constexpr int kSmem = kStages * kStage + 1024 /* alignment */ + 384 /* barriers, left */;
 };
 
 // 2^k times the 64-bit integer F, rounded to nearest even
@@ -337,8 +337,11 @@ __device__ __forceinline__ double assemble(long long F, int k) {
 //              per element in registers over all moduli (sixteen warps: four a
 //              scheduler, and half the unrolled code of eight)
 // Element (m, n) is written (or added) at (m % rm) + (m / rm) sm + n sn.  Every
-// wait is bounded; a timeout sets bits in *err and the CTA drains and exits.
-template <int BN>
+// wait is bounded; a timeout sets bits in *err, and the CTA drains and exits with
+// NaN in the tiles that it has not finished, as do the CTAs that find the flag
+// set, so that no later kernel or caller takes stale memory for a result.
+// DROP: failure-detection test; the producer issues no loads, the waits are short.
+template <int BN, bool DROP = false>
 __global__ void __launch_bounds__(kThreads, 1)
 residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB,
                     const __grid_constant__ ResidueGemm g) {
@@ -351,10 +354,12 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constan
   uint64_t* acce = accf + kBufs;                // accumulator drained
   uint64_t* mdone = acce + kBufs;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mdone + 1);
+  long long* left = reinterpret_cast<long long*>(mdone + 2);   // an epilogue warp's first unfinished tile
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int num_m = (g.M + BM - 1) / BM, num_n = (g.N + BN - 1) / BN;
   const long long tiles = static_cast<long long>(num_m) * num_n;
   const int nk = g.Kp / BK;
+  constexpr uint32_t polls = DROP ? 1u << 10 : 1u << 22;
   // A timed-out CTA stops by its own bounded waits; the others look at the flag
   // once a tile, with the load in flight over the tile before (a load per ring
   // stage put ~700 cycles into the producer's loop).
@@ -377,6 +382,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constan
     }
     ptx::mbar_init(ptx::smem_u32(mdone), 1);
     ptx::fence_mbar_init();
+    for (int w = 0; w < kEpiWarps; ++w) left[w] = tiles;
   }
   if (warp == 1) {
     ptx::tmem_alloc(ptx::smem_u32(tmem_slot), kBufs * BN);
@@ -402,7 +408,8 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constan
         const long long round = it / kStages;
         if (round > 0)
           ok = ptx::mbar_wait(ptx::smem_u32(&bars[kStages + s]), static_cast<uint32_t>((round - 1) & 1), g.err,
-                              ptx::kErrWaitEmpty);
+                              ptx::kErrWaitEmpty, polls);
+        if (DROP) ok = false;
         if (!ok) break;
         uint8_t* st = smem + s * kStage;
         const uint32_t full = ptx::smem_u32(&bars[s]);
@@ -414,7 +421,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constan
     const long long first = it > kStages ? it - kStages : 0;
     for (long long k = first; k < it; ++k)   // every issued copy has landed before the CTA may exit
       ptx::mbar_wait(ptx::smem_u32(&bars[k % kStages]), static_cast<uint32_t>((k / kStages) & 1), g.err,
-                     ptx::kErrWaitDrain);
+                     ptx::kErrWaitDrain, polls);
   } else if (warp == 1) {
     // The whole warp runs the loop and one elected lane issues: descriptors and
     // barrier addresses stay in uniform registers (a lone thread building them
@@ -432,12 +439,12 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constan
       stop = aborted();
       for (int i = 0; i < g.nm && ok; ++i) {
         if (!first)
-          ok = ptx::mbar_wait_warp(bar0 + 8 * (2 * kStages + kBufs + b), bpar, g.err, ptx::kErrWaitAccum);
+          ok = ptx::mbar_wait_warp(bar0 + 8 * (2 * kStages + kBufs + b), bpar, g.err, ptx::kErrWaitAccum, polls);
         if (!ok) break;
         ptx::tc_fence_after();
         const uint32_t d = tmem + b * BN;
         for (int kc = 0; kc < nk; ++kc) {
-          ok = ptx::mbar_wait_warp(bar0 + 8 * s, par, g.err, ptx::kErrWaitFull);
+          ok = ptx::mbar_wait_warp(bar0 + 8 * s, par, g.err, ptx::kErrWaitFull, polls);
           if (!ok) break;
           ptx::tc_fence_after();
           const uint64_t da = desc0 + s * (kStage >> 4), db = da + (kABytes >> 4);
@@ -461,7 +468,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constan
     }
     // every MMA has completed before the tensor memory is freed
     ptx::mma_commit_if(issue, ptx::smem_u32(mdone));
-    ptx::mbar_wait_warp(ptx::smem_u32(mdone), 0u, g.err, ptx::kErrWaitDrain);
+    ptx::mbar_wait_warp(ptx::smem_u32(mdone), 0u, g.err, ptx::kErrWaitDrain, polls);
   } else if (warp >= 2) {
     const int quarter = warp % 4;                // tensor-memory lanes 32 * quarter ..
     const int col0 = ((warp - 2) / 4) * kCols;
@@ -469,10 +476,13 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constan
     long long t = 0;
     bool go = true;
     int stop = 0;
-    for (long long q = blockIdx.x; q < tiles && go; q += gridDim.x) {
+    for (long long q = blockIdx.x; q < tiles; q += gridDim.x) {
       int m0, n0;
       origin(q, m0, n0);
-      if (__any_sync(0xffffffffu, stop)) break;   // tcgen05.ld is warp-collective
+      if (__any_sync(0xffffffffu, stop)) {        // tcgen05.ld is warp-collective
+        if (lane == 0) left[warp - 2] = q;
+        break;
+      }
       stop = aborted();
       long long F[kCols];
 #pragma unroll
@@ -482,10 +492,10 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constan
         const bool two = 2 * j + 1 < g.nm;
         const int b0 = static_cast<int>(t % kBufs), b1 = static_cast<int>((t + 1) % kBufs);
         bool ok = ptx::mbar_wait(ptx::smem_u32(&accf[b0]), static_cast<uint32_t>((t / kBufs) & 1), g.err,
-                                 ptx::kErrWaitAccum);
+                                 ptx::kErrWaitAccum, polls);
         if (two && ok)
           ok = ptx::mbar_wait(ptx::smem_u32(&accf[b1]), static_cast<uint32_t>(((t + 1) / kBufs) & 1), g.err,
-                              ptx::kErrWaitAccum);
+                              ptx::kErrWaitAccum, polls);
         ptx::tc_fence_after();
         if (!__all_sync(0xffffffffu, ok)) {
           go = false;
@@ -527,7 +537,10 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constan
         }
         t += two ? 2 : 1;
       }
-      if (!go) break;
+      if (!go) {
+        if (lane == 0) left[warp - 2] = q;
+        break;
+      }
       const int m = m0 + quarter * 32 + lane;
       if (m < g.M) {
         const int ea = g.expA[m];
@@ -550,6 +563,19 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constan
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 1) ptx::tmem_dealloc(tmem, kBufs * BN);
+  // tiles given up after a timeout (here, where the epilogue's registers are free)
+  if (warp < 2) return;
+#pragma unroll 1
+  for (long long q = left[warp - 2]; q < tiles; q += gridDim.x) {
+    int m0, n0;
+    origin(q, m0, n0);
+    const int m = m0 + (warp % 4) * 32 + lane, n1 = n0 + ((warp - 2) / 4) * kCols;
+    if (m >= g.M) continue;
+    double* out = g.out + (m % g.rm) + static_cast<long long>(m / g.rm) * g.sm;
+#pragma unroll 1
+    for (int n = n1; n < min(g.N, n1 + kCols); ++n)
+      out[static_cast<long long>(n) * g.sn] = __longlong_as_double(0x7ff8000000000000ll);
+  }
 }
 
 // ------------------------------------------------------------------ host side
@@ -670,13 +696,14 @@ int tile_columns(int M, int N, int sms) {
   return best;
 }
 
-template <int BN>
+template <int BN, bool DROP = false>
 cudaError_t launch_gemm(const CUtensorMap& a, const CUtensorMap& b, const ResidueGemm& g, int sms, cudaStream_t s) {
-  const cudaError_t e = cudaFuncSetAttribute(residue_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const cudaError_t e = cudaFuncSetAttribute(residue_gemm_kernel<BN, DROP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              RCfg<BN>::kSmem);
   if (e != cudaSuccess) return e;
   const long long tiles = static_cast<long long>((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN);
-  residue_gemm_kernel<BN><<<static_cast<unsigned>(tiles < sms ? tiles : sms), kThreads, RCfg<BN>::kSmem, s>>>(a, b, g);
+  residue_gemm_kernel<BN, DROP>
+      <<<static_cast<unsigned>(tiles < sms ? tiles : sms), kThreads, RCfg<BN>::kSmem, s>>>(a, b, g);
   return cudaGetLastError();
 }
 
@@ -826,12 +853,13 @@ cudaError_t residue_transform(const tpt_plan_s* p, int d, bool inverse, const do
       g.expB = rd.expo[tab];
       g.n_fastest = 1;
     }
-    const int bn = tile_columns(g.M, g.N, sms);
+    const int bn = p->res_drop_loads ? 128 : tile_columns(g.M, g.N, sms);
     if (!tc::make_operand_map(&mat, rd.tab[tab], n, ld, ld, d == 0 ? BM : bn)) return cudaErrorInvalidValue;
     if (!tc::make_operand_map(&data, sl, lines, ld, ld, d == 0 ? bn : BM)) return cudaErrorInvalidValue;
     const CUtensorMap& ma = d == 0 ? mat : data;
     const CUtensorMap& mb = d == 0 ? data : mat;
-    e = bn == 128 ? launch_gemm<128>(ma, mb, g, sms, s) : bn == 64 ? launch_gemm<64>(ma, mb, g, sms, s)
+    e = p->res_drop_loads ? launch_gemm<128, true>(ma, mb, g, sms, s)
+        : bn == 128 ? launch_gemm<128>(ma, mb, g, sms, s) : bn == 64 ? launch_gemm<64>(ma, mb, g, sms, s)
                                                                    : launch_gemm<32>(ma, mb, g, sms, s);
     if (e != cudaSuccess) return e;
   }

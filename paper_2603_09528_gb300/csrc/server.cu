@@ -206,6 +206,10 @@ struct tpt_server_s {
         }
       }
     }
+    if (st == TPT_OK) {
+      *step = TPT_STEP_SOLVE;
+      st = tpt::fp64_wait_status(r->plan, aligned(buf[2]), s);
+    }
     for (void* b : buf)
       if (b) cudaFreeAsync(b, s);
     const int ss = cuda_st(cudaStreamSynchronize(s));

@@ -168,6 +168,7 @@ struct tpt_plan_s {
   // ready: the float64 DGEMM
   tpt::ResidueDir res[2];
   size_t res_cap = tpt::kResidueScratch;   // bytes of residues per pass
+  bool res_drop_loads = false;     // failure-detection test: their producers issue no loads
   bool ozaki = false;              // a TPT_PREC_FP64_OZAKI plan
   void* res_scratch = nullptr;     // scratch of an Ozaki plan's single-step transform entry point
   int stage_timing = 0;           // record per-stage CUDA events in tpt_solve
@@ -336,6 +337,11 @@ size_t residue_scratch_bytes(const tpt_plan_s* p);
 void residue_limit(tpt_plan_s* p, size_t bytes);
 cudaError_t residue_transform(const tpt_plan_s* p, int d, bool inverse, const double* in, double* out,
                               bool accumulate, void* scratch, int* err, cudaStream_t s);
+
+// After a float64 solve on workspace `work` and a synchronisation of s:
+// TPT_ERR_TIMEOUT when a bounded wait of its transforms ran out (the solution
+// then holds NaN), else TPT_OK.  Mixed plans report theirs themselves.
+int fp64_wait_status(const tpt_plan_s* p, const void* work, cudaStream_t s);
 
 // Times the transform GEMMs of a mixed plan over the candidate tiles and keeps
 // the fastest per stage (gemm_tune.cu).
