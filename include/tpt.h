@@ -543,6 +543,13 @@ int tpt_test_fail_allocations(long long after);
  * paper has no counterpart.                                                */
 int tpt_test_gemm_timeout(unsigned polls, void* work_dev, size_t work_bytes, void* stream);
 
+/* A split-bf16 transform GEMM whose MMAs run over pairs of CTAs, and in each
+ * pair CTA `rank` (0 or 1) stops loading after three stages: the waits run
+ * out (`polls` as above), the pair waits for the copies that it did issue and
+ * returns, and the call reports TPT_ERR_TIMEOUT.  work_dev: 256-byte aligned
+ * device scratch of at least 128 MiB.  The paper has no counterpart.       */
+int tpt_test_pair_timeout(unsigned polls, int rank, void* work_dev, size_t work_bytes, void* stream);
+
 /* on = 1: from now on the tensor-core transforms in this float64 plan's
  * solves issue no loads, with waits of about 0.1 ms: each runs out, sets the
  * solve's flag and leaves NaN.  0 turns it off.  INVALID_ARG for a plan

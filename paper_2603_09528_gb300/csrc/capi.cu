@@ -507,6 +507,13 @@ int tpt_test_gemm_timeout(unsigned polls, void* work_dev, size_t work_bytes, voi
   return tpt::gemm_timeout_test(polls, work_dev, dev, static_cast<cudaStream_t>(stream));
 }
 
+int tpt_test_pair_timeout(unsigned polls, int rank, void* work_dev, size_t work_bytes, void* stream) {
+  if (!work_dev || polls == 0 || rank < 0 || rank > 1) return TPT_ERR_INVALID_ARG;
+  if (reinterpret_cast<uintptr_t>(work_dev) % 256 != 0 || work_bytes < tpt::pair_timeout_bytes())
+    return TPT_ERR_INVALID_ARG;
+  return tpt::pair_timeout_test(polls, rank, work_dev, static_cast<cudaStream_t>(stream));
+}
+
 int tpt_test_transform_timeout(tpt_plan p, int on) {
   if (!on_device(p) || !(p->res[0].ready || p->res[1].ready)) return TPT_ERR_INVALID_ARG;
   p->res_drop_loads = on != 0;

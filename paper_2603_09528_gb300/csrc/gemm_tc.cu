@@ -242,6 +242,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
   uint64_t* acce = accf + 2;
   uint64_t* mdone = acce + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mdone + 1);
+  // CG2: what each CTA's producer issued, 2 * stages + (1: it stopped early)
+  unsigned long long* issued = reinterpret_cast<unsigned long long*>(mdone + 2);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int num_m = (g.M + BM - 1) / BM, num_n = (g.N + BN - 1) / BN;
@@ -346,7 +348,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
           ok = ptx::mbar_wait(ptx::smem_u32(&bars[C::STAGES + s]), static_cast<uint32_t>((round - 1) & 1), gq->err,
                               ptx::kErrWaitEmpty, polls);
         if (!ok) break;
-        if (g.drop_loads) {      // failure-detection test: no stage ever fills
+        // failure-detection tests: no stage ever fills, or one CTA of a pair stops after three
+        if (g.drop_loads == kDropAll || (CG2 && g.drop_loads == kDropPair0 + rank && it == 3)) {
           ok = false;
           break;
         }
@@ -396,13 +399,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
     // drain: every issued stage's copies have landed before the CTA may exit
     // (the same bound as the main waits; a timed-out drain is recorded in
     // g.err, and every caller then treats the output as invalid)
-    // A pair's second CTA has no barrier of its own copies: when the loop ended
-    // early it leaves them two milliseconds.
+    // A pair's copies all count on its first CTA's barriers; when a producer
+    // stopped early the two may have issued different stages, and the drain is
+    // the pair's (below), after both have said how many.
     const long long first = it > C::STAGES ? it - C::STAGES : 0;
-    if (CG2 && rank == 1) {
-      if (!ok || stop)
-        for (int t = 0; t < 2000; ++t) __nanosleep(1000);
-    } else
+    const bool early = !ok || stop;
+    if (CG2) {
+      const unsigned long long said = 2ull * static_cast<unsigned long long>(it) + (early ? 1 : 0);
+      issued[rank] = said;
+      ptx::st_cluster_u64(ptx::mapa(ptx::smem_u32(&issued[rank]), 1 - rank), said);
+    }
+    if (!CG2 || (rank == 0 && !early))
     for (long long k = first; k < it; ++k)
       ptx::mbar_wait(ptx::smem_u32(&bars[k % C::STAGES]), static_cast<uint32_t>((k / C::STAGES) & 1), last_err,
                      ptx::kErrWaitDrain, polls);
@@ -588,6 +595,25 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
   ptx::tc_fence_before();
   __syncthreads();
   if (PAIR) ptx::cluster_sync();   // no CTA leaves while its peer may still signal it
+  if (CG2 && ((issued[0] | issued[1]) & 1)) {   // the same in both CTAs
+    // Early exit: the first CTA waits for every copy that either issued.  A
+    // stage's phase completes with its own arrival and 2 * STAGE bytes; where
+    // only one CTA issued the stage, the other's half is taken out.  Neither is
+    // more than STAGES ahead (a stage is issued again only after the MMA that
+    // read both halves), so stages before `first` have landed.
+    if (rank == 0 && threadIdx.x == 0) {
+      const long long n0 = static_cast<long long>(issued[0] >> 1), n1 = static_cast<long long>(issued[1] >> 1);
+      const long long last = n0 > n1 ? n0 : n1;
+      for (long long k = last > C::STAGES ? last - C::STAGES : 0; k < last; ++k) {
+        const uint32_t full = ptx::smem_u32(&bars[k % C::STAGES]);
+        if (k >= n0) ptx::mbar_arrive_expect_tx(full, C::STAGE);
+        else if (k >= n1) ptx::mbar_complete_tx(full, C::STAGE);
+        ptx::mbar_wait(full, static_cast<uint32_t>((k / C::STAGES) & 1), g.err, ptx::kErrWaitDrain);
+      }
+    }
+    __syncthreads();
+    ptx::cluster_sync();
+  }
   if (warp == 1) {
     if (CG2) ptx::tmem_dealloc2(tmem, C::TMEM_COLS);
     else ptx::tmem_dealloc(tmem, C::TMEM_COLS);
@@ -732,7 +758,7 @@ cudaError_t launch(const Operand& A, const Operand& B, const GemmOut& g, cudaStr
 // m-tiles slower (320^3 62 / 74), and so is the float-pair x inverse, which HBM
 // bounds (0.421 / 0.427).
 bool pair_mma(const GemmOut& g, int num_m, int num_n) {
-  if (g.pair != 0 || g.max_ctas > 0 || g.drop_loads || g.K < 384 || num_m % 2 != 0) return false;
+  if (g.pair != 0 || g.max_ctas > 0 || g.drop_loads == kDropAll || g.K < 384 || num_m % 2 != 0) return false;
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)

@@ -4124,13 +4124,52 @@ int gemm_timeout_test(unsigned polls, void* work, int dev, cudaStream_t s) {
   MX_CUDA(cudaMemsetAsync(work, 0, 256, s));
   tc::GemmOut g = gout(M, N, K, kBig, 0, M, out, nullptr, tc::kOutF32, 0, 0, err);
   g.polls = polls;
-  g.drop_loads = 1;
+  g.drop_loads = tc::kDropAll;
   g.tma_out = 0;
   MX_CUDA(tc::gemm(tc::kKindBF16, 1, operand(pa, M, K, K), operand(pb, N, K, K), g, s));
   int h = 0;
   MX_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
   MX_CUDA(cudaStreamSynchronize(s));
   (void)dev;
+  return h ? TPT_ERR_TIMEOUT : TPT_OK;
+}
+
+namespace {
+constexpr int kPairTestM = 512, kPairTestK = 384;
+int pair_test_n() {   // two rounds of 128 x 256 tiles on every SM
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
+  return 2 * sm_count(dev) * 256 / (kPairTestM / 128);
+}
+}  // namespace
+
+size_t pair_timeout_bytes() {
+  const size_t n = pair_test_n();
+  return 256 + 2 * (align256(2 * kPairTestM * kPairTestK) + align256(2 * n * kPairTestK)) + 4 * n * kPairTestM;
+}
+
+int pair_timeout_test(unsigned polls, int rank, void* work, cudaStream_t s) {
+  const int M = kPairTestM, N = pair_test_n(), K = kPairTestK;
+  char* w = static_cast<char*>(work) + 256;
+  void *pa[2], *pb[2];
+  for (void** p : {&pa[0], &pa[1]}) {
+    *p = w;
+    w += align256(2 * static_cast<size_t>(M) * K);
+  }
+  for (void** p : {&pb[0], &pb[1]}) {
+    *p = w;
+    w += align256(2 * static_cast<size_t>(N) * K);
+  }
+  int* err = static_cast<int*>(work);
+  MX_CUDA(cudaMemsetAsync(work, 0, pair_timeout_bytes(), s));
+  tc::GemmOut g = gout(M, N, K, kBig, 0, M, w, nullptr, tc::kOutF32, 0, 0, err);
+  g.bn = 256;
+  g.polls = polls;
+  g.drop_loads = tc::kDropPair0 + rank;
+  MX_CUDA(tc::gemm(tc::kKindBF16, 2, operand(pa, M, K, K), operand(pb, N, K, K), g, s));
+  int h = 0;
+  MX_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+  MX_CUDA(cudaStreamSynchronize(s));
   return h ? TPT_ERR_TIMEOUT : TPT_OK;
 }
 

@@ -12,6 +12,9 @@ namespace tc {
 
 enum { kKindBF16 = 0, kKindTF32 = 1 };
 enum { kOutSplitBF16 = 0, kOutBF16 = 1, kOutF32 = 2, kOutF64 = 3, kOutDF = 4 };
+// failure-detection tests: no CTA loads anything, or CTA 0 (kDropPair0 + 1: CTA
+// 1) of each pair that runs its MMAs together stops after three stages
+enum { kDropAll = 1, kDropPair0 = 2 };
 
 // K-major operand: `rows` rows of K elements, row stride `ld` elements; one
 // plane, or a hi/lo pair of bf16 planes.  Base addresses 16-byte aligned and
@@ -46,7 +49,7 @@ struct GemmOut {
   // default, about 2^22) and a producer that issues no loads, so that the
   // waits run out and the kernel returns with TPT_ERR_TIMEOUT in *err.
   unsigned polls = 0;
-  int drop_loads = 0;
+  int drop_loads = 0;   // kDrop*
 };
 
 // One GEMM of a grouped launch: its tensor maps (A0, A1, B0, B1, O0, O1; the

@@ -285,6 +285,10 @@ int mixed_thomas_test(tpt_plan_s* p, const float* t2, void* t3_0, void* t3_1, vo
 // A transform GEMM whose producer issues no loads, with `polls` polls per
 // bounded wait: TPT_ERR_TIMEOUT when the waits ran out and said so.
 int gemm_timeout_test(unsigned polls, void* work, int dev, cudaStream_t s);
+// A split-bf16 GEMM on CTA pairs in each of which CTA `rank` stops loading after
+// three stages; work holds pair_timeout_bytes().
+size_t pair_timeout_bytes();
+int pair_timeout_test(unsigned polls, int rank, void* work, cudaStream_t s);
 int tc_gemm_test(int precision, int M, int N, int K, const double* A, const double* B, double* D,
                  void* work, int dev, cudaStream_t s, int tile = 0, int pair = 0);
 int tc_gemm_out_test(int precision, int M, int N, int K, const double* A, const double* B, int out_kind,
