@@ -270,19 +270,22 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 // r = (f - fshift) - (alpha phi + beta (Lx + Ly + Lz) phi); one thread per
 // (i, j) marching along kseg planes (blockIdx.z picks them).  End couplings of non-periodic directions are zero,
-// so wrapped neighbour indices only ever meet a zero coefficient.  The
-// beta-scaled rows are formed once (x and y per thread, z per block in shared
-// memory when ROWS, with alpha folded into the z diagonal), so that a point
-// costs six FMAs for the neighbours and three for the diagonals, all taken off f,
-// on GB300's float64 pipe (~1/64 of the float32 rate, the bound of this kernel),
-// one more for the shift of a singular problem and one for sum r^2 where it is
-// read (SUMS).  Diagonals last: taken first they leave up to 1.4 times the
-// rounding error on noise.  With the terms summed before they leave f, the sums
-// always and each plane loaded when it is used, a 256^3 Poisson solve took
-// 3734 us (now 3655) and 512^3 33.5 ms (32.9).  The three diagonals are applied
-// one by one: rounding their sum, the same at every point of a uniform direction,
-// shifted the refined solution by eps times the condition number (6e-12 on 1024
-// uniform points).  sums[0] += sum r^2; with ALL also sums[1] += sum r and
+// so wrapped neighbour indices only ever meet a zero coefficient.  The rows
+// of x and y are read once per thread, those of z once per block (shared memory
+// when ROWS).  A point costs nine operations for L phi and one to take beta L phi
+// off f on GB300's float64 pipe (~1/64 of the float32 rate, the bound of this
+// kernel), one more for alpha phi or for the shift of a singular problem, and one
+// for sum r^2 where it is read (SUMS).  A refined solution carries this kernel's
+// rounding, so the order is the one that leaves the smallest partial sums: each
+// direction's second difference complete before the next, its diagonal between its
+// neighbours, f last; and beta multiplies the sum, not the rows, whose rounding
+// would be the same at every refinement.  Error of a refined solve in the 2-norm,
+// 64^3 uniform points Helmholtz / Dirichlet Poisson / 96 x 100 x 40 stretched
+// Helmholtz: 1.4e-16 / 2.0e-16 / 2.2e-16; with beta-scaled rows, f first and the
+// diagonals last 3.3e-16 / 2.1e-15 / 5.5e-15 (one operation less, two for
+// Helmholtz: 256^3 Poisson 3657 us, this 3694); with the neighbours, one summed
+// diagonal, then f 2.6e-16 / 5.1e-16 / 4.5e-15.  The loads of a plane are issued
+// a plane ahead.  sums[0] += sum r^2; with ALL also sums[1] += sum r and
 // sums[2] += sum vol*r.
 template <bool ROWS, bool SUMS, bool ALL>
 __global__ void __launch_bounds__(128)
@@ -293,14 +296,14 @@ residual_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ f,
                      const double* __restrict__ dyf, const double* __restrict__ dzf,
                      double alpha, double beta, const double* __restrict__ fshift_p,
                      double* sums, int kseg) {
-  extern __shared__ double zrow[];   // beta a_k, beta b_k + alpha, beta c_k (ROWS)
+  extern __shared__ double zrow[];   // a_k, b_k, c_k (ROWS)
   const int k0 = blockIdx.z * kseg, k1 = min(nz, k0 + kseg);
   if (ROWS) {
     const int tid = threadIdx.x + blockDim.x * threadIdx.y, nt = blockDim.x * blockDim.y;
     for (int k = k0 + tid; k < k1; k += nt) {
-      zrow[k] = beta * rz[k];
-      zrow[nz + k] = fma(beta, rz[nz + k], alpha);
-      zrow[2 * nz + k] = beta * rz[2 * nz + k];
+      zrow[k] = rz[k];
+      zrow[nz + k] = rz[nz + k];
+      zrow[2 * nz + k] = rz[2 * nz + k];
     }
     __syncthreads();
   }
@@ -312,9 +315,8 @@ residual_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ f,
     const long long base = i + sy * j;
     const int im = (i == 0) ? nx - 1 : i - 1, ip = (i == nx - 1) ? 0 : i + 1;
     const int jm = (j == 0) ? ny - 1 : j - 1, jp = (j == ny - 1) ? 0 : j + 1;
-    const double ax = beta * rx[i], cx = beta * rx[2 * nx + i];
-    const double ay = beta * ry[j], cy = beta * ry[2 * ny + j];
-    const double bx = beta * rx[nx + i], by = beta * ry[ny + j];
+    const double ax = rx[i], bx = rx[nx + i], cx = rx[2 * nx + i];
+    const double ay = ry[j], by = ry[ny + j], cy = ry[2 * ny + j];
     const double fshift = fshift_p ? *fshift_p : 0.0;
     const double vxy = ALL ? dxf[i] * dyf[j] : 0.0;
     double pm = phi[base + sz * (k0 == 0 ? nz - 1 : k0 - 1)];   // k = 0: wrap partner, multiplied by a_0 = 0
@@ -332,19 +334,20 @@ residual_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ f,
       q += step;
       fn = *fq, nxm = q[xm], nxp = q[xp], nym = q[ym], nyp = q[yp];
       const double pp = phi[base + sz * ((k == nz - 1) ? 0 : k + 1)];
-      const double az = ROWS ? zrow[k] : beta * rz[k];
-      const double bz = ROWS ? zrow[nz + k] : fma(beta, rz[nz + k], alpha);
-      const double cz = ROWS ? zrow[2 * nz + k] : beta * rz[2 * nz + k];
-      double val = fshift_p ? fk - fshift : fk;
-      val = fma(-ax, vxm, val);
-      val = fma(-cx, vxp, val);
-      val = fma(-ay, vym, val);
-      val = fma(-cy, vyp, val);
-      val = fma(-az, pm, val);
-      val = fma(-cz, pp, val);
-      val = fma(-bx, p0, val);
-      val = fma(-by, p0, val);
-      val = fma(-bz, p0, val);
+      const double az = ROWS ? zrow[k] : rz[k];
+      const double bz = ROWS ? zrow[nz + k] : rz[nz + k];
+      const double cz = ROWS ? zrow[2 * nz + k] : rz[2 * nz + k];
+      double acc = ax * vxm;
+      acc = fma(bx, p0, acc);
+      acc = fma(cx, vxp, acc);
+      acc = fma(ay, vym, acc);
+      acc = fma(by, p0, acc);
+      acc = fma(cy, vyp, acc);
+      acc = fma(az, pm, acc);
+      acc = fma(bz, p0, acc);
+      acc = fma(cz, pp, acc);
+      const double rest = fshift_p ? fk - fshift : alpha != 0.0 ? fma(-alpha, p0, fk) : fk;
+      const double val = fma(-beta, acc, rest);
       r[o] = val;
       if (SUMS) s2 = fma(val, val, s2);
       if (ALL) {
