@@ -415,12 +415,16 @@ field_sums_kernel(int nx, int ny, long long lines, const double* __restrict__ f,
   }
 }
 
-// Canonical gauge (reading R4): the volume-weighted mean of phi to a few ulps
-// of the sum of |vol phi| whatever the cancellation, in two deterministic
-// levels: a warp sums an x-line with FMAs (Nx / 32 terms a lane) and the lines
-// with error-free additions (TwoSum), block partial sums as (hi, lo) pairs,
-// then one block over them.  (TwoSum at every point cost ten operations of the
-// float64 pipe: 512^3 2.21 ms, now 0.38.)
+// Canonical gauge (reading R4): the volume-weighted mean of phi to within 6 u of
+// the mean of |phi| (u = 2^-53), whatever the cancellation and the sizes, in two
+// deterministic levels.  A lane of the warp that sums an x-line takes its values
+// two at a time (two roundings) into a compensated sum (Kahan: 2 u of the sum of
+// magnitudes for any order and length); the lines, weighted by dy dz (two
+// roundings), meet in error-free additions (TwoSum) as (hi, lo) pairs per block,
+// then one block over them.  2.5 operations of the float64 pipe a point, which
+// bounds the kernel; TwoSum at every point, to 3 u, took nine (512^3 2.21 ms), a
+// plain FMA chain along the line, whose bound grows with Nx / 32, one (0.38; a
+// 512^3 solve 33.10 ms, this 33.46).
 __device__ __forceinline__ void two_sum_d(double a, double b, double& s, double& e) {
   s = a + b;
   const double bb = s - a;
@@ -441,13 +445,20 @@ wsum_partial_fp64_kernel(int nx, int ny, int nz, const double* __restrict__ phi,
   double hi = 0.0, lo = 0.0;
   for (long long L = blockIdx.x * 8LL + threadIdx.x / 32; L < lines; L += gridDim.x * 8LL) {   // x-line (j, k)
     const double* row = phi + static_cast<long long>(nx) * L;
-    double sl = 0.0;
-    for (int i = lane; i < nx; i += 32) sl = fma(dxf[i], row[i], sl);
-    const double v = (dyf[L % ny] * dzf[L / ny]) * sl;
+    double sl = 0.0, c = 0.0;            // the lane's share is sl - c
+#pragma unroll 4
+    for (int i = lane; i < nx; i += 64) {
+      double y = fma(dxf[i], row[i], -c);
+      if (i + 32 < nx) y = fma(dxf[i + 32], row[i + 32], y);
+      const double t = sl + y;
+      c = (t - sl) - y;
+      sl = t;
+    }
+    const double wyz = dyf[L % ny] * dzf[L / ny];
     double s, e;
-    two_sum_d(hi, v, s, e);
+    two_sum_d(hi, wyz * sl, s, e);
     hi = s;
-    lo += e;
+    lo += fma(-wyz, c, e);
   }
   __shared__ double sh[2][256];
   sh[0][threadIdx.x] = hi;
