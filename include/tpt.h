@@ -556,6 +556,11 @@ int tpt_test_pair_timeout(unsigned polls, int rank, void* work_dev, size_t work_
  * without such transforms.  The paper has no counterpart.                  */
 int tpt_test_transform_timeout(tpt_plan plan, int on);
 
+/* The moduli of the residue arithmetic behind the float64 transforms of
+ * contraction length K (1 to 2048, else INVALID_ARG), for tests: at most 18
+ * pairwise coprime integers.  Needs no device.                             */
+int tpt_test_residue_moduli(int K, int* moduli, int* count);
+
 /* Name of a cudaError_t value as reported in tpt_result.cuda_error.        */
 const char* tpt_cuda_error_name(int cuda_error);
 

@@ -127,6 +127,7 @@ SIGNATURES = [
     ("tpt_cuda_error_name", C.c_char_p, [C.c_int]),
     ("tpt_test_fail_allocations", C.c_int, [C.c_longlong]),
     ("tpt_test_gemm_timeout", C.c_int, [C.c_uint, C.c_void_p, C.c_size_t, C.c_void_p]),
+    ("tpt_test_residue_moduli", C.c_int, [C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_int)]),
     ("tpt_test_pair_timeout", C.c_int, [C.c_uint, C.c_int, C.c_void_p, C.c_size_t, C.c_void_p]),
     ("tpt_test_transform_timeout", C.c_int, [C.c_void_p, C.c_int]),
     ("tpt_set_stage_timing", C.c_int, [C.c_void_p, C.c_int]),

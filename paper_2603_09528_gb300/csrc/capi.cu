@@ -507,6 +507,14 @@ int tpt_test_gemm_timeout(unsigned polls, void* work_dev, size_t work_bytes, voi
   return tpt::gemm_timeout_test(polls, work_dev, dev, static_cast<cudaStream_t>(stream));
 }
 
+int tpt_test_residue_moduli(int K, int* moduli, int* count) {
+  tpt::ResidueSystem s;
+  if (!moduli || !count || !tpt::residue_system(K, &s)) return TPT_ERR_INVALID_ARG;
+  *count = s.nm;
+  for (int i = 0; i < s.nm; ++i) moduli[i] = s.p[i];
+  return TPT_OK;
+}
+
 int tpt_test_pair_timeout(unsigned polls, int rank, void* work_dev, size_t work_bytes, void* stream) {
   if (!work_dev || polls == 0 || rank < 0 || rank > 1) return TPT_ERR_INVALID_ARG;
   if (reinterpret_cast<uintptr_t>(work_dev) % 256 != 0 || work_bytes < tpt::pair_timeout_bytes())

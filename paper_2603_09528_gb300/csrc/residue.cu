@@ -9,7 +9,7 @@
 // row of the transform matrix.  For pairwise coprime moduli p_1 .. p_n with
 // product P, the integer product x = sum_k X_A X_B, |x| < P / 2, is fixed by
 // its residues, and each residue is one bf16 GEMM over centred residues
-// |r| <= rmax (exact in bf16 up to 256) with rmax^2 K <= 2^24, so that every
+// |r| <= 256 (exact in bf16) with max|r_A| max|r_B| K <= 2^24, so that every
 // partial sum is an integer below 2^24 and the float32 accumulator is exact in
 // any order.  With  K = 512: 14 moduli below 364 (P > 2^117); K <= 256: 13
 // below 514.  Summing slice products instead (Ozaki scheme I, eight 7-bit
@@ -38,9 +38,11 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 #include <cmath>
 #include <cstdint>
+#include <cstdlib>
 #include <cstring>
 #include <vector>
 
@@ -99,8 +101,8 @@ __device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
 // 2^(k + 14 j) mod p (|v| < 2^24, exact), r = v - p rint(v / p), stored as two
 // bf16 at dst + i * Kp for modulus i (and dst + 64 + i * Kp for the second pair
 // when `two`).  Paired float32 instructions, and the constants of a modulus
-// loaded once for both pairs; v / p is an odd multiple of 1/(2p) away from a tie
-// by more than the error of v * (1/p), so |r| <= p / 2 exactly.
+// loaded once for both pairs.  The rounded 1/p can take q past a tie for large v:
+// |r| is at most data_residue_max(p), p / 2 or one more.
 __device__ __forceinline__ void store_residues(const SliceConst& sc, int k, const float2 (&l)[2][4], bool two,
                                                __nv_bfloat16* dst, int Kp) {
   const float2 mg = both(kMagic), nmg = both(-kMagic);
@@ -589,6 +591,26 @@ int inverse_mod(int a, int p) {
   return 1;   // p == 1
 }
 
+// 2^bit mod p, centred.
+int centred_power(int bit, int p) {
+  const int v = static_cast<int>((1LL << bit) % p);
+  return 2 * v > p ? v - p : v;
+}
+
+// Largest |r| that store_residues leaves for modulus p: r = v - p rint(v inv) with
+// inv = (1 + d) / p, so |r| <= p / 2 + |v| |d|, |v| at most the digits' largest
+// magnitudes (2^13 three times and 2^15) times their constants'.
+int data_residue_max(int p) {
+  long long vmax = 0;
+  for (int k = 0; k <= kMaxUp; ++k) {
+    long long v = 0;
+    for (int j = 0; j < 4; ++j) v += (j < 3 ? 1LL << 13 : 1LL << 15) * std::abs(centred_power(k + 14 * j, p));
+    vmax = std::max(vmax, v);
+  }
+  const double d = static_cast<double>(1.0f / p) * p - 1.0;   // exact
+  return static_cast<int>(0.5 * p + static_cast<double>(vmax) * std::fabs(d));
+}
+
 }  // namespace
 
 bool residue_system(int K, ResidueSystem* s) {
@@ -604,6 +626,10 @@ bool residue_system(int K, ResidueSystem* s) {
     bool coprime = true;
     for (int i = 0; i < s->nm; ++i) coprime = coprime && gcd(p, s->p[i]) == 1;
     if (!coprime) continue;
+    // exact operands and sums, proven for this modulus (a residue one beyond p / 2
+    // is too much for p = 495 at K = 274 and p = 491 at K = 279 only)
+    const long long rdata = data_residue_max(p);
+    if (rdata > 256 || rdata * (p / 2) * K > (1LL << 24)) continue;
     s->p[s->nm++] = p;
     P *= static_cast<unsigned>(p);
     int L = 0;
@@ -638,10 +664,7 @@ SliceConst slice_const(const ResidueSystem& s) {
   c.L = s.L;
   for (int i = 0; i < s.nm; ++i) {
     const int p = s.p[i];
-    auto centred = [&](int bit) {
-      const long long v = (1LL << bit) % p;
-      return static_cast<float>(2 * v > p ? v - p : v);
-    };
+    auto centred = [&](int bit) { return static_cast<float>(centred_power(bit, p)); };
     for (int k = 0; k <= kMaxUp; ++k)
       c.c[k][i] = make_float4(centred(k), centred(k + 14), centred(k + 28), centred(k + 42));
     c.inv[i] = 1.0f / p;
