@@ -141,10 +141,11 @@ __device__ __forceinline__ void slice_line(const SliceConst& sc, int K, int Kp, 
   // |X_B| leaves free, by finer rounding and then by its residues' scale, so that
   // x keeps the resolution of the fraction F.  t sums an upper bound of
   // |x| / 2^(e - 20), from the leading 20 bits.
+  const int e1 = e == kRowNonFinite ? 0 : e + 1022;
   uint32_t t = 0;
   for (int k = lane; k < K; k += 32) {
     const uint32_t hi = static_cast<uint32_t>(get(k) >> 32);
-    const int d = e + 1022 - static_cast<int>((hi >> 20) & 0x7ff);
+    const int d = e1 - static_cast<int>((hi >> 20) & 0x7ff);
     t += d < 20 && d >= 0 ? ((0x100000u | (hi & 0xfffffu)) >> (d + 1)) + 1u : 1u;
   }
 #pragma unroll
@@ -525,9 +526,10 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constan
             for (int h = 0; h < 2; ++h) {
               const int ui = __float_as_int(h ? u.y : u.x);
               const uint32_t vi = __float_as_uint(h ? v.y : v.x);
-              long long w = static_cast<long long>(ui) * pr.clo + F[c0 + c + h];
-              w += static_cast<long long>(static_cast<unsigned long long>(static_cast<uint32_t>(ui * pr.chi)) << 32);
-              F[c0 + c + h] = w + vi;
+              const unsigned long long w =
+                  static_cast<unsigned long long>(static_cast<long long>(ui) * pr.clo) + F[c0 + c + h];
+              const unsigned long long wh = static_cast<uint32_t>(ui) * static_cast<uint32_t>(pr.chi);   // mod 2^32
+              F[c0 + c + h] = static_cast<long long>(w + (wh << 32) + vi);
             }
           }
         }
