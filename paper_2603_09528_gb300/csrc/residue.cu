@@ -61,22 +61,25 @@ constexpr uint32_t kMagicBits = 0x4B400000u;    // its bits; bits(kMagic + n) = 
 
 // ------------------------------------------------------------------ residues of the operands
 
-// The bits of a row's maximum |x| -> e with max < 2^e (0 for a zero or
-// subnormal row, kRowNonFinite when the row holds an infinity or a NaN).
+// The bits of a row's maximum |x| -> e with max < 2^e (0 for a zero row,
+// kRowNonFinite when the row holds an infinity or a NaN).
 constexpr int kRowNonFinite = INT_MAX;
 __device__ __forceinline__ int row_exponent(unsigned long long maxbits) {
   const int ex = static_cast<int>(maxbits >> 52);
-  return ex == 0x7ff ? kRowNonFinite : ex == 0 ? 0 : ex - 1022;
+  if (ex == 0x7ff) return kRowNonFinite;
+  return ex > 0 ? ex - 1022 : maxbits ? -1010 - __clzll(static_cast<long long>(maxbits)) : 0;
 }
 
-// X = round(x 2^(b - e)) for |x| < 2^e, from the bits of x (subnormal: 0).
+// X = round(x 2^(b - e)) for |x| < 2^e, from the bits of x.
 __device__ __forceinline__ long long fixed_point(unsigned long long bits, int e, int b) {
-  const int ex = static_cast<int>((bits >> 52) & 0x7ff);
-  const unsigned long long mant = (bits & ((1ull << 52) - 1)) | (1ull << 52);
+  int ex = static_cast<int>((bits >> 52) & 0x7ff);
+  unsigned long long mant = bits & ((1ull << 52) - 1);
+  if (ex) mant |= 1ull << 52;
+  else ex = 1;   // zero or subnormal
   const int sh = 1075 - b + e - ex;   // x = mant 2^(ex - 1075)
   long long X = sh <= 0 ? static_cast<long long>(mant << (-sh & 63))
                         : static_cast<long long>((mant + (1ull << ((sh - 1) & 63))) >> (sh & 63));
-  if (ex == 0 || sh > 54) X = 0;
+  if (sh > 54) X = 0;
   return static_cast<long long>(bits) < 0 ? -X : X;
 }
 
@@ -140,7 +143,9 @@ __device__ __forceinline__ void slice_line(const SliceConst& sc, int K, int Kp, 
   // far below K max|X_A| max|X_B|: it is scaled up by the 2^up that its sum of
   // |X_B| leaves free, by finer rounding and then by its residues' scale, so that
   // x keeps the resolution of the fraction F.  t sums an upper bound of
-  // |x| / 2^(e - 20), from the leading 20 bits.
+  // |x| / 2^(e - 20), from the leading 20 bits (a subnormal value's are below
+  // those of the smallest normal one, which is the bound it gets); a line of
+  // subnormal values alone stays as it is.
   const int e1 = e == kRowNonFinite ? 0 : e + 1022;
   uint32_t t = 0;
   for (int k = lane; k < K; k += 32) {
@@ -151,7 +156,7 @@ __device__ __forceinline__ void slice_line(const SliceConst& sc, int K, int Kp, 
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   int up = sc.L - 35 - sc.bits - (32 - __clz(static_cast<int>(t + 2u)));
-  up = up < 0 || e == kRowNonFinite ? 0 : up > kMaxUp ? kMaxUp : up;
+  up = up < 0 || e == kRowNonFinite || e1 < 1 ? 0 : up > kMaxUp ? kMaxUp : up;
   if (lane == 0) *expo = e == kRowNonFinite ? e : e - up;
   const int more = min(up, kMaxDataBits - sc.bits);   // as far as the digits reach, the line keeps more bits
   const int bits = sc.bits + more;
