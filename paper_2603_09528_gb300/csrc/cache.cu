@@ -333,6 +333,16 @@ int entry_mixed_tables(DirEntry& e, int fmt, int dev, void* q[2][2], float** lam
   return TPT_OK;
 }
 
+int entry_residue_tables(DirEntry& e, const DevDir& dd, int role, ResidueDir* out) {
+  std::lock_guard<std::mutex> g(e.mu);
+  if (!e.residue.ready) {
+    const int st = residue_tables(e.arena, e.n, dd, role, e.xform == TPT_XFORM_FFT, e.fft_kind, &e.residue);
+    if (st != TPT_OK) return st;
+  }
+  *out = e.residue;
+  return TPT_OK;
+}
+
 void BasisCache::trim() {
   std::lock_guard<std::mutex> g(mu_);
   for (;;) {

@@ -33,6 +33,7 @@ struct DirEntry {
   bool mixed_ready[3] = {false, false, false};
   void* q[3][2][2] = {};                 // [format][forward | inverse][plane]
   float* lam_f[3] = {nullptr, nullptr, nullptr};
+  ResidueDir residue;                    // residues of the float64 matrices (the same for x and y)
 };
 
 class BasisCache {
@@ -73,7 +74,12 @@ int create_plan(const tpt_desc* desc, int cuda_device, BasisCache* cache, tpt_pl
 // first use (mixed.cu calls this from the plan's mixed setup).
 int entry_mixed_tables(DirEntry& e, int fmt, int dev, void* q[2][2], float** lam_f);
 
-// Shared table builders (cache.cu, mixed.cu).
+// Residue tables of a cached direction, built on first use from the float64
+// operands dd of `role` (residue.cu calls this from the plan's setup).
+int entry_residue_tables(DirEntry& e, const DevDir& dd, int role, ResidueDir* out);
+
+// Shared table builders (cache.cu, mixed.cu, residue.cu).
+int residue_tables(DevArena& a, int n, const DevDir& dd, int role, bool fft, int kind, ResidueDir* out);
 int upload_fp64_basis(DevArena& a, const Eigen1D& e, const std::vector<double>& dxf, int role, DevDir* out);
 int upload_fft_tables(DevArena& a, int n, const Eigen1D& e, FftTables* t, double** lam);
 double null_fhat(const Dir1D& d, const Eigen1D& e, bool fft);

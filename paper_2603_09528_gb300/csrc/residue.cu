@@ -46,6 +46,7 @@
 #include <cstring>
 #include <vector>
 
+#include "cache.h"
 #include "ptx.h"
 #include "residue.h"
 #include "tc.h"
@@ -752,12 +753,11 @@ long long lines_per_pass(const tpt_plan_s* p, int d) {
 
 }  // namespace
 
-int residue_setup(tpt_plan_s* p, int d) {
-  const int n = p->n[d];
-  ResidueDir& rd = p->res[d];
+int residue_tables(DevArena& a, int n, const DevDir& dd, int role, bool fft, int kind, ResidueDir* out) {
+  ResidueDir rd;
   if (!residue_system(n, &rd.sys)) return TPT_ERR_UNSUPPORTED;
   rd.kp = (n + BK - 1) / BK * BK;
-  const size_t tab = static_cast<size_t>(n) * rd.sys.nm * rd.kp * 2;
+  const size_t tab = al256(static_cast<size_t>(n) * rd.sys.nm * rd.kp * 2), expo = al256(n * sizeof(int));
   MatrixConst mc;
   std::memset(&mc, 0, sizeof(mc));
   mc.nm = rd.sys.nm;
@@ -766,40 +766,48 @@ int residue_setup(tpt_plan_s* p, int d) {
     mc.p[i] = rd.sys.p[i];
     mc.y[i] = rd.sys.y[i];
   }
-  void* tab_d = nullptr;   // angles of a Fourier-transformed direction
-  std::vector<double> angles;
-  if (p->xform[d] == TPT_XFORM_FFT) {
+  std::vector<double> angles;   // of a Fourier-transformed direction
+  if (fft) {
     const long double pi2 = 6.283185307179586476925286766559005768L;
-    const int m = p->fft[d].kind == 1 ? 4 * n : n;
+    const int m = kind == 1 ? 4 * n : n;
     for (int k = 0; k < m; ++k) angles.push_back(static_cast<double>(std::cos(pi2 * k / m)));
-    if (p->fft[d].kind == 0)
+    if (kind == 0)
       for (int k = 0; k < n; ++k) angles.push_back(static_cast<double>(std::sin(pi2 * k / n)));
-    const int st = p->arena.upload(angles.data(), angles.size() * sizeof(double), &tab_d);
-    if (st != TPT_OK) return st;
   }
+  void* mem = nullptr;
+  const int st = a.alloc(2 * (tab + expo) + angles.size() * sizeof(double), &mem);
+  if (st != TPT_OK) return st;
+  char* w = static_cast<char*>(mem);
+  double* angles_d = reinterpret_cast<double*>(w + 2 * (tab + expo));
+  if (fft && cudaMemcpyAsync(angles_d, angles.data(), angles.size() * sizeof(double), cudaMemcpyHostToDevice,
+                             a.stream) != cudaSuccess)
+    return TPT_ERR_CUDA;
   for (int inv = 0; inv < 2; ++inv) {
-    void* t = nullptr;
-    int st = p->arena.alloc(al256(tab) + static_cast<size_t>(n) * sizeof(int), &t);
-    if (st != TPT_OK) return st;
-    rd.tab[inv] = t;
-    rd.expo[inv] = reinterpret_cast<int*>(static_cast<char*>(t) + al256(tab));
+    rd.tab[inv] = w + inv * (tab + expo);
+    rd.expo[inv] = reinterpret_cast<int*>(w + inv * (tab + expo) + tab);
+    __nv_bfloat16* t = static_cast<__nv_bfloat16*>(rd.tab[inv]);
     note_launch(1);
-    if (tab_d) {
-      const FourierRows rows{static_cast<const double*>(tab_d), n, p->fft[d].kind, inv};
-      matrix_residues_kernel<<<n, 256, 0, p->arena.stream>>>(n, rd.kp, rows, static_cast<__nv_bfloat16*>(t),
-                                                             rd.expo[inv], mc);
+    if (fft) {
+      const FourierRows rows{angles_d, n, kind, inv};
+      matrix_residues_kernel<<<n, 256, 0, a.stream>>>(n, rd.kp, rows, t, rd.expo[inv], mc);
     } else {
       // rows = output modes: x transforms read A[r][k] = mat[r + n k], y
       // transforms B[r][k] = mat[k + n r]
-      const DenseRows rows{inv ? p->ddir[d].inv : p->ddir[d].fwd, d == 0 ? 1 : n, d == 0 ? n : 1};
-      matrix_residues_kernel<<<n, 256, 0, p->arena.stream>>>(n, rd.kp, rows, static_cast<__nv_bfloat16*>(t),
-                                                             rd.expo[inv], mc);
+      const DenseRows rows{inv ? dd.inv : dd.fwd, role == 0 ? 1 : n, role == 0 ? n : 1};
+      matrix_residues_kernel<<<n, 256, 0, a.stream>>>(n, rd.kp, rows, t, rd.expo[inv], mc);
     }
     if (cudaGetLastError() != cudaSuccess) return TPT_ERR_CUDA;
   }
-  if (tab_d && cudaStreamSynchronize(p->arena.stream) != cudaSuccess) return TPT_ERR_CUDA;   // angles dies here
+  if (cudaStreamSynchronize(a.stream) != cudaSuccess) return TPT_ERR_CUDA;   // angles dies here; entries are shared
   rd.ready = true;
+  *out = rd;
   return TPT_OK;
+}
+
+int residue_setup(tpt_plan_s* p, int d) {
+  const bool fft = p->xform[d] == TPT_XFORM_FFT;
+  if (p->basis[d]) return entry_residue_tables(*p->basis[d], p->ddir[d], d, &p->res[d]);
+  return residue_tables(p->arena, p->n[d], p->ddir[d], d, fft, p->fft[d].kind, &p->res[d]);
 }
 
 size_t residue_scratch_bytes(const tpt_plan_s* p) {

@@ -330,8 +330,8 @@ int group_enqueue(GroupSolve* g, double* d_scal, cudaStream_t s);
 int group_solve_adaptive(GroupSolve* g, double* d_scal, double* h_scal, cudaStream_t s);
 
 // Float64 transforms by residue arithmetic on the tensor cores (residue.cu):
-// the tables of direction d (built on the plan's stream from the float64
-// matrices already on the device), the scratch of one transform, and the
+// the tables of direction d (built from the float64 matrices already on the
+// device, and shared by the plans of one cached direction), the scratch of one transform, and the
 // transform itself: out (+)= the transform of in.
 int residue_setup(tpt_plan_s* p, int d);
 size_t residue_scratch_bytes(const tpt_plan_s* p);
