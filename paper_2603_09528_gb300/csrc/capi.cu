@@ -389,6 +389,11 @@ int create_plan_impl(const tpt_desc* desc, int cuda_device, tpt::BasisCache* cac
     if (p->ozaki && gemm && p->n[d] > tpt::kOzakiMaxK) return fail(TPT_ERR_UNSUPPORTED);
     if (!(p->ozaki && gemm) && !residue_pays(p, d)) continue;
     st = tpt::residue_setup(p, d);
+    if (st == TPT_ERR_OOM && !p->ozaki) {   // no room for the tables: the transforms that need none
+      cudaGetLastError();
+      tpt::clear_cuda_error();
+      continue;
+    }
     if (st != TPT_OK) return fail(st);
   }
   if (cudaStreamSynchronize(p->arena.stream) != cudaSuccess) {
