@@ -143,6 +143,17 @@ int tpt_plan_create(const tpt_desc* desc, int cuda_device, tpt_plan* out);
 /* Bytes of device workspace tpt_solve() needs (256-byte aligned).          */
 int tpt_workspace_bytes(tpt_plan plan, size_t* bytes);
 
+/* Bring the scratch of a float64 plan's tensor-core transforms, which is part
+ * of its workspace (at most 512 MB, 0 for the other plans), down to `bytes`:
+ * the transforms then go in smaller passes over z, with the same results.
+ * Where `bytes` is less than one z plane takes, 0 above all, a TPT_PREC_FP64
+ * plan uses the float64 FMA GEMM and the FFT from then on, which need no
+ * scratch and whose operands keep all their bits element by element (an Ozaki
+ * plan keeps one plane's).  A limit above the present size changes nothing:
+ * a workspace sized before stays large enough.  Not to be called while a
+ * solve on this plan is in flight.                                         */
+int tpt_plan_limit_scratch(tpt_plan plan, size_t bytes);
+
 /* Solve (alpha I + beta L) phi = f.  f_dev and phi_dev hold Nx*Ny*Nz float64
  * (phi_dev may equal f_dev); work_dev holds tpt_workspace_bytes() bytes, is
  * 256-byte aligned and is not used concurrently by another call.  With
@@ -394,11 +405,12 @@ typedef struct tpt_batch_s* tpt_batch;
 int tpt_batch_create(const tpt_desc* descs, int count, int cuda_device, int nstreams, tpt_batch* out);
 
 /* Device workspace of one tpt_batch_solve (256-byte aligned): per capture
- * stream the largest tpt_workspace_bytes of its instances.                 */
+ * stream the largest tpt_workspace_bytes of its instances, as they are at this
+ * call (after tpt_plan_limit_scratch on instances: less).                  */
 int tpt_batch_workspace_bytes(tpt_batch batch, size_t* bytes);
 
 /* Borrowed handle of instance i (owned by the batch; valid until
- * tpt_batch_destroy).  Changing its coefficients or tiles makes the next
+ * tpt_batch_destroy).  Changing its coefficients, tiles or scratch makes the next
  * tpt_batch_solve recapture.                                                */
 int tpt_batch_plan(tpt_batch batch, int i, tpt_plan* out);
 

@@ -89,6 +89,23 @@ void release(tpt_batch b) {
   delete b;
 }
 
+// Places the capture streams' workspaces one after another; returns their sum.
+size_t layout(tpt_batch b) {
+  size_t total = 0;
+  b->lane_off.assign(b->lanes.size(), 0);
+  for (size_t k = 0; k < b->lanes.size(); ++k) {
+    size_t need = 256;
+    for (int i : b->lanes[k]) {
+      size_t w = 0;
+      tpt_workspace_bytes(b->plans[i], &w);
+      need = std::max(need, align256(w));
+    }
+    b->lane_off[k] = total;
+    total += need;
+  }
+  return total;
+}
+
 // Work estimate of one instance for the stream assignment: the transform
 // GEMMs dominate, 2 n_x n_y n_z (n_x + n_y) per correction.
 double cost_of(const tpt_plan_s* p) {
@@ -193,17 +210,7 @@ int tpt_batch_create(const tpt_desc* descs, int count, int cuda_device, int nstr
     b->lanes[k].push_back(i);
     load[k] += cost_of(b->plans[i]);
   }
-  b->lane_off.assign(lanes, 0);
-  for (int k = 0; k < lanes; ++k) {
-    size_t need = 256;
-    for (int i : b->lanes[k]) {
-      size_t w = 0;
-      tpt_workspace_bytes(b->plans[i], &w);
-      need = std::max(need, align256(w));
-    }
-    b->lane_off[k] = b->ws_bytes;
-    b->ws_bytes += need;
-  }
+  b->ws_bytes = layout(b);
   int st = TPT_OK;
   b->streams.assign(lanes, nullptr);
   b->joins.assign(lanes, nullptr);
@@ -256,6 +263,8 @@ int tpt_batch_get_grouped(tpt_batch b, int* grouped) {
 
 int tpt_batch_workspace_bytes(tpt_batch b, size_t* bytes) {
   if (!b || !bytes) return TPT_ERR_INVALID_ARG;
+  b->ws_streams = layout(b);
+  if (!b->grouped) b->ws_bytes = b->ws_streams;
   *bytes = b->ws_bytes;
   return TPT_OK;
 }

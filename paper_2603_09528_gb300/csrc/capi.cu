@@ -716,6 +716,12 @@ int tpt_workspace_bytes(tpt_plan p, size_t* bytes) {
   return TPT_OK;
 }
 
+int tpt_plan_limit_scratch(tpt_plan p, size_t bytes) {
+  if (!on_device(p)) return TPT_ERR_INVALID_ARG;
+  if (p->precision == TPT_PREC_FP64) tpt::residue_limit(p, bytes);
+  return TPT_OK;
+}
+
 int tpt_solve(tpt_plan p, const double* f, double* phi, void* work, void* stream, tpt_info* info) {
   if (!on_device(p) || !f || !phi || !work) return TPT_ERR_INVALID_ARG;
   if (reinterpret_cast<uintptr_t>(work) % 256 != 0) return TPT_ERR_INVALID_ARG;

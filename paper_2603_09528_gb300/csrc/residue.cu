@@ -822,9 +822,11 @@ size_t residue_scratch_bytes(const tpt_plan_s* p) {
 }
 
 void residue_limit(tpt_plan_s* p, size_t bytes) {
+  if (bytes >= residue_scratch_bytes(p)) return;
   p->res_cap = bytes;   // lines_per_pass leaves out the alignment of its two regions:
   if (residue_scratch_bytes(p) > bytes && bytes > 512) p->res_cap = bytes - 512;
   if (residue_scratch_bytes(p) > bytes && !p->ozaki) p->res[0].ready = p->res[1].ready = false;
+  ++p->generation;      // recorded graphs hold the old passes
 }
 
 cudaError_t residue_transform(const tpt_plan_s* p, int d, bool inverse, const double* in, double* out,

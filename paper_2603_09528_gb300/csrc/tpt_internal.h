@@ -335,9 +335,10 @@ int group_solve_adaptive(GroupSolve* g, double* d_scal, double* h_scal, cudaStre
 // transform itself: out (+)= the transform of in.
 int residue_setup(tpt_plan_s* p, int d);
 size_t residue_scratch_bytes(const tpt_plan_s* p);
-// Bring that scratch down to `bytes` (before the plan's workspace is sized):
-// smaller passes, down to one z plane; a FP64 plan for which that is still too
-// much takes the float64 FMA GEMM.
+// Bring that scratch down to `bytes`: smaller passes, down to one z plane; a FP64
+// plan for which that is still too much takes the float64 FMA GEMM and the FFT.  A
+// limit above the present size changes nothing, so that no workspace that was
+// sized before becomes too small.
 void residue_limit(tpt_plan_s* p, size_t bytes);
 cudaError_t residue_transform(const tpt_plan_s* p, int d, bool inverse, const double* in, double* out,
                               bool accumulate, void* scratch, int* err, cudaStream_t s);

@@ -127,12 +127,21 @@ class Plan:
     def _attach(self, h, n):
         self._h = h
         self.n = tuple(int(v) for v in n)
+        self._size_workspace()
+        self.npts = self.n[0] * self.n[1] * self.n[2]
+
+    def _size_workspace(self):
         nb = C.c_size_t()
         check(lib.tpt_workspace_bytes(self._h, C.byref(nb)), "tpt_workspace_bytes")
         self.workspace_bytes = int(nb.value)
-        self.npts = self.n[0] * self.n[1] * self.n[2]
 
     # ------------------------------------------------------------------
+    def limit_scratch(self, nbytes: int):
+        """tpt_plan_limit_scratch: a smaller workspace for a float64 plan; 0 also
+        keeps its transforms on the float64 FMA GEMM and the FFT."""
+        check(lib.tpt_plan_limit_scratch(self._h, int(nbytes)), "tpt_plan_limit_scratch")
+        self._size_workspace()
+
     def new_workspace(self) -> torch.Tensor:
         return torch.empty(self.workspace_bytes, dtype=torch.uint8, device="cuda:%d" % self.device)
 
@@ -400,14 +409,17 @@ class Batch:
               "tpt_batch_create")
         self._h = h
         del keep
-        nb = C.c_size_t()
-        check(lib.tpt_batch_workspace_bytes(self._h, C.byref(nb)), "tpt_batch_workspace_bytes")
-        self.workspace_bytes = int(nb.value)
+        self._size_workspace()
         self.plans = []
         for i, sp in enumerate(specs):
             ph = C.c_void_p()
             check(lib.tpt_batch_plan(self._h, i, C.byref(ph)), "tpt_batch_plan")
             self.plans.append(Plan.borrowed(ph, sp["n"], self.device))
+
+    def _size_workspace(self):
+        nb = C.c_size_t()
+        check(lib.tpt_batch_workspace_bytes(self._h, C.byref(nb)), "tpt_batch_workspace_bytes")
+        self.workspace_bytes = int(nb.value)
 
     def new_workspace(self) -> torch.Tensor:
         return torch.empty(self.workspace_bytes, dtype=torch.uint8, device="cuda:%d" % self.device)
@@ -422,9 +434,13 @@ class Batch:
         """tpt_batch_set_grouped: grouped launches (True) or capture streams
         (False); the workspace size follows the mode."""
         check(lib.tpt_batch_set_grouped(self._h, int(bool(on))), "tpt_batch_set_grouped")
-        nb = C.c_size_t()
-        check(lib.tpt_batch_workspace_bytes(self._h, C.byref(nb)), "tpt_batch_workspace_bytes")
-        self.workspace_bytes = int(nb.value)
+        self._size_workspace()
+
+    def limit_scratch(self, nbytes: int):
+        """Plan.limit_scratch of every instance; the batch's workspace follows."""
+        for p in self.plans:
+            p.limit_scratch(nbytes)
+        self._size_workspace()
 
     def autotune(self, work: torch.Tensor, stream=None):
         check(lib.tpt_batch_autotune(self._h, _ptr(work), _stream(stream)), "tpt_batch_autotune")
