@@ -19,7 +19,7 @@ namespace {
 // the process exits.
 constexpr unsigned long long kNoAllocMaxPoints = 1ull << 22;
 
-// c' of the forward elimination, one value per point.  Host code must not pass
+// Reciprocal pivots of the elimination, one value per point.  Host code must not pass
 // this name to a kernel: in host code it is a host-side stand-in, not a device
 // address.  The device address is taken once per device with
 // cudaGetSymbolAddress (noalloc_scratch below).
