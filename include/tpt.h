@@ -198,6 +198,12 @@ const char* tpt_status_string(int status);
 int tpt_transform(tpt_plan plan, int dir, int inverse, const double* in_dev, double* out_dev,
                   void* stream);
 
+/* The same as a float64 plan's solves run it, in a solve's workspace (work_dev as
+ * for tpt_solve): the tensor-core transforms where the plan has them.
+ * UNSUPPORTED for a mixed plan.                                             */
+int tpt_solve_transform(tpt_plan plan, int dir, int inverse, const double* in_dev, double* out_dev,
+                        void* work_dev, void* stream);
+
 /* Modal tridiagonal solve along z for every (i, j) (solution step 2.3):
  * (alpha + beta(lx_i + ly_j)) phi + beta T_z phi = fhat, float64, in place
  * allowed.  For a singular problem the null line is projected to compatible

@@ -99,6 +99,7 @@ class tpt_serving_stats(C.Structure):
 # (name, restype, argtypes) of every entry point declared in include/tpt.h
 SIGNATURES = [
     ("tpt_plan_create", C.c_int, [C.POINTER(tpt_desc), C.c_int, C.POINTER(C.c_void_p)]),
+    ("tpt_solve_transform", C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
     ("tpt_plan_limit_scratch", C.c_int, [C.c_void_p, C.c_size_t]),
     ("tpt_workspace_bytes", C.c_int, [C.c_void_p, C.POINTER(C.c_size_t)]),
     ("tpt_solve", C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,

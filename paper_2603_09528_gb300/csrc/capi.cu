@@ -756,6 +756,18 @@ int tpt_transform(tpt_plan p, int dir, int inverse, const double* in, double* ou
                          static_cast<cudaStream_t>(stream));
 }
 
+int tpt_solve_transform(tpt_plan p, int dir, int inverse, const double* in, double* out, void* work, void* stream) {
+  if (!on_device(p) || !in || !out || !work || in == out || (dir != 0 && dir != 1)) return TPT_ERR_INVALID_ARG;
+  if (reinterpret_cast<uintptr_t>(work) % 256 != 0) return TPT_ERR_INVALID_ARG;
+  if (p->precision != TPT_PREC_FP64) return TPT_ERR_UNSUPPORTED;
+  DeviceGuard guard(p->dev);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  double* ds = static_cast<double*>(work);   // as in fp64_solve: scalars, four regions, scratch
+  TPT_CUDA(cudaMemsetAsync(ds, 0, kSlot * sizeof(double), s));
+  return apply_transform(p, dir, inverse != 0, in, out, false, static_cast<char*>(work) + 256 + 4 * region_bytes(p),
+                         reinterpret_cast<int*>(ds + 10), s);
+}
+
 int tpt_thomas(tpt_plan p, const double* fhat, double* phihat, double* scratch, void* stream) {
   if (!on_device(p) || !fhat || !phihat || !scratch) return TPT_ERR_INVALID_ARG;
   DeviceGuard guard(p->dev);

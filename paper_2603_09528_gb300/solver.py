@@ -214,6 +214,13 @@ class Plan:
                                 _stream(stream)), "tpt_transform")
         return out
 
+    def solve_transform(self, x: torch.Tensor, direction: int, inverse: bool, work: torch.Tensor, out=None, stream=None):
+        """tpt_solve_transform: the transform as a float64 plan's solves run it."""
+        out = self.new_field() if out is None else out
+        check(lib.tpt_solve_transform(self._h, direction, int(inverse), _ptr(x), _ptr(out), _ptr(work),
+                                      _stream(stream)), "tpt_solve_transform")
+        return out
+
     def thomas(self, fhat: torch.Tensor, out=None, scratch=None, stream=None):
         out = self.new_field() if out is None else out
         scratch = self.new_field() if scratch is None else scratch

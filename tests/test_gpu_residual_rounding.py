@@ -3,7 +3,7 @@ every operation rounds once, so the error is at most u times the sum of the
 partial sums' magnitudes in the kernel's order, x- d x+ | y- d y+ | z- d z+, then
 f - alpha phi less beta times that.  On smooth fields those partial sums are small, and another order (f first,
 or the six neighbours before the diagonals) exceeds the bound many times.  Sizes:
-one block and several, several z segments, ragged edges."""
+one block and several, several z segments, ragged edges, z rows from memory."""
 import numpy as np
 import pytest
 
@@ -36,7 +36,7 @@ def _partials(f, phi, dirs, alpha, beta):
     return r, abs(beta) * total + (np.abs(rest) if alpha else 0.0) + np.abs(r)
 
 
-@pytest.mark.parametrize("n", [(64, 64, 64), (33, 6, 1), (1, 9, 50), (70, 45, 130)])
+@pytest.mark.parametrize("n", [(64, 64, 64), (33, 6, 1), (1, 9, 50), (70, 45, 130), (9, 5, 2100)])
 @pytest.mark.parametrize("kind", ["smooth", "noise"])
 @pytest.mark.parametrize("stretch", [0.0, 2.0])
 @pytest.mark.parametrize("alpha,beta", [(0.0, 1.0), (1.0, -5e-4)])

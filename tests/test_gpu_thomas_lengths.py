@@ -65,7 +65,7 @@ def test_lines_satisfy_their_rows(nz, lines, coef):
     assert (err <= tol).all(), (n, coef, float((err / tol).max()))
 
 
-@pytest.mark.parametrize("n", [(5, 7, 2), (30, 26, 3), (5, 7, 1963), (26, 30, 2048)])
+@pytest.mark.parametrize("n", [(5, 7, 2), (30, 26, 3), (5, 7, 1963), (26, 30, 2048), (5, 7, 2049)])
 def test_solves_with_kept_pivots_match_the_oracle(n):
     """Two corrections: the second reads the first one's pivots.  The coefficients
     keep the condition number below 100, so 1e-12 is 40 times eps cond."""
