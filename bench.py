@@ -1083,20 +1083,41 @@ def dominant_kernel(plan, prec, n, f_dev, steps, stream):
         pass
     out = plan.new_field()
     reps = max(3, steps)
-    plan.transform(f_dev, 0, False, out=out, stream=stream)
+    residues = prec == 0 and 24 <= n[0] <= 2048   # solves transform by residues on the tensor cores
+
+    def transform():
+        if residues:
+            plan.solve_transform(f_dev, 0, False, work, out=out, stream=stream)
+        else:
+            plan.transform(f_dev, 0, False, out=out, stream=stream)
+
+    work = plan.new_workspace() if residues else None
+    transform()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     torch.cuda.synchronize()
     e0.record(stream)
     for _ in range(reps):
-        plan.transform(f_dev, 0, False, out=out, stream=stream)
+        transform()
     e1.record(stream)
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / reps
     flops = 2.0 * n[0] * n[0] * n[1] * n[2]
     achieved = flops / (ms / 1e3) / 1e12
+    if residues:
+        import ctypes
+        from paper_2603_09528_gb300 import _lib
+        moduli, count = (ctypes.c_int * 18)(), ctypes.c_int()
+        if _lib.lib.tpt_test_residue_moduli(n[0], moduli, ctypes.byref(count)) != 0:
+            raise RuntimeError("no moduli for a transform of %d points" % n[0])
+        peak = peaks.get("bf16_tflops", 1900.0)
+        bf16 = achieved * count.value
+        return {"kernel": "slice_x_kernel + residue_gemm_kernel (x forward transform of a float64 solve, %d exact "
+                          "bf16 products)" % count.value, "bound": "tensor",
+                "achieved": bf16, "peak": peak, "unit": "TFLOP/s", "frac": bf16 / peak, "traffic": None,
+                "ms_per_launch": ms, "flops_per_launch": flops * count.value, "float64_tflops": achieved}
     if prec == 0:
         peak = 1.25   # GB300 float64 rate in TFLOP/s, nominal (an FMA counts two flops)
-        return {"kernel": "dgemm_cm_kernel (x forward transform by itself; solves transform 24 to 2048 points by residues)", "bound": "alu",
+        return {"kernel": "dgemm_cm_kernel (x forward transform)", "bound": "alu",
                 "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "peak_source": "nominal GB300 float64 rate (MEASURED_PEAKS.json has no float64 entry)",
                 "traffic": None, "ms_per_launch": ms, "flops_per_launch": flops}

@@ -88,8 +88,9 @@ enum { TPT_XFORM_AUTO = 0, TPT_XFORM_GEMM = 1, TPT_XFORM_FFT = 2 };
  * also in the single-step tpt_transform; GEMM directions of at most 576 points
  * (else UNSUPPORTED).  A FP64 plan runs the same transforms in its solves for
  * GEMM directions of 24 to 2048 points and, with the Fourier matrices, for FFT
- * directions of 32 to 1024 points; the float64 FMA GEMM and the FFT otherwise
- * and in tpt_transform.  Reported as TPT_PREC_FP64 by the plan's inspection calls. */
+ * directions of 32 to 1024 points; the float64 FMA GEMM and the FFT otherwise,
+ * after tpt_plan_limit_scratch(plan, 0) and in tpt_transform.  Reported as
+ * TPT_PREC_FP64 by the plan's inspection calls.                             */
 enum { TPT_PREC_FP64 = 0, TPT_PREC_MIXED_BF16 = 1, TPT_PREC_MIXED_BF16X3 = 2,
        TPT_PREC_MIXED_TF32 = 3, TPT_PREC_FP64_OZAKI = 4 };
 

@@ -508,7 +508,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ 
           mvalid ? (static_cast<long long>(m % gu.rm) + static_cast<long long>(m / gu.rm) * gu.sm) : 0;
       // Float pairs that are read: the lines of the warp's next chunk are asked
       // into L2 while this one is updated, which keeps twice the reads in flight
-      // (512^3 solve 7.16 -> 7.09 ms, 24 uneven instances 6.04 -> 5.99).  Measured
+      // (512^3, in turn: x inverse 0.417 -> 0.399 ms, solve 7.205 -> 7.170; 24 uneven
+      // instances 5.98 -> 5.93).  Measured
       // slower: the whole update without tests per column on paired float32
       // instructions (x inverse of 512^3 0.42 -> 0.55 ms).
       const bool ahead = OUT == kOutDF && acc_out && m0 + quarter * 32 < gu.M;
@@ -738,7 +739,9 @@ cudaError_t launch(const Operand& A, const Operand& B, const GemmOut& g, cudaStr
 // ms, y forward 0.272 / 0.246, y inverse 0.260 / 0.247; at K = 256 the same
 // (256^3 y forward 33.2 / 32.5 us, x forward 37.7 / 38.4), with an odd number of
 // m-tiles slower (320^3 62 / 74), and so is the float-pair x inverse, which HBM
-// bounds (0.421 / 0.427).
+// bounds (0.421 / 0.427).  Solves without / with pairs around the line: y of 320,
+// 352 and 384 points the same to 0.1 %, 392 1247 / 1155 us, 416 1123 / 1105, 448
+// 1165 / 1147.
 bool pair_mma(const GemmOut& g, int num_m, int num_n) {
   if (g.pair != 0 || g.max_ctas > 0 || g.drop_loads == kDropAll || g.K < 384 || num_m % 2 != 0) return false;
   int dev = 0, sms = 152;

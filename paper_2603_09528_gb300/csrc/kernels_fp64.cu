@@ -586,7 +586,9 @@ cudaError_t thomas_fp64(const tpt_plan_s* p, const double* fhat, double* phihat,
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->dev);
   // Two threads a line up to 128 lines per SM, where the chain bounds the kernel
   // (61x97x75 45 -> 27 us and 25 -> 20); above, the float64 pipe does and the extra
-  // operations of the meeting cost (a 256^3 Helmholtz solve 3.45 -> 3.54 ms).
+  // operations of the meeting cost (a 256^3 Helmholtz solve 3.45 -> 3.54 ms).  Solves
+  // of 128 rows, one thread / two: 84 lines per SM 556 / 518 us, 126 739 / 710, 129
+  // 852 / 845, 168 1111 / 1102, 263 and 431 the same.
   const bool split = nz > 1 && lines <= 128LL * sms;
   int bs = split ? 64 : 128;
   while (bs > 32 && lines < 2LL * sms * bs) bs /= 2;   // two blocks per SM, down to a warp

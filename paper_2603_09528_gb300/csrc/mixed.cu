@@ -1120,7 +1120,8 @@ __device__ __forceinline__ void converge_body(double* scal, double npts, double 
 
 // The stopping test as the last act of a residual: the warp that arrives last at
 // the counter (scal[13]) has every warp's share of sum r^2 before it.  scal null:
-// no test.
+// no test.  A block's last act, the fence, lengthens the 512^3 residual by 1.3 %
+// (0.658 -> 0.666 ms), about what the launch of its own that it replaces took.
 struct Conv {
   double* scal;
   double npts, vol, rtol;
@@ -2590,7 +2591,9 @@ cudaError_t launch_thomas2_nt(const tpt_plan_s* p, const MixedWork& w, cudaStrea
 // lines per thread (thomas2_kernel); `variant` 0 picks the two-line kernel above
 // 112 rows (per launch, one-line / two-line: 256^3 45.7 / 30.4 us, 150x277x133
 // 26.1 / 19.0, 128^3 11.2 / 10.1; 192x192x96 15.4 / 16.0, 300x200x40 15.4 /
-// 18.3).  Up to there a singular problem also keeps its null line off the
+// 18.3; solves around the line: 64x64x120 183 / 173 us, 256x256x113 564 / 535,
+// 512x512x116 2023 / 1911, and below it 64x64x104 178 / 170, 256x256x104 546 / 522,
+// 128x128x100 the same).  Up to there a singular problem also keeps its null line off the
 // block-wide scans of the two-line kernel.
 int thomas_variant(int nz, int variant) {
   if (variant == 1) return 1;

@@ -21,17 +21,21 @@
 // sum is kept as a 64-bit binary fraction F in registers, whose wrap-around is
 // the "mod 1".  Two moduli are taken together: n = r_i p_j + r_j p_i (exact in
 // float32), F += n C + rint(n e) with C + e = 2^64 / (p_i p_j).  F is off by at
-// most half a unit per pair, 2^-61 P in all, which is below 2^-54 of a typical
-// |x| even though |x| is ~2^-9.5 P.  The matrix is scaled by P / 2^L (L the bit
+// most half a unit per pair: 2^-61 P in all, 2^-64.4 P in the root mean square
+// (seven pairs).  A typical |x| is ~2^-9.5 P, of which that is 2^-51.5 at most and
+// 2^-54.9 typically: the size of one rounding.  The matrix is scaled by P / 2^L (L the bit
 // length of P) when it is rounded, so x = F 2^(L-64) times powers of two and the
 // result is assembled from its bits: no operation of the float64 pipe (1/64 of
 // the float32 rate on GB300) is spent on a point, except the sum of an
 // accumulating transform.  The rounding of the operands (2^-54 of a row's
-// maximum) is the whole error; the float64 FMA chain it replaces rounds at each
+// maximum, not of each value) and that of F are the whole error; the float64 FMA chain it replaces rounds at each
 // of the K steps (relative 2-norm error of one transform of noise, K = 512: 9e-17
-// against 7.5e-16; K = 64: 9e-17 against 2.6e-16).
+// against 7.5e-16; K = 64: 9e-17 against 2.6e-16).  In a solve the two cannot be
+// told apart element by element either, on grids stretched by 1.5 to 9 and for
+// right-hand sides of noise, smooth, with one huge value, or over twelve decades:
+// the float64 rounding of the eigenvectors themselves is larger.
 //
-// Measured (GB300, one transform of 512^3 points): 3.0 ms along x, 3.1 ms along
+// Measured (GB300, one transform of 512^3 points): 3.05 ms along x, 3.1 ms along
 // y (GEMM 2.0, slicing 1.0 and 1.1), where the float64 FMA GEMM, at that pipe's
 // peak, takes 109.7 ms; 256^3 0.30 ms against 6.9.
 #include <cuda.h>
