@@ -145,7 +145,8 @@ int tpt_plan_create(const tpt_desc* desc, int cuda_device, tpt_plan* out);
 int tpt_workspace_bytes(tpt_plan plan, size_t* bytes);
 
 /* Bring the scratch of a float64 plan's tensor-core transforms, which is part
- * of its workspace (at most 512 MB, 0 for the other plans), down to `bytes`:
+ * of its workspace (at most 512 MB, or one z plane's where that is more; 0
+ * for the other plans), down to `bytes`:
  * the transforms then go in smaller passes over z, with the same results.
  * Where `bytes` is less than one z plane takes, 0 above all, a TPT_PREC_FP64
  * plan uses the float64 FMA GEMM and the FFT from then on, which need no

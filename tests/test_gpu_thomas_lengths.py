@@ -39,16 +39,14 @@ def _rows(x, d, shift, beta):
     return a * lo + diag * x + c * up, abs(a * lo) + abs(diag * x) + abs(c * up)
 
 
-LINES = [(5, 7), (160, 125)]        # two threads a line; 20,000 lines: one
+# two threads a line, and 20,000 lines: one (which takes no static shared memory)
+SIZES = [(5, 7, nz) for nz in (1, 2, 3, 8, 9, 33, 1962, 1963, 2048, 2049)] + [(160, 125, nz) for nz in (1, 2, 3, 8, 9, 33)]
 
 
-@pytest.mark.parametrize("nz", [1, 2, 3, 8, 9, 33, 1962, 1963, 2048, 2049])
-@pytest.mark.parametrize("lines", LINES)
+@pytest.mark.parametrize("n", SIZES)
 @pytest.mark.parametrize("coef", [(0.0, 1.0), (1.0, -5e-4)])
-def test_lines_satisfy_their_rows(nz, lines, coef):
-    if nz > 100 and lines == LINES[1]:
-        pytest.skip("one thread a line takes no static shared memory")
-    n = lines + (nz,)
+def test_lines_satisfy_their_rows(n, coef):
+    nz = n[2]
     dirs, plan = _plan(n, *coef)
     f = S.uniform_rhs(n, 21)
     x = tpt.field_to_host(plan.thomas(tpt.field_to_device(f)), n)
