@@ -90,9 +90,11 @@ void release(tpt_batch b) {
 }
 
 // Places the capture streams' workspaces one after another; returns their sum.
+// Where nothing has changed it writes nothing, so that asking for the size stays
+// safe beside a solve.
 size_t layout(tpt_batch b) {
   size_t total = 0;
-  b->lane_off.assign(b->lanes.size(), 0);
+  std::vector<size_t> off(b->lanes.size(), 0);
   for (size_t k = 0; k < b->lanes.size(); ++k) {
     size_t need = 256;
     for (int i : b->lanes[k]) {
@@ -100,9 +102,10 @@ size_t layout(tpt_batch b) {
       tpt_workspace_bytes(b->plans[i], &w);
       need = std::max(need, align256(w));
     }
-    b->lane_off[k] = total;
+    off[k] = total;
     total += need;
   }
+  if (off != b->lane_off) b->lane_off = off;
   return total;
 }
 
@@ -263,8 +266,11 @@ int tpt_batch_get_grouped(tpt_batch b, int* grouped) {
 
 int tpt_batch_workspace_bytes(tpt_batch b, size_t* bytes) {
   if (!b || !bytes) return TPT_ERR_INVALID_ARG;
-  b->ws_streams = layout(b);
-  if (!b->grouped) b->ws_bytes = b->ws_streams;
+  const size_t streams = layout(b);
+  if (streams != b->ws_streams) {
+    b->ws_streams = streams;
+    if (!b->grouped) b->ws_bytes = streams;
+  }
   *bytes = b->ws_bytes;
   return TPT_OK;
 }
